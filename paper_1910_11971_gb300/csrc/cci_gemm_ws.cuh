@@ -57,11 +57,10 @@
 // 9 + kIssuers .. + 3 as the second producer group), warp 8 allocates TMEM and
 // issues the MMAs, warps 9 .. 8 + kIssuers issue the TMA copies as soon as a
 // stage is free (so copy latency overlaps the producers' work), stage by stage in
-// turn: the copies one thread issues are processed one box after another
-// (measured on GB300: about 0.5 us per box of 16-64 KB from one issuer; copy
-// throughput grows with the number of issuing warps), so up to six warps issue
-// (one per stage in flight; PK: three, one activation box per stage).  Every
-// mbarrier wait is bounded (CCI_ERR_TIMEOUT, abort flag, drain, TMEM freed).
+// turn: what a box costs its issuer is the length of the issue loop, whatever the
+// box's size, so up to six warps issue (one per stage in flight; PK: three, one
+// activation box per stage).  Every mbarrier wait is bounded (CCI_ERR_TIMEOUT,
+// abort flag, drain, TMEM freed).
 #pragma once
 
 #include <cuda.h>
@@ -80,6 +79,23 @@ enum ASrc { kA2d = 0, kA4d = 1, kAGather = 2, kAHalo = 3 };
 // by 4-D TMA: rows m = (bi*PB + pi)*QB + qi of the tile are the pixels
 // (b0 + bi, p0 + pi, q0 + qi); rows >= QB*PB*BB are unused.  Halo copies: QB = Q,
 // BB = 1, rows m = pi*(Q + 2) + qi (qi >= Q unused), rows = PB*(Q + 2)
+// division of a tile index (below 2^31) by a size that is fixed for the launch, as
+// a multiply and a shift (Granlund and Montgomery): the quotient of n is
+// (umulhi(n, mul) + n) >> shift with shift = ceil(log2 d) and
+// mul = floor(2^32 (2^shift - d) / d) + 1.  The copy issuers and the epilogue form
+// tile coordinates once per tile: a run-time 64-bit division there is a serial
+// chain of a hundred instructions in the one thread that keeps the copies going.
+struct TileDiv {
+    uint32_t d = 1, mul = 1, shift = 0;
+    TileDiv() = default;
+    explicit TileDiv(int64_t div) : d(static_cast<uint32_t>(div))
+    {
+        while ((uint64_t(1) << shift) < d) ++shift;
+        mul = static_cast<uint32_t>((((uint64_t(1) << shift) - d) << 32) / d + 1);
+    }
+    __device__ __forceinline__ uint32_t quot(uint32_t n) const { return (__umulhi(n, mul) + n) >> shift; }
+};
+
 struct ConvBox {
     int QB, PB, BB;  // box extent along q, p and the batch
     int nQ, nP;      // boxes along q and p (the batch index is the rest)
@@ -90,6 +106,7 @@ struct ConvBox {
     int resident;    // halo copies: the layer's whole weight matrix stays in the stages
                      // (one N tile, every stage of a tile a stage of the ring): the
                      // weights are copied for the CTA's first tile only
+    TileDiv byQ, byP, byN;  // division by nQ, by nP and by the N tiles (set at the launch)
 };
 
 // activation tensor maps: [0] for products (2-D over X[N][Cin]); for a
@@ -167,9 +184,9 @@ struct Cfg {
     static_assert(kStages >= 3, "too few pipeline stages");
     static_assert(kTmemCols == 128 || kTmemCols == 256 || kTmemCols == 512, "TMEM allocation not a power of 2");
     static_assert(!kARaw || kAColBase + kStages * 64 <= 512, "A stages do not fit in tensor memory");
-    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: one
-    // thread's copies are processed one box at a time, so several issuers keep
-    // more boxes moving.  kIssuers <= kStages keeps every empty-barrier wait
+    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: a box
+    // costs its issuer the same loop whatever its size, so several issuers keep
+    // more bytes moving.  kIssuers <= kStages keeps every empty-barrier wait
     // within one phase of the barrier (no parity aliasing).
     // (kAHalo: one more warp, which copies the halos)
     // PK: three issuers (one activation box per stage) and a second group of four
@@ -731,17 +748,23 @@ __device__ __forceinline__ void expand_item(uint32_t (&out)[8][4], const Runs<K>
 
 // (box along q, box along p, batch box) of M tile mt
 struct BoxIdx {
-    int qb, pb;
-    int64_t bb;
+    int qb, pb, bb;
 };
-__device__ __forceinline__ BoxIdx box_of(int64_t mt, const ConvBox &box)
+__device__ __forceinline__ BoxIdx box_of(int mt, const ConvBox &box)
 {
-    BoxIdx i;
-    i.qb = static_cast<int>(mt % box.nQ);
-    const int64_t t = mt / box.nQ;
-    i.pb = static_cast<int>(t % box.nP);
-    i.bb = t / box.nP;
-    return i;
+    const uint32_t t = box.byQ.quot(static_cast<uint32_t>(mt)), b = box.byP.quot(t);
+    return BoxIdx{static_cast<int>(mt - t * box.byQ.d), static_cast<int>(t - b * box.byP.d), static_cast<int>(b)};
+}
+
+// output pixel -> input pixel of tap offset a = k - pad under a stride of 1 or 2:
+// input index p_out * stride + a lies on parity lattice r at place p_out + d
+struct TapSite {
+    int r, d;
+};
+__device__ __forceinline__ TapSite tap_site(int a, int stride)
+{
+    const int r = a & (stride - 1);
+    return TapSite{r, (a - r) >> (stride - 1)};
 }
 
 // PK: tmB0 / tmB1 are the maps of the packed values and indices (2-D over
@@ -750,7 +773,7 @@ template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC
 __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads, 1)
     gemm_ws_kernel(FwdParams p, const __grid_constant__ AMaps tmA, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmY, ConvBox box,
-                   int64_t n_ct, int64_t n_tiles)
+                   int n_tiles)
 {
     using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
     constexpr int kM = C::kM, kN = C::kN, kKS = C::kKS, kStages = C::kStages;
@@ -771,13 +794,13 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     const uint32_t crank = C::kPairUnits ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
     // work units: tiles (CG = 1) or pair tiles of 2 x 128 rows (CG = 2), strided over
     // the CTAs (CG = 1) or the CTA pairs (CG = 2)
-    const int64_t u0 = C::kPairUnits ? blockIdx.x / 2 : blockIdx.x;
-    const int64_t ustep = C::kPairUnits ? gridDim.x / 2 : gridDim.x;
-    // unit u -> (M tile, N tile): one 64-bit division, the remainder by multiply-subtract
-    auto split_unit = [&](int64_t u, int64_t &mt, int64_t &ct) {
-        const int64_t q = u / n_ct;
-        ct = u - q * n_ct;
-        mt = C::kPairUnits ? 2 * q + crank : q;
+    const int u0 = C::kPairUnits ? blockIdx.x / 2 : blockIdx.x;
+    const int ustep = C::kPairUnits ? gridDim.x / 2 : gridDim.x;
+    // unit u -> (M tile, N tile)
+    auto split_unit = [&](int u, int &mt, int &ct) {
+        const int q = static_cast<int>(box.byN.quot(static_cast<uint32_t>(u)));
+        ct = u - q * static_cast<int>(box.byN.d);
+        mt = C::kPairUnits ? 2 * q + static_cast<int>(crank) : q;
     };
 
     if (tid == 0) {
@@ -853,140 +876,156 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         const uint32_t erow = static_cast<uint32_t>(EPI == 2 ? p.kin : kKS) * (TF32 ? 4u : 2u);  // bytes per row
         const uint32_t a_bytes = (ASRC == kA4d ? static_cast<uint32_t>(box.rows) : static_cast<uint32_t>(kM)) * erow;
         const uint32_t b_bytes = static_cast<uint32_t>(C::kBPlanes * C::kBRows) * erow;
-        const int cpt = static_cast<int>(p.Cin / kKS);  // stages per tap (kA4d)
         const uint32_t halo_bytes =
             static_cast<uint32_t>((box.QB + p.KW - 1) * (box.PB + p.KH - 1)) * 128u;  // kAHalo
-        // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows;
-        // the other issuer warps copy the weight stages in turn
-        const int issuer = warp - (C::kHalo ? 10 : 9);
-        constexpr int kBIssuers = C::kHalo ? C::kIssuers - 1 : C::kIssuers;
-        int it = 0;
-        bool ok = true;
+        // One lane of each warp runs its loop, with every coordinate advanced by adds
+        // and compares.  What a box costs is the length of this loop, not its bytes:
+        // with the coordinates formed by run-time divisions a stage took one issuer
+        // over 2000 cycles and six of them about 550; without, a probe of this loop
+        // issues a box every 246 cycles from one warp and every 135 from two (2 to
+        // 32 KB alike, 25-29 TB/s over the GPU from L2).
         if (C::kHalo && warp == 9) {
-            int hc = 0;
-            const int chunks = nks / taps;
-            for (int64_t u = u0; u < n_tiles && ok; u += ustep) {
-                int64_t mt, ct;
-                split_unit(u, mt, ct);
-                const BoxIdx bi = box_of(mt, box);
-                for (int c = 0; c < chunks && ok; ++c, ++hc) {
-                    // buffer hb is free once the MMAs of chunk hc - nh completed; this
-                    // warp waited for chunk hc - 1 - nh before, so the phase cannot alias
-                    const int hb = hc % box.nh;
-                    if (hc >= box.nh) ok = tc::mbar_wait(&S->hempty[hb], ((hc / box.nh) - 1) & 1, abort, p.status);
-                    if (!ok) break;
-                    if (lane == 0) {
+            // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows
+            if (lane == 0) {
+                int hb = 0;
+                uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
+                const int chunks = nks / taps;
+                bool ok = true;
+                for (int u = u0; u < n_tiles && ok; u += ustep) {
+                    int mt, ct;
+                    split_unit(u, mt, ct);
+                    const BoxIdx bi = box_of(mt, box);
+                    const int y = bi.pb * box.PB - p.ph;
+                    for (int c = 0; c < chunks; ++c) {
+                        // buffer hb is free once the MMAs of the chunk nh before completed
+                        ok = tc::mbar_wait(&S->hempty[hb], ph, abort, p.status);
+                        if (!ok) break;
                         if constexpr (CG == 2) {
                             // each CTA's halo (its own M tile) completes on the even CTA's
                             // barrier, which expects both
                             if (crank == 0) tc::mbar_arrive_expect_tx(&S->hfull[hb], 2 * halo_bytes);
-                            tma_load_4d_pair(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, bi.pb * box.PB - p.ph,
-                                             static_cast<int>(bi.bb), map_to_rank(tc::smem_u32(&S->hfull[hb]), 0));
+                            tma_load_4d_pair(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, y, bi.bb,
+                                             map_to_rank(tc::smem_u32(&S->hfull[hb]), 0));
                         } else {
                             tc::mbar_arrive_expect_tx(&S->hfull[hb], halo_bytes);
-                            tc::tma_load_4d(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, bi.pb * box.PB - p.ph,
-                                            static_cast<int>(bi.bb), &S->hfull[hb]);
+                            tc::tma_load_4d(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, y, bi.bb, &S->hfull[hb]);
+                        }
+                        if (++hb == box.nh) {
+                            hb = 0;
+                            ph ^= 1u;
                         }
                     }
-                    __syncwarp();
                 }
             }
-        } else if (!(PK && C::kHalo))  // PK halo stages hold only the producers' weight tiles
-        for (int64_t u = u0; u < n_tiles && ok; u += ustep) {
-            int64_t mt, ct;
-            split_unit(u, mt, ct);
-            const int64_t co0 = ct * kN + (CG == 2 ? crank * C::kBRows : 0);  // this CTA's B rows
-            BoxIdx bi{0, 0, 0};
-            if constexpr (ASRC == kA4d || ASRC == kAHalo) bi = box_of(mt, box);
-            // resident weights (halo copies): only the first tile's stages are copied
-            if (C::kHalo && box.resident && it >= nks) break;
-            for (int ks = 0; ks < nks && ok; ++ks, ++it) {
-                if (it % kBIssuers != issuer) continue;
-                const int s = it % kStages;
-                if (it >= kStages) ok = tc::mbar_wait(&S->empty[s], ((it / kStages) - 1) & 1, abort, p.status);
-                if (!ok) break;
-                if constexpr (ASRC == kAHalo) {
-                    const int c = ks / taps, t = ks - c * taps;  // stages: chunk by chunk, taps in turn
-                    if (lane == 0) {
-                        const int x = static_cast<int>(t * p.Cin) + c * 64;
-                        if constexpr (CG == 2) {  // this CTA's half of the rows, on the even CTA's barrier
-                            if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * C::kBBytes);
-                            tma_load_2d_pair(base + s * C::kStage, &tmB0, x, static_cast<int>(co0),
-                                             map_to_rank(tc::smem_u32(&S->full[s]), 0));
-                        } else {
-                            tc::mbar_arrive_expect_tx(&S->full[s], C::kBBytes);
-                            tc::tma_load_2d(base + s * C::kStage, &tmB0, x, static_cast<int>(ct * kN), &S->full[s]);
+        } else if (lane == 0 && !(PK && C::kHalo)) {  // PK halo stages hold only the producers' weight tiles
+            // the stages of this warp: every kBIssuers-th, from its own number on
+            constexpr int kBIssuers = C::kHalo ? C::kIssuers - 1 : C::kIssuers;
+            int s = warp - (C::kHalo ? 10 : 9), ks = s;
+            uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
+            // a stage's place in its tile: (tap, chunk of kKS channels), chunks innermost
+            // (kA4d) or taps innermost (kAHalo); one chunk after the other for products
+            int kh = 0, kw = 0, c = 0;
+            const int cpt = ASRC == kA4d ? static_cast<int>(p.Cin / kKS) : 1;  // chunks per tap
+            auto step = [&](int by) {
+                if constexpr (ASRC == kA4d) {
+                    c += by;
+                    while (c >= cpt) {
+                        c -= cpt;
+                        if (++kw == p.KW) {
+                            kw = 0;
+                            if (++kh == p.KH) kh = 0;
                         }
                     }
-                    __syncwarp();
-                    continue;
+                } else if constexpr (ASRC == kAHalo) {
+                    kw += by;  // the tap's number
+                    while (kw >= taps) {
+                        kw -= taps;
+                        if (++c == nks / taps) c = 0;
+                    }
                 }
-                if (lane == 0 && CG == 2) {
-                    // both CTAs' copies complete on the even CTA's full barrier, which
-                    // expects the bytes of the pair (PK: the activations only; each
-                    // CTA's packed runs land on its own aux barrier)
-                    const uint32_t st = base + s * C::kStage;
-                    const uint32_t bst = st + C::kAPlane;
-                    const uint32_t fb = map_to_rank(tc::smem_u32(&S->full[s]), 0);
-                    if constexpr (PK) {
-                        if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * a_bytes);
-                    } else {
-                        if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * (C::kBBytes + a_bytes));
-                        tma_load_2d_pair(bst, &tmB0, ks * kKS, static_cast<int>(co0), fb);
-                    }
-                    if constexpr (ASRC == kA2d) {
-                        tma_load_2d_pair(st, &tmA.m[0], ks * kKS, static_cast<int>(mt * kM), fb);
-                    } else {
-                        const int tap = ks / cpt;
-                        const int ci0 = (ks - tap * cpt) * kKS;
-                        const int kh = tap / p.KW, kw = tap - (tap / p.KW) * p.KW;
-                        const int ah = kh - p.ph, aw = kw - p.pw;
-                        const int rh = ((ah % p.sh) + p.sh) % p.sh, rw = ((aw % p.sw) + p.sw) % p.sw;
-                        const int dh = (ah - rh) / p.sh, dw = (aw - rw) / p.sw;
-                        tma_load_4d_pair(st, &tmA.m[rh * p.sw + rw], ci0, bi.qb * box.QB + dw,
-                                         bi.pb * box.PB + dh, static_cast<int>(bi.bb * box.BB), fb);
-                    }
-                } else if (lane == 0) {
-                    const uint32_t st = base + s * C::kStage;
-                    const uint32_t bst = st + C::kBOff;
+            };
+            step(ks);
+            // resident weights (halo copies): only the first tile's stages are copied
+            const int u_end = C::kHalo && box.resident ? (u0 + 1 < n_tiles ? u0 + 1 : n_tiles) : n_tiles;
+            int u = u0, mt = 0, ct = 0;
+            BoxIdx bi{0, 0, 0};
+            bool fresh = true;  // the tile's coordinates are to be formed
+            while (true) {
+                while (ks >= nks && u < u_end) {
+                    ks -= nks;
+                    u += ustep;
+                    fresh = true;
+                }
+                if (u >= u_end) break;
+                if (fresh) {
+                    split_unit(u, mt, ct);
+                    if constexpr (ASRC == kA4d) bi = box_of(mt, box);
+                    fresh = false;
+                }
+                if (!tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
+                const uint32_t st = base + s * C::kStage;
+                const uint32_t bst = st + C::kBOff;
+                const int co0 = ct * kN + (CG == 2 ? static_cast<int>(crank) * C::kBRows : 0);  // this CTA's B rows
+                // the barrier that the copies complete on: the even CTA's of a pair, which
+                // expects the bytes of both (PK: the activations only)
+                const uint32_t fb = CG == 2 ? map_to_rank(tc::smem_u32(&S->full[s]), 0) : tc::smem_u32(&S->full[s]);
+                if constexpr (ASRC == kAHalo) {
+                    if (CG == 1 || crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], CG * C::kBBytes);
+                    const int x = kw * static_cast<int>(p.Cin) + c * 64;
+                    if constexpr (CG == 2)  // this CTA's half of the rows
+                        tma_load_2d_pair(bst, &tmB0, x, co0, fb);
+                    else
+                        tc::tma_load_2d(bst, &tmB0, x, co0, &S->full[s]);
+                } else {
                     // the activation copy completes on aux (raw fp32, split afterwards) or full
-                    uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
-                    if constexpr (C::kARaw) tc::mbar_arrive_expect_tx(abar, a_bytes);
-                    if constexpr (PK) {
-                        tc::mbar_arrive_expect_tx(&S->full[s], a_bytes);
-                    } else {
-                        tc::mbar_arrive_expect_tx(&S->full[s], b_bytes + (C::kATma ? a_bytes : 0u));
-                        if constexpr (MC) {
+                    if constexpr (C::kARaw) tc::mbar_arrive_expect_tx(&S->aux[s], a_bytes);
+                    if (CG == 1 || crank == 0)
+                        tc::mbar_arrive_expect_tx(&S->full[s],
+                                                  CG * ((PK ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
+                    if constexpr (!PK) {
+                        if constexpr (CG == 2) {
+                            tma_load_2d_pair(bst, &tmB0, ks * kKS, co0, fb);
+                        } else if constexpr (MC) {
                             // this CTA's half of the B rows into both CTAs (the same offsets);
                             // each CTA's full barrier expects the whole tile
                             const uint32_t half = crank * (C::kBPlane / 2);
-                            const int y = static_cast<int>(co0) + static_cast<int>(crank) * (kN / 2);
-                            tma_load_2d_mc(bst + half, &tmB0, ks * kKS, y, tc::smem_u32(&S->full[s]));
+                            const int y = co0 + static_cast<int>(crank) * (kN / 2);
+                            tma_load_2d_mc(bst + half, &tmB0, ks * kKS, y, fb);
                             if constexpr (C::kBPlanes > 1)
-                                tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, tc::smem_u32(&S->full[s]));
+                                tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, fb);
                         } else {
-                            tc::tma_load_2d(bst, &tmB0, ks * kKS, static_cast<int>(co0), &S->full[s]);
+                            tc::tma_load_2d(bst, &tmB0, ks * kKS, co0, &S->full[s]);
                             if constexpr (C::kBPlanes > 1)  // fp32 plane 1: 64 bf16 per stage
-                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, static_cast<int>(co0), &S->full[s]);
+                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, co0, &S->full[s]);
                         }
                     }
+                    uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
                     if constexpr (ASRC == kA2d) {
-                        tc::tma_load_2d(st, &tmA.m[0], ks * kKS, static_cast<int>(mt * kM), abar);
+                        if constexpr (CG == 2)
+                            tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
+                        else
+                            tc::tma_load_2d(st, &tmA.m[0], ks * kKS, mt * kM, abar);
                     } else if constexpr (ASRC == kA4d) {
-                        const int tap = ks / cpt;
-                        const int ci0 = (ks - tap * cpt) * kKS;
-                        const int kh = tap / p.KW, kw = tap - (tap / p.KW) * p.KW;
-                        // input row h = p_out * sh + ah lies on lattice rh at h' = p_out + dh
-                        const int ah = kh - p.ph, aw = kw - p.pw;
-                        const int rh = ((ah % p.sh) + p.sh) % p.sh, rw = ((aw % p.sw) + p.sw) % p.sw;
-                        const int dh = (ah - rh) / p.sh, dw = (aw - rw) / p.sw;
-                        tc::tma_load_4d(st, &tmA.m[rh * p.sw + rw], ci0, bi.qb * box.QB + dw, bi.pb * box.PB + dh,
-                                        static_cast<int>(bi.bb * box.BB), abar);
+                        // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
+                        const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
+                        const CUtensorMap *m = &tmA.m[th.r * p.sw + tw.r];
+                        const int x1 = bi.qb * box.QB + tw.d, x2 = bi.pb * box.PB + th.d, x3 = bi.bb * box.BB;
+                        if constexpr (CG == 2)
+                            tma_load_4d_pair(st, m, c * kKS, x1, x2, x3, fb);
+                        else
+                            tc::tma_load_4d(st, m, c * kKS, x1, x2, x3, abar);
                     }
                 }
-                __syncwarp();
+                ks += kBIssuers;
+                step(kBIssuers);
+                s += kBIssuers;  // kBIssuers <= kStages
+                if (s >= kStages) {
+                    s -= kStages;
+                    ph ^= 1u;
+                }
             }
         }
+        __syncwarp();
     } else if (PK && ((warp >= 4 && warp < 8) || warp >= 9 + C::kIssuers)) {
         // ------------------------------------------------------------ weight producers (PK)
         // two groups of four warps (4-7 and the four after the issuers) take the
@@ -1013,15 +1052,16 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // pair, of each N tile).  Advanced stage by stage without division (one
         // per tile).
         struct Cursor {
-            int64_t u, co, g, r;
+            int u;
+            int64_t co, g, r;
             int ks, t, ch, j0;
             bool chk;
         };
         auto tile_start = [&](Cursor &cu) {
             if (cu.u >= n_tiles) return;
-            int64_t mt, ct;
+            int mt, ct;
             split_unit(cu.u, mt, ct);
-            cu.co = ct * kN + crank * C::kBRows + m0;
+            cu.co = static_cast<int64_t>(ct) * kN + crank * C::kBRows + m0;
             cu.g = cu.co >> lg;
             cu.j0 = static_cast<int>(cu.co & (p.G - 1));
             cu.chk = mt < CG;
@@ -1126,7 +1166,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
 #pragma unroll
                 for (int i = 0; i < 8; ++i) dst[i] = make_uint4(0, 0, 0, 0);
                 if (tile >= n_tiles || ks >= nks) return;
-                const int64_t n0 = (tile / n_ct) * kM;
+                int mt, ct;
+                split_unit(static_cast<int>(tile), mt, ct);
+                const int64_t n0 = static_cast<int64_t>(mt) * kM;
                 if (tile != xsite_tile) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
@@ -1176,8 +1218,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         }
         if constexpr (!C::kATma) {
             // the same work units, in the same order, as the TMA issuers and the MMAs
-            for (int64_t tile = u0; tile < n_tiles && ok; tile += ustep) {
-                const int64_t n0 = (tile / n_ct) * kM;
+            for (int tile = u0; tile < n_tiles && ok; tile += ustep) {
+                int mt, ct;
+                split_unit(tile, mt, ct);
+                const int64_t n0 = static_cast<int64_t>(mt) * kM;
                 ColumnSite site[8];
                 bool colok[8];
                 if constexpr (!TF32) {
@@ -1308,7 +1352,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             // reconvergence between the stages' MMAs (the gaps between stages, not
             // the MMAs, bounded this product)
             if (lane == 0) {
-                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     if (t >= 2) ok = tc::mbar_wait(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
                     if (!ok) break;
@@ -1338,7 +1382,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 uint32_t ph = 0u;  // parity of the full-barrier phase to wait for
                 const uint64_t sunits = C::kStage >> 4, bunits = C::kBOff >> 4;
                 const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;  // MMAs per stage (EPI = 2)
-                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
                     if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1383,7 +1427,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 const uint64_t wq_units = static_cast<uint64_t>(box.QB + p.KW - 1) * 8u;
                 const uint64_t hunits = hbytes >> 4, sunits = C::kStage >> 4;
                 const bool res = box.resident != 0;
-                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
                     if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1438,7 +1482,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             }
             ok = false;  // the generic loop below is not entered
         }
-        for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
+        for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
             const int acc = t & 1;
             // CG = 2: the phase includes arrivals of the odd CTA's epilogue
             if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1502,11 +1546,21 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         int chunk_no = 0;
         // CG = 2: the odd CTA releases an accumulator on the even CTA's barrier
         const uint32_t tmem_empty_remote = CG == 2 ? map_to_rank(tc::smem_u32(&S->tmem_empty[0]), 0) : 0u;
-        for (int64_t u = u0 + eg * ustep; u < n_tiles && ok; u += kEG * ustep, t += kEG) {
+        // halo tiles: row m = pi * (Q + 2) + qi goes to staged row pi * Q + qi (the box
+        // of the store), the two unused columns of each row nowhere
+        int srow = m;
+        bool stage_row = true;
+        if constexpr (ASRC == kAHalo) {
+            const int wq = box.QB + p.KW - 1;
+            const int pi = m / wq, qi = m - pi * wq;
+            srow = pi * box.QB + qi;
+            stage_row = pi < box.PB && qi < box.QB;
+        }
+        for (int u = u0 + eg * ustep; u < n_tiles && ok; u += kEG * ustep, t += kEG) {
             const int acc = t & 1;
-            int64_t mt, ct;
+            int mt, ct;
             split_unit(u, mt, ct);
-            const int co0 = static_cast<int>(ct * kN);
+            const int co0 = ct * kN;
             BoxIdx bi{0, 0, 0};
             if constexpr (ASRC == kA4d || ASRC == kAHalo) bi = box_of(mt, box);
             ok = tc::mbar_wait(&S->tmem_full[acc], (t / 2) & 1, abort, p.status);
@@ -1554,16 +1608,6 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 const uint32_t buf = ybuf + static_cast<uint32_t>(kYG * eg + (chunk_no % kYG)) * C::kYBuf;
                 if (etid == 0) tc::bulk_wait_read<kYG - 1>();
                 tc::named_sync(ebar, 128);
-                // halo tiles: row m = pi * (Q + 2) + qi goes to staged row pi * Q + qi
-                // (the box of the store), the two unused columns of each row nowhere
-                int srow = m;
-                bool stage_row = true;
-                if constexpr (ASRC == kAHalo) {
-                    const int wq = box.QB + p.KW - 1;
-                    const int pi = m / wq, qi = m - (m / wq) * wq;
-                    srow = pi * box.QB + qi;
-                    stage_row = pi < box.PB && qi < box.QB;
-                }
                 if (stage_row) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
@@ -1574,10 +1618,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 tc::named_sync(ebar, 128);
                 if (etid == 0) {
                     if constexpr (ASRC == kA4d || ASRC == kAHalo)
-                        tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB,
-                                         static_cast<int>(bi.bb * box.BB));
+                        tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB, bi.bb * box.BB);
                     else
-                        tc::tma_store_2d(&tmY, buf, co0 + c0, static_cast<int>(mt * kM));
+                        tc::tma_store_2d(&tmY, buf, co0 + c0, mt * kM);
                     tc::bulk_commit();
                 }
             }
@@ -1819,6 +1862,10 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     // CG = 2 or MC: units are pair tiles (two M tiles), one per cluster of two CTAs
     constexpr int kCl = C::kPairUnits ? 2 : 1;
     const int64_t n_tiles = n_ct * (kCl == 2 ? (m_tiles + 1) / 2 : m_tiles);
+    if (n_tiles >= (int64_t(1) << 30)) return cudaErrorInvalidValue;  // unit numbers are 32-bit, with the grid added
+    box.byQ = TileDiv(box.nQ);
+    box.byP = TileDiv(box.nP);
+    box.byN = TileDiv(n_ct);
     const int64_t slots = sm_count() / kCl;
     const int64_t grid = kCl * (n_tiles < slots ? n_tiles : slots);
     // programmatic dependent launch: may start once every block of the preceding
@@ -1838,7 +1885,8 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     la[1].val.clusterDim.z = 1;
     cfg.attrs = la;
     cfg.numAttrs = kCl == 2 ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box, n_ct, n_tiles);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box,
+                                             static_cast<int>(n_tiles));
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
