@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // 32 KB alike, 25-29 TB/s over the GPU from L2).
         if (C::kHalo && warp == 9) {
             // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows
-            if (lane == 0) {
+            if (tc::elect_one()) {
                 int hb = 0;
                 uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
                 const int chunks = nks / taps;
@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     }
                 }
             }
-        } else if (lane == 0 && !(PK && C::kHalo)) {  // PK halo stages hold only the producers' weight tiles
+        } else if (!(PK && C::kHalo) && tc::elect_one()) {  // PK halo stages hold only the producers' weight tiles
             // the stages of this warp: every kBIssuers-th, from its own number on
             constexpr int kBIssuers = C::kHalo ? C::kIssuers - 1 : C::kIssuers;
             int s = warp - (C::kHalo ? 10 : 9), ks = s;
@@ -1340,7 +1340,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         const int hchunks = ASRC == kAHalo ? nks / taps : 0;
         const uint64_t hdesc0 = tc::sw128_desc(hbuf), bdesc0 = tc::sw128_desc(base);
         const uint32_t empty0 = tc::smem_u32(&S->empty[0]);
-        const uint32_t issue = lane == 0 ? 1u : 0u;  // the lane that issues (a predicate in the stage block)
+        const uint32_t issue = tc::elect_one() ? 1u : 0u;  // the lane that issues (a predicate in the stage block)
         auto commit = [&](uint64_t *bar) {
             if constexpr (CG == 2)
                 mma_commit_pair(bar);
@@ -1351,7 +1351,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             // one thread runs the whole issue loop: no per-stage divergence or warp
             // reconvergence between the stages' MMAs (the gaps between stages, not
             // the MMAs, bounded this product)
-            if (lane == 0) {
+            if (tc::elect_one()) {
                 for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     if (t >= 2) ok = tc::mbar_wait(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1377,7 +1377,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             // bf16 stages of one A and one B plane: one thread runs the issue loop,
             // each stage's MMAs and its commit issued from one block (pairs: from the
             // even CTA, which alone enters with ok set)
-            if (lane == 0 && ok) {
+            if (ok && tc::elect_one()) {
                 int s = 0;
                 uint32_t ph = 0u;  // parity of the full-barrier phase to wait for
                 const uint64_t sunits = C::kStage >> 4, bunits = C::kBOff >> 4;
@@ -1421,7 +1421,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             // released; otherwise each tap is a stage of the ring.  Descriptors in
             // 16-byte units: + wq_units per halo row of taps, + 8 per column,
             // + hunits per halo buffer, + sunits per stage.
-            if (lane == 0 && ok) {
+            if (ok && tc::elect_one()) {
                 int hs = 0, hb = 0;
                 uint32_t hsph = 0u, hph = 0u;
                 const uint64_t wq_units = static_cast<uint64_t>(box.QB + p.KW - 1) * 8u;
@@ -1495,7 +1495,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 ok = tc::mbar_wait<PK && CG == 2>(&S->full[s], (it / kStages) & 1, abort, p.status);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (lane == 0) {
+                if (tc::elect_one()) {
                     const uint32_t st = base + s * C::kStage;
                     const uint32_t bst = st + C::kBOff;
                     if constexpr (TF32) {
@@ -1524,10 +1524,11 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                                          ks > 0 ? 1u : 0u, issue, empty0 + 8u * s);
                 __syncwarp();
             }
-            if (ok && lane == 0) commit(&S->tmem_full[acc]);
+            if (ok && tc::elect_one()) commit(&S->tmem_full[acc]);
             __syncwarp();
         }
-        if (lane == 0 && (CG == 1 || crank == 0)) commit(&S->drain);
+        // (the same thread as issued the MMAs: a commit covers its own thread's)
+        if ((CG == 1 || crank == 0) && tc::elect_one()) commit(&S->drain);
         __syncwarp();
         int no_abort = 0;
         tc::mbar_wait(&S->drain, 0, &no_abort, p.status);
@@ -1537,7 +1538,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // whose accumulator is g)
         constexpr int kEG = C::kEG;
         const int eg = warp >> 2;              // this thread's group
-        const int etid = tid - 128 * eg;       // thread within the group; 0 issues its stores
+        const int etid = tid - 128 * eg;       // thread within the group
+        const bool storer = (warp & 3) == 0 && tc::elect_one();  // the thread that issues the group's stores
         const int ebar = 1 + eg;               // the group's named barrier
         int t = eg;
         bool ok = true;
@@ -1606,7 +1608,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 // the store issued from it kYPerGroup chunks earlier has read it
                 constexpr int kYG = C::kYPerGroup;
                 const uint32_t buf = ybuf + static_cast<uint32_t>(kYG * eg + (chunk_no % kYG)) * C::kYBuf;
-                if (etid == 0) tc::bulk_wait_read<kYG - 1>();
+                if (storer) tc::bulk_wait_read<kYG - 1>();
                 tc::named_sync(ebar, 128);
                 if (stage_row) {
 #pragma unroll
@@ -1616,7 +1618,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc::named_sync(ebar, 128);
-                if (etid == 0) {
+                if (storer) {
                     if constexpr (ASRC == kA4d || ASRC == kAHalo)
                         tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB, bi.bb * box.BB);
                     else
@@ -1625,7 +1627,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 }
             }
         }
-        if (etid == 0) tc::bulk_wait_all();
+        if (storer) tc::bulk_wait_all();
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
