@@ -15,6 +15,7 @@ X [N][Cin] (product) or NHWC [B][H][W][Cin] (convolution), Y fp32.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional, Sequence, Tuple
 
@@ -109,16 +110,20 @@ def decode_status(word: int) -> int:
     return int(lib().cci_decode_device_status(ctypes.c_uint32(int(word) & 0xffffffff)))
 
 
+_DTYPE_CODES = {torch.float32: F32, torch.bfloat16: BF16}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    raise TypeError(f"unsupported dtype {t.dtype}: float32 or bfloat16")
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported dtype {t.dtype}: float32 or bfloat16")
+    return code
 
 
 def _stream(device: torch.device) -> int:
-    return torch.cuda.current_stream(device).cuda_stream
+    # the handle alone: a Stream object for it costs 2 us a call
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def _cuda_contig(t: torch.Tensor, name: str) -> None:
@@ -179,14 +184,13 @@ def workspace_size(algo: int, dtype: torch.dtype, Cout: int, R: int) -> int:
 
 
 def new_workspace(algo: int, dtype: torch.dtype, Cout: int, R: int, device) -> Optional[torch.Tensor]:
-    n = workspace_size(algo, dtype, Cout, R)
-    return torch.empty(n, dtype=torch.uint8, device=device) if n else None
+    return _workspace(workspace_size(algo, dtype, Cout, R), device)
 
 
 def _ws(workspace: Optional[torch.Tensor]):
     if workspace is None:
         return None, 0
-    return workspace.data_ptr(), workspace.numel() * workspace.element_size()
+    return workspace.data_ptr(), workspace.nbytes
 
 
 def linear(X: torch.Tensor, values: torch.Tensor, idx: torch.Tensor, Cout: int, G: int, K: int, *,
@@ -201,7 +205,7 @@ def linear(X: torch.Tensor, values: torch.Tensor, idx: torch.Tensor, Cout: int, 
     _cuda_contig(X, "X")
     N, Cin = X.shape
     if workspace is None and algo == ALGO_AUTO:
-        workspace = auto_workspace(X.dtype, Cin, Cin, Cout, G, K, X.device)
+        workspace = _workspace(_auto_bytes(X.dtype, Cin, Cin, Cout, G, K, False), X.device)
     elif workspace is None and algo == ALGO_DENSE_TC_WS:
         workspace = new_workspace(algo, X.dtype, Cout, Cin, X.device)
     Y = out if out is not None else torch.empty((N, Cout), dtype=torch.float32, device=X.device)
@@ -277,7 +281,7 @@ def conv2d(X: torch.Tensor, values: torch.Tensor, idx: torch.Tensor, Cout: int, 
     Y = out if out is not None else torch.empty((B, max(P, 0), max(Q, 0), Cout), dtype=torch.float32,
                                                 device=X.device)
     if workspace is None and algo == ALGO_AUTO:
-        workspace = auto_workspace(X.dtype, Cin, KH * KW * Cin, Cout, G, K, X.device, max(stride))
+        workspace = _workspace(_auto_bytes(X.dtype, Cin, KH * KW * Cin, Cout, G, K, max(stride) > 2), X.device)
     elif workspace is None and algo == ALGO_DENSE_TC_WS:
         workspace = new_workspace(algo, X.dtype, Cout, KH * KW * Cin, X.device)
     wp, wb = _ws(workspace)
@@ -373,8 +377,8 @@ def linear_fused(X: torch.Tensor, values: torch.Tensor, idx: torch.Tensor, Cout:
     else the workspace one, whose workspace is allocated here when not given)."""
     _cuda_contig(X, "X")
     N, Cin = X.shape
-    if workspace is None and not kernel_name(X.dtype, Cin, Cin, Cout, G, K).startswith("dense_tc_fused"):
-        workspace = new_workspace(ALGO_DENSE_TC_WS, X.dtype, Cout, Cin, X.device)
+    if workspace is None:
+        workspace = _workspace(_epilogue_bytes(X.dtype, Cin, Cin, Cout, G, K, False), X.device)
     Y = out if out is not None else torch.empty((N, Cout), dtype=out_dtype, device=X.device)
     if bias is not None:
         _cuda_contig(bias, "bias")
@@ -400,9 +404,8 @@ def conv2d_fused(X: torch.Tensor, values: torch.Tensor, idx: torch.Tensor, Cout:
     P, Q = conv_out_hw(H, W, KH, KW, stride, pad)
     Y = out if out is not None else torch.empty((B, max(P, 0), max(Q, 0), Cout), dtype=out_dtype,
                                                 device=X.device)
-    fused = kernel_name(X.dtype, Cin, KH * KW * Cin, Cout, G, K).startswith("dense_tc_fused") and max(stride) <= 2
-    if workspace is None and not fused:
-        workspace = new_workspace(ALGO_DENSE_TC_WS, X.dtype, Cout, KH * KW * Cin, X.device)
+    if workspace is None:
+        workspace = _workspace(_epilogue_bytes(X.dtype, Cin, KH * KW * Cin, Cout, G, K, max(stride) > 2), X.device)
     if bias is not None:
         _cuda_contig(bias, "bias")
     wp, wb = _ws(workspace)
@@ -476,12 +479,33 @@ def auto_workspace(dtype: torch.dtype, Cin: int, R: int, Cout: int, G: int, K: i
     for a product, KH*KW*Cin for a convolution of the given largest stride), from
     PyTorch memory: None when that family needs none (the library allocates
     nothing itself)."""
-    name = kernel_name(dtype, Cin, R, Cout, G, K, ALGO_AUTO)
-    if name.startswith("dense_tc_fused") and stride <= 2:
-        return None
-    if not lib().cci_kernel_name(F32 if dtype == torch.float32 else BF16, Cin, R, Cout, G, K, ALGO_DENSE_TC_WS):
-        return None
-    return new_workspace(ALGO_DENSE_TC_WS, dtype, Cout, R, device)
+    return _workspace(_auto_bytes(dtype, Cin, R, Cout, G, K, stride > 2), device)
+
+
+# What a layer's sizes alone settle, looked up once per layer shape: these
+# questions to the library took 5 of the 17 us that a call spent in Python.
+@functools.lru_cache(maxsize=4096)
+def _auto_bytes(dtype: torch.dtype, Cin: int, R: int, Cout: int, G: int, K: int, wide_stride: bool) -> int:
+    """Workspace bytes with which AUTO reaches its fastest family (0: none needed)."""
+    if _fused_first(dtype, Cin, R, Cout, G, K, wide_stride):
+        return 0
+    if not kernel_name(dtype, Cin, R, Cout, G, K, ALGO_DENSE_TC_WS):
+        return 0
+    return workspace_size(ALGO_DENSE_TC_WS, dtype, Cout, R)
+
+
+@functools.lru_cache(maxsize=4096)
+def _epilogue_bytes(dtype: torch.dtype, Cin: int, R: int, Cout: int, G: int, K: int, wide_stride: bool) -> int:
+    """Workspace bytes of the entry points with an output stage (0: none needed)."""
+    return 0 if _fused_first(dtype, Cin, R, Cout, G, K, wide_stride) else workspace_size(ALGO_DENSE_TC_WS, dtype, Cout, R)
+
+
+def _fused_first(dtype, Cin, R, Cout, G, K, wide_stride) -> bool:
+    return kernel_name(dtype, Cin, R, Cout, G, K, ALGO_AUTO).startswith("dense_tc_fused") and not wide_stride
+
+
+def _workspace(nbytes: int, device) -> Optional[torch.Tensor]:
+    return torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else None
 
 
 def fma_probe(out: torch.Tensor, blocks: int, threads: int, iters: int) -> None:

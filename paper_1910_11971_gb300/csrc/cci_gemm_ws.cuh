@@ -1738,25 +1738,33 @@ inline int sm_count()
     return sms > 0 ? sms : 1;
 }
 
+// the next larger box extent that covers n in fewer boxes than extent e does (the
+// smallest extent for its number of boxes), or n + 1 after the whole extent
+inline int next_extent(int n, int e)
+{
+    const int boxes = (n + e - 1) / e;
+    return boxes == 1 ? n + 1 : (n + boxes - 2) / (boxes - 1);
+}
+
 // the output-pixel box with the fewest M tiles (ties: longer runs along q, then
-// p).  Only the smallest box of each tile count along q and p is tried.
+// p).  Only the smallest box of each tile count along q and p is tried, and those
+// are stepped through directly: a call's host time is the floor of a small layer.
 inline ConvBox choose_box(int64_t B, int64_t P, int64_t Q)
 {
     ConvBox best{1, 1, 1, 1, 1, 1, B};
     int64_t best_tiles = -1;
-    for (int64_t QB = 1; QB <= Q && QB <= 128; ++QB) {
-        const int64_t nq = (Q + QB - 1) / QB;
-        if ((Q + nq - 1) / nq != QB) continue;
-        for (int64_t PB = 1; PB <= P && QB * PB <= 128; ++PB) {
-            const int64_t np = (P + PB - 1) / PB;
-            if ((P + np - 1) / np != PB) continue;
-            const int64_t BB = (128 / (QB * PB)) < B ? 128 / (QB * PB) : B;
+    const int q_all = static_cast<int>(Q), p_all = static_cast<int>(P);  // below 2^30 (a_source)
+    for (int QB = 1; QB <= q_all && QB <= 128; QB = next_extent(q_all, QB)) {
+        const int64_t nq = (q_all + QB - 1) / QB;
+        for (int PB = 1; PB <= p_all && QB * PB <= 128; PB = next_extent(p_all, PB)) {
+            const int64_t np = (p_all + PB - 1) / PB;
+            const int BB = (128 / (QB * PB)) < B ? 128 / (QB * PB) : static_cast<int>(B);
             const int64_t tiles = nq * np * ((B + BB - 1) / BB);
             if (best_tiles < 0 || tiles <= best_tiles) {
                 best_tiles = tiles;
-                best.QB = static_cast<int>(QB);
-                best.PB = static_cast<int>(PB);
-                best.BB = static_cast<int>(BB);
+                best.QB = QB;
+                best.PB = PB;
+                best.BB = BB;
             }
         }
     }
