@@ -1918,18 +1918,15 @@ struct Plan {
     AMaps am;
 };
 // halo box of a bf16 3x3, stride-1, padding-1 convolution: PB output rows of
-// the full width per tile.  Used for layers of 256 input channels or more (four
-// chunks or more per tile: the per-tap copies there move 9 x the halo's bytes,
-// and the halo copies measured 7-11 % faster on the 14 x 14 ResNet-50 layers;
-// with 64 or 128 channels the tile is bound by the MMAs' shared-memory reads
-// and the per-tap form measured faster), and for 64 -> 64 layers, whose nine
-// weight tiles stay resident in the stages (no per-tap weight copies either),
-// whose output rows per tile are at least three quarters of the 4-D box's
-// (images narrower than the tile fit several per 4-D box, not per halo)
-inline bool halo_box(const FwdParams &p, const ConvBox &a4d, ConvBox *hb)
+// the full width per tile.  Used for layers of min_cin input channels or more
+// (the per-tap copies there move 9 x the halo's bytes), and for 64 -> 64 layers,
+// whose nine weight tiles stay resident in the stages (no per-tap weight copies
+// either), whose output rows per tile are at least three quarters of the 4-D
+// box's (images narrower than the tile fit several per 4-D box, not per halo)
+inline bool halo_box(const FwdParams &p, const ConvBox &a4d, int64_t min_cin, ConvBox *hb)
 {
     if (!(p.is_conv && p.KH == 3 && p.KW == 3 && p.sh == 1 && p.sw == 1 && p.ph == 1 && p.pw == 1 &&
-          p.Cin % 64 == 0 && (p.Cin >= 256 || (p.Cin == 64 && p.Cout <= 64)) && p.P == p.H && p.Q == p.W &&
+          p.Cin % 64 == 0 && (p.Cin >= min_cin || (p.Cin == 64 && p.Cout <= 64)) && p.P == p.H && p.Q == p.W &&
           p.Q + 2 <= 66))
         return false;
     const int wq = static_cast<int>(p.Q) + 2;
@@ -1943,13 +1940,17 @@ inline bool halo_box(const FwdParams &p, const ConvBox &a4d, ConvBox *hb)
     return true;
 }
 
-inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl)
+// halo copies from 128 input channels on: over CTA pairs with 128-wide N tiles
+// they measured faster than the per-tap copies (128 -> 128 at 28 x 28, 64 images
+// 18.8 -> 16.6 us a pass, 128 images 29.1 -> 24.3 us).  The fused family, whose
+// producers bound it, takes them from 256 on.
+inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t halo_cin = 128)
 {
     pl->asrc = a_source(p, ks);
     pl->box = ConvBox{1, 1, 1, 1, 1, 1, 1};
     if (pl->asrc == kA4d) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
     ConvBox hb;
-    if (pl->asrc == kA4d && !tf32 && halo_box(p, pl->box, &hb)) {
+    if (pl->asrc == kA4d && !tf32 && halo_box(p, pl->box, halo_cin, &hb)) {
         pl->asrc = kAHalo;
         pl->box = hb;
     }

@@ -24,19 +24,17 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
         if (asrc == kA2d) return launch_cfg<false, kA2d, 256, 2>(p, pl.box, pl.am, stream);
         return launch_cfg<false, kA4d, 256, 2>(p, pl.box, pl.am, stream);
     }
-    const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
     if (asrc == kAHalo) {
         // 3x3 convolutions from halo copies (tiles of nine stages per chunk at least)
         // CTA pairs (256-row tiles, each CTA copying its own halo and half of every
-        // weight tile) for layers of 256+ input channels whose 256-wide N tile wins
-        // the pair tile-round count: every tile re-reads the layer's weights, whose
-        // copies bound those layers (14 x 14 ResNet-50 layers: 0.0396 -> 0.0375 ms)
-        if (p.Cin >= 256 && choose_bn(m_tiles, p.Cout, 256, 2) == 256)
-            return launch_cfg<false, kAHalo, 256, 2>(p, pl.box, pl.am, stream);
-        if (bn == 64) return launch_cfg<false, kAHalo, 64, 1>(p, pl.box, pl.am, stream);
-        if (bn == 128) return launch_cfg<false, kAHalo, 128, 1>(p, pl.box, pl.am, stream);
-        return launch_cfg<false, kAHalo, 256, 1>(p, pl.box, pl.am, stream);
+        // weight tile) for every layer but the 64 -> 64 ones: a pair's stage brings 8 KB
+        // of weights per SM for 256 cycles of MMAs.  With the issue loops lean, 128-wide
+        // tiles beat 256-wide ones (256 channels at 14 x 14, 128 images 27.5 -> 26.7 us)
+        if (p.Cin >= 128 && p.Cout > 64 && m_tiles > 1)
+            return launch_cfg<false, kAHalo, 128, 2>(p, pl.box, pl.am, stream);
+        return launch_cfg<false, kAHalo, 64, 1>(p, pl.box, pl.am, stream);  // 64 channels out, or one M tile
     }
+    const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
     // tiles of at most 4 stages: the output write dominates, two epilogue groups
     // with two staging buffers each; longer ones keep the shared memory for stages
     const bool short_k = nks <= 4 && asrc != kAGather;

@@ -786,6 +786,22 @@ def test_halo_conv3x3_pair_tiles_ragged(dev):
         assert_within_tol(f64(Y[b]).reshape(-1, Cout), Yo, S, f"ragged halo pair conv image {b}")
 
 
+# halo copies over CTA pairs with 128-wide N tiles from 128 input channels on: one
+# row block per image (an odd count, a pair without a second tile), ragged last
+# row blocks and N tiles, a single row block (which runs 64-wide single tiles)
+@pytest.mark.parametrize("B,H,Wi,Cin,Cout", [(3, 28, 28, 128, 128), (5, 9, 9, 128, 72), (2, 13, 17, 192, 264),
+                                             (1, 4, 30, 128, 128)])
+def test_halo_conv3x3_pairs_from_128_channels(dev, B, H, Wi, Cin, Cout):
+    G, K = 8, 2
+    g = torch.Generator().manual_seed(B * 31 + H + Cin + Cout)
+    X = torch.randn((B, H, Wi, Cin), generator=g).clamp_min(0).to(BF16)
+    W = torch.randn((Cout, 9 * Cin), generator=g).to(BF16)
+    Y = run_conv(dev, X, W, (3, 3, (1, 1), (1, 1), Cout), G, K, cci.ALGO_DENSE_TC_WS)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.conv2d(f64(X), Wd, mask, 3, 3, (1, 1), (1, 1))
+    assert_within_tol(f64(Y).reshape(-1, Cout), Yo, S, f"halo pairs B={B} {H}x{Wi} {Cin}->{Cout}")
+
+
 # ---------------------------------------------------------------------------
 # CTA-pair tiles (tcgen05 cta_group::2): bf16 layers with at least 16 stages of
 # 64 reduction indices and 256-wide N tiles run as 256-row tiles split over two
