@@ -137,14 +137,14 @@ __global__ void __launch_bounds__(128) decompress_rows_kernel(FwdParams p, uint1
     if (r >= p.R) return;
     const int64_t co = static_cast<int64_t>(blockIdx.y) * 8;
     const int lg = 31 - __clz(p.G);
-    const int64_t groups = p.Cout / p.G;
+    const int64_t groups = p.Cout >> lg;
     const int64_t g = co >> lg;
     const int j0 = static_cast<int>(co & (p.G - 1));
     ws::pk::Runs<K> run;
     ws::pk::load_item<K>(run, p, g, r, groups);
     uint32_t out[8][4];
     bool bad = false;
-    ws::pk::expand_item<K>(out, run, p.G, g, j0, groups, 8, true, bad);
+    ws::pk::expand_item<K>(out, run, p.G, g, j0, groups, true, bad);
     if (bad) report(p.status, CCI_ERR_INDEX);
 #pragma unroll
     for (int jj = 0; jj < 8; ++jj)

@@ -633,26 +633,29 @@ __device__ __forceinline__ void expand_group(uint32_t (&out)[8][4], const uint32
     }
 }
 
-// true if an index set of the group at one of the item's first nr reduction
-// indices is not strictly increasing or has an index >= G (cci_pack never
-// writes such sets)
+// true if an index set of the group at one of the item's eight reduction indices
+// is not strictly increasing or has an index >= G (cci_pack never writes such
+// sets).  G is a power of two, so an index is below it when no higher bit is set:
+// one AND per word.  Order is tested on pairs of bytes spread to 16-bit halves,
+// two pairs per subtraction: hi + 255 - lo reaches 256 exactly when hi > lo.
 template <int K>
-__device__ __forceinline__ bool bad_sets(const uint32_t *iw, int G, int nr)
+__device__ __forceinline__ bool bad_sets(const uint32_t *iw, int G)
 {
-    bool bad = false;
+    const uint32_t above = (0xffu & ~static_cast<uint32_t>(G - 1)) * 0x01010101u;
+    uint32_t high = 0u, grows = 0x01000100u;  // bits 8 and 24 stay while every pair grows
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        if (r >= nr) break;
-        int prev = -1;
-#pragma unroll
-        for (int s = 0; s < K; ++s) {
-            const int b = r * K + s;
-            const int j = static_cast<int>((iw[b >> 2] >> (8 * (b & 3))) & 0xffu);
-            bad |= j >= G || j <= prev;
-            prev = j;
-        }
+    for (int w = 0; w < 2 * K; ++w) {
+        high |= iw[w];
+        if constexpr (K >= 2)  // slots (0, 1), (2, 3), ... of the word's set(s)
+            grows &= ((iw[w] >> 8) & 0x00ff00ffu) + 0x00ff00ffu - (iw[w] & 0x00ff00ffu);
+        if constexpr (K >= 4)  // slots (1, 2) of words w and w + 1
+            if (w % 2 == 0)
+                grows &= (prmt(iw[w], iw[w + 1], 0x6622u) & 0x00ff00ffu) + 0x00ff00ffu -
+                         (prmt(iw[w], iw[w + 1], 0x5511u) & 0x00ff00ffu);
+        if constexpr (K == 8)  // slots (3, 4): the two words of one set
+            if (w % 2 == 0) grows &= ((iw[w + 1] & 0xffu) + 0xffu - (iw[w] >> 24)) | 0x01000000u;
     }
-    return bad;
+    return (high & above) != 0u || grows != 0x01000100u;
 }
 
 // the K-slot runs of an item's group(s) at its 8 reduction indices, in
@@ -724,22 +727,21 @@ __device__ __forceinline__ void load_item(Runs<K> &run, const FwdParams &p, int6
 }
 
 // the item's 8 rows of 8 bf16 (4 words each) from its runs (group g, first row
-// j0 of the group); chk: check the index sets of its group(s) at the first nr
-// indices (bad set on a bad one)
+// j0 of the group); chk: check the index sets of its group(s) (bad set on a bad one)
 template <int K>
 __device__ __forceinline__ void expand_item(uint32_t (&out)[8][4], const Runs<K> &run, int G, int64_t g, int j0,
-                                            int64_t groups, int nr, bool chk, bool &bad)
+                                            int64_t groups, bool chk, bool &bad)
 {
     if constexpr (Runs<K>::NG == 2) {
         if (G == 4) {
-            if (chk && g < groups) bad |= bad_sets<K>(run.i[0], G, nr);
-            if (chk && g + 1 < groups) bad |= bad_sets<K>(run.i[1], G, nr);
+            if (chk && g < groups) bad |= bad_sets<K>(run.i[0], G);
+            if (chk && g + 1 < groups) bad |= bad_sets<K>(run.i[1], G);
             expand_group<K, 0, 4, true>(out, run.v[0], run.i[0], 0);
             expand_group<K, 4, 8, true>(out, run.v[1], run.i[1], 4);
             return;
         }
     }
-    if (chk && j0 == 0 && g < groups) bad |= bad_sets<K>(run.i[0], G, nr);
+    if (chk && j0 == 0 && g < groups) bad |= bad_sets<K>(run.i[0], G);
     expand_group<K, 0, 8, true>(out, run.v[0], run.i[0], -j0);  // G = 8: j0 = 0
 }
 
@@ -1041,8 +1043,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         const int pt = tid - (q ? 32 * (9 + C::kIssuers) : 128);
         const int m0 = (pt >> 3) * 8, c = pt & 7;
         const bool active = m0 < C::kBRows;
-        const int64_t groups = p.Cout / p.G;
         const int lg = 31 - __clz(p.G);  // G is a power of two
+        const int64_t groups = p.Cout >> lg;
         const uint32_t full_remote = CG == 2 ? map_to_rank(tc::smem_u32(&S->full[0]), 0) : 0u;
         bool bad = false;
         // a stage of this CTA, in the MMAs' order, and the item's place in it: the
@@ -1107,9 +1109,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     if (!ok || cur.u >= n_tiles) break;
                     uint32_t out[8][4];
                     if (active) {
-                        const int64_t left = p.R - cur.r;
-                        const int nr = left <= 0 ? 0 : (left >= 8 ? 8 : static_cast<int>(left));
-                        pk::expand_item<K>(out, ring[b], p.G, cur.g, cur.j0, groups, nr, cur.chk, bad);
+                        // R is a multiple of 8: the eight indices lie wholly inside or out
+                        pk::expand_item<K>(out, ring[b], p.G, cur.g, cur.j0, groups, cur.chk && cur.r < p.R, bad);
                     }
                     load(ring[b]);
                     if (pass > 0) ok = tc::mbar_wait(&S->empty[s], (pass - 1) & 1, abort, p.status);
