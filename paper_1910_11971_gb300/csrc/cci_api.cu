@@ -174,6 +174,8 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
         }
         if (dense_ok && ws_ok && aligned(p.X, 16) && aligned(p.Y, 16)) {
             algo = CCI_ALGO_DENSE_TC_WS;
+        } else if (narrow_ok(p, dtype, p.N)) {
+            return to_status(launch_narrow(p, stream));
         } else if (!auto_prefers_fused(K)) {
             const int r = try_fused(p, dtype, stream);
             if (r != 0) return fused_status(r);
@@ -861,10 +863,12 @@ extern "C" cci_status cci_linear_host(const void *X_host, cci_dtype dtype, int64
         FwdParams p = linear_params(xd, nc, Cin, values, idx, Cout, yd, dev_status);
         p.G = G;
         p.K = K;
+        p.N_call = N;
         if (fused) {
             result = to_status(launch_gemm_pk(p, cs));
-        } else if (c == 0) {
-            // the first chunk decompresses the weights into the workspace
+        } else if (c == 0 || narrow_ok(p, dtype, N)) {
+            // the first chunk decompresses the weights into the workspace (few columns
+            // in all: every chunk expands them as it multiplies)
             result = forward(p, dtype, G, K, CCI_ALGO_DENSE_TC_WS, ws, l.ws, cs);
         } else {
             p.wdense = ws;

@@ -35,6 +35,13 @@ cudaError_t launch_gemm_ws(const FwdParams &p, int dtype, cudaStream_t stream);
 cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream);
 cudaError_t launch_gemm_ws_tf32(const FwdParams &p, cudaStream_t stream);
 
+// products of at most 128 columns in one launch (cci_narrow.cu; bf16, no
+// workspace): the packed weights (p.values, p.idx, p.G, p.K) expanded and
+// multiplied once, the reduction split over a cluster.  N: the columns of the
+// whole call (a host-buffer product runs chunks of it, with the bits of the whole)
+bool narrow_ok(const FwdParams &p, int dtype, int64_t N);
+cudaError_t launch_narrow(const FwdParams &p, cudaStream_t stream);
+
 // fused tensor-core product (cci_gemm_pk*.cu): the GEMM of the workspace family
 // with the packed weights (p.values, p.idx, p.G, p.K) expanded into each B tile
 // in shared memory; bf16 only.  gemm_pk_shape_ok: (G, K), packed-array shape and

@@ -1,0 +1,83 @@
+"""Products of at most 128 columns with 1024 reduction indices or more: one launch
+that expands the packed weights as it multiplies, the reduction split over a
+cluster.  Every output against the fp64 oracle at the tolerance of all products
+(1e-5 of sum |w||x|), with the output stage's bf16 rounding where it applies."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1910_11971_gb300 as cci
+from paper_1910_11971_gb300 import workloads as wl
+from parity_util import TOL, assert_within_tol, f64, oracle_reference
+
+pytestmark = pytest.mark.gpu
+BF16 = torch.bfloat16
+
+
+@pytest.fixture(scope="module")
+def dev():
+    return torch.device("cuda:0")
+
+
+# columns at the edges of the MMA's N (16, 32, 64, 128); reductions at the edge of
+# the rule, with a ragged last stage, and deep enough for 2, 4 and 8 parts of
+# unequal length; channels below, at and past a tile of 128; every K, G 4 to 32
+CASES = [(1, 1024, 64, 4, 1), (16, 1032, 72, 8, 2), (17, 1536, 1000, 8, 4), (32, 2048, 128, 16, 8), (33, 1096, 136, 4, 2),
+         (64, 4096, 256, 32, 4), (65, 2056, 160, 32, 1), (100, 2048, 1000, 8, 1), (127, 1160, 96, 16, 2),
+         (128, 3000, 264, 8, 2), (5, 1024, 20, 4, 1), (128, 4096, 4096, 16, 4)]
+
+
+@pytest.mark.parametrize("N,Cin,Cout,G,K", CASES)
+def test_narrow_product(dev, N, Cin, Cout, G, K):
+    X, W = wl.random_small(N + Cin + Cout, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    st = cci.new_status(dev)
+    Y = cci.linear(X.to(dev), v, i, Cout, G, K, status=st)
+    assert cci.read_status(st) == 0
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    assert_within_tol(f64(Y), Yo, S, f"narrow product {N} x {Cin} -> {Cout}")
+
+
+@pytest.mark.parametrize("N,Cin,Cout,G,K", [(16, 1024, 136, 8, 2), (100, 2048, 1000, 8, 4), (3, 4096, 96, 32, 8)])
+@pytest.mark.parametrize("bf16_out", [False, True])
+def test_narrow_product_output_stage(dev, N, Cin, Cout, G, K, bf16_out):
+    X, W = wl.random_small(7 + N, "bf16", N, Cin, Cout)
+    bias = torch.linspace(-2.0, 2.0, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    Y = cci.linear_fused(X.to(dev), v, i, Cout, G, K, bias=bias.to(dev), relu=True,
+                         out_dtype=BF16 if bf16_out else torch.float32)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    b = f64(bias)
+    ref = np.maximum(Yo + b, 0.0)
+    lim = TOL * (S + np.abs(b)) + (2.0 ** -8 * np.abs(ref) if bf16_out else 0.0)
+    assert (np.abs(f64(Y) - ref) <= lim).all()
+
+
+def test_narrow_product_reports_bad_index_sets(dev):
+    """An index >= G, a repeated and an unordered index, each alone in the last
+    group and the last reduction index, are reported."""
+    N, Cin, Cout, G, K = 8, 1032, 264, 8, 4
+    X, W = wl.random_small(3, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    for bad in ([0, 1, 2, G], [0, 1, 1, 2], [0, 2, 1, 3], [255, 1, 2, 3]):
+        j = i.clone()
+        j[-1, -1] = torch.tensor(bad, dtype=torch.uint8)
+        st = cci.new_status(dev)
+        cci.linear(X.to(dev), v, j, Cout, G, K, status=st)
+        assert cci.read_status(st) == 10, bad
+
+
+@pytest.mark.parametrize("N,chunk", [(100, 32), (300, 100)])
+def test_host_chunks_keep_the_bits_of_the_whole(dev, N, chunk):
+    """A host-buffer product cut into chunks of few columns equals the whole
+    product bit for bit: below and above the rule's 128 columns."""
+    Cin, Cout, G, K = 2048, 264, 8, 2
+    X, W = wl.random_small(11, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    Y = cci.linear(X.to(dev), v, i, Cout, G, K).cpu()
+    Yh = cci.linear_host(X.pin_memory(), v, i, Cout, G, K, chunk=chunk)
+    torch.cuda.synchronize()
+    assert torch.equal(Y.view(torch.int32), Yh.view(torch.int32))
