@@ -85,7 +85,8 @@ typedef enum cci_dtype {
 typedef enum cci_algo {
     CCI_ALGO_AUTO = 0,      /* the fastest family this build has for (G, K, dtype, shape): the
                                workspace tensor-core family when a large enough workspace is
-                               given (cci_linear_ws); else the fused tensor-core family
+                               given (cci_linear_ws; its products of few columns need
+                               none); else the fused tensor-core family
                                (CCI_ALGO_DENSE_TC) for bf16 layers that have it; else the
                                CUDA-core families */
     CCI_ALGO_GENERIC = 1,   /* generic kernel: any G <= 256, any K, any alignment */
@@ -119,7 +120,10 @@ typedef enum cci_algo {
                                workspace: plane 0 [Cout][R] fp32 hi, then plane 1
                                [Cout][ceil(R/32)*64] bf16 (per 32-wide chunk of r, 32
                                bf16(hi(w)) then 32 bf16(lo(w))).  Cin % 4 == 0, R % 4 == 0.
-                               Needs cci_workspace_size() bytes */
+                               Needs cci_workspace_size() bytes.  bf16 products of at
+                               most 128 columns and at least 1024 reduction indices
+                               (K <= 8) expand the weights inside the product instead
+                               and leave the workspace as it is */
 } cci_algo;
 
 /*
@@ -421,8 +425,8 @@ cci_status cci_dense_planes(const void *W, cci_dtype dtype, int64_t Cout, int64_
  *     stream capture.  The address is cached for the life of the process: after
  *     cudaDeviceReset() on that device the cached address is stale, so do not
  *     call this entry point again on a device that was reset;
- *   - every call shares the one array per device and leaves it holding the last
- *     call's dense weights; each call rewrites the part it reads, so nothing
+ *   - every call shares the one array per device, which holds the dense weights of
+ *     the last call that used it; each call rewrites the part it reads, so nothing
  *     needs clearing, but calls that overlap on the GPU (other streams, other
  *     threads) race on the array and must be serialised by the caller.
  * Errors: as cci_linear; CCI_ERR_UNSUPPORTED for shapes the dense kernel lacks;
