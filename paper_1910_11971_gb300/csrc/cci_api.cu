@@ -174,7 +174,9 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
         }
         if (dense_ok && ws_ok && aligned(p.X, 16) && aligned(p.Y, 16)) {
             algo = CCI_ALGO_DENSE_TC_WS;
-        } else if (narrow_ok(p, dtype, p.N)) {
+        } else if (narrow_ok(p, dtype, p.N) && fused_may(p, dtype)) {
+            // few columns: as fast and as strict about index sets as the fused family,
+            // for the layers that family takes
             return to_status(launch_narrow(p, stream));
         } else if (!auto_prefers_fused(K)) {
             const int r = try_fused(p, dtype, stream);
