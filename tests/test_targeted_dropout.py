@@ -90,3 +90,44 @@ def test_td_mask_matches_oracle(dtype, Cout, R, G, K, rate):
     assert (m.cpu().numpy() == mr).all()
     got = f64(Wo)
     assert (got == Wr).all() and (np.signbit(got) == np.signbit(Wr)).all()
+
+
+# the vector form (R a multiple of 4, 16-byte aligned tensors): rows of one vector
+# and of a ragged last block, ties, infinities, signed zeros, G 4 to 32
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("Cout,R,G,K,rate", [(64, 4, 4, 1, 0.5), (64, 516, 16, 8, 0.7), (40, 1028, 8, 4, 1.0),
+                                             (64, 12, 32, 8, 0.9), (48, 2052, 16, 1, 0.5), (16, 512, 4, 2, 0.0)])
+@pytest.mark.parametrize("aligned_mask", [True, False])
+def test_td_mask_vectors_match_oracle(dtype, Cout, R, G, K, rate, aligned_mask):
+    from paper_1910_11971_gb300 import build as cci_build
+    cci_build.build()
+    dev = torch.device("cuda:0")
+    g = torch.Generator().manual_seed(Cout + R + K)
+    W = (torch.randn((Cout, R), generator=g) * 2).round() / 2  # ties
+    W[0, :4] = -0.0
+    W[1, 1] = float("inf")
+    W[2, 1] = -float("inf")
+    W = W.to(dtype)
+    u = torch.rand((Cout, R), generator=g)
+    off = 0 if aligned_mask else 1
+    m = torch.empty(Cout * R + 1, dtype=torch.uint8, device=dev)[off:off + Cout * R].view(Cout, R)
+    st = cci.new_status(dev)
+    Wo, m = cci.td_mask(W.to(dev), G, K, rate, u.to(dev), mask=m, status=st)
+    assert cci.read_status(st) == 0
+    Wr, mr = oracle.td_mask(f64(W), G, K, rate, u.numpy())
+    assert (m.cpu().numpy() == mr).all()
+    got = f64(Wo)
+    assert (got == Wr).all() and (np.signbit(got) == np.signbit(Wr)).all()
+
+
+@pytest.mark.gpu
+def test_td_mask_vectors_report_nan():
+    from paper_1910_11971_gb300 import build as cci_build
+    cci_build.build()
+    dev = torch.device("cuda:0")
+    W = torch.randn(16, 64)
+    W[9, 62] = float("nan")
+    st = cci.new_status(dev)
+    cci.td_mask(W.to(dev), 8, 2, 0.5, torch.rand(16, 64).to(dev), status=st)
+    assert cci.read_status(st) == 6
