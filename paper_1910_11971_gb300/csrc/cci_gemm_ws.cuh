@@ -16,10 +16,17 @@
 //                plane 1 over [Cout][ceil(R / 32) * 64] bf16);
 //   activations  one of (the template's ASRC):
 //     kA2d      products: TMA over X[N][Cin];
-//     kA4d      stride-1 convolutions with Cin a multiple of the stage depth:
-//               TMA over X[B][H][W][Cin] with a box of QB x PB x BB output
-//               pixels (QB*PB*BB <= 128 rows), shifted by the tap (kh, kw); the
-//               zero padding is the copy's out-of-range fill;
+//     kA4d      convolutions of strides up to 2: TMA over X[B][H][W][Cin] with a
+//               box of QB x PB x BB output pixels (QB*PB*BB <= 128 rows), shifted
+//               by the tap (kh, kw); the zero padding is the copy's out-of-range
+//               fill.  A stage is a chunk of a tap's channels; Cin is a multiple of
+//               the stage depth;
+//     kATap     the same for the other channel counts, in bf16: a tap's last chunk
+//               is filled with zeros past Cin in both operands (the weights are
+//               copied as [co][tap][ci] boxes) and takes the MMAs of the channels
+//               it has.  Counting them costs the issuing thread some 45 cycles a
+//               stage, so whole stages keep their own form (3x3, 320 -> 32 at 8 x 8:
+//               10.1 us against 11.0 counted);
 //     kAHalo    bf16 3x3 convolutions with unit stride and padding 1: per tile
 //               and 64-channel chunk one TMA copy of the input halo, rows
 //               (p, q) of PB input rows + 2 by Q + 2 columns (the padding is the
@@ -73,7 +80,10 @@
 namespace cci {
 namespace ws {
 
-enum ASrc { kA2d = 0, kA4d = 1, kAGather = 2, kAHalo = 3 };
+enum ASrc { kA2d = 0, kA4d = 1, kAGather = 2, kAHalo = 3, kATap = 4 };
+
+// activations copied as 4-D boxes of output pixels
+__host__ __device__ constexpr bool is_box(int asrc) { return asrc == kA4d || asrc == kATap; }
 
 // output-pixel box of one M tile of a convolution whose activations are copied
 // by 4-D TMA: rows m = (bi*PB + pi)*QB + qi of the tile are the pixels
@@ -139,6 +149,8 @@ struct Cfg {
     static constexpr bool kPairUnits = CG == 2 || MC;  // units of two M tiles over a cluster of two
     static constexpr int kKS = TF32 ? 32 : 64;  // r per stage: one 128-byte row
     static constexpr bool kATma = !TF32 && ASRC != kAGather;  // A copied by TMA into its plane
+    static constexpr bool kTapChunks = ASRC == kATap;
+    static_assert(!kTapChunks || (!TF32 && !PK && EPI == 1 && !MC), "ragged channels: bf16, workspace weights");
     static constexpr bool kHalo = ASRC == kAHalo;  // A: per-chunk halo buffers, stages hold B only
     static_assert(!kHalo || (!TF32 && (CG == 1 || !PK)), "halo copies: bf16 tiles (pairs: workspace weights)");
     // raw fp32 A by TMA; the producers split it into its two planes and write both to
@@ -378,10 +390,27 @@ __device__ __forceinline__ void row3_f16(uint32_t d, uint64_t adesc, uint64_t bd
 // from one block executed by the issuing thread alone.  The separate per-MMA
 // form took ~360 cycles per stage to issue on GB300 (clock stamps), against 512
 // cycles of MMA work: the issue, not the tensor pipe, set the stage period.
-template <uint32_t kIdesc>
+// kCounted: only the first n16 (1-4) MMAs, as stage_f16
+template <uint32_t kIdesc, bool kCounted = false>
 __device__ __forceinline__ void stage_f16_pair(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t acc0,
-                                               uint32_t bar)
+                                               uint32_t bar, uint32_t n16 = 4)
 {
+    if constexpr (kCounted)
+        asm volatile(
+            "{\n.reg .pred pa, p1, p2, p3, pt;\n.reg .b64 ad, bd;\n"
+            "setp.ne.b32 pa, %3, 0;\nsetp.eq.b32 pt, 0, 0;\n"
+            "setp.gt.u32 p1, %7, 1;\nsetp.gt.u32 p2, %7, 2;\nsetp.gt.u32 p3, %7, 3;\n"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %4, pa;\n"
+            "add.s64 ad, %1, 2;\nadd.s64 bd, %2, 2;\n"
+            "@p1 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
+            "add.s64 ad, %1, 4;\nadd.s64 bd, %2, 4;\n"
+            "@p2 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
+            "add.s64 ad, %1, 6;\nadd.s64 bd, %2, 6;\n"
+            "@p3 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%5], %6;\n}\n" ::"r"(d),
+            "l"(adesc), "l"(bdesc), "r"(acc0), "n"(kIdesc), "r"(bar), "h"(static_cast<uint16_t>(3)), "r"(n16)
+            : "memory");
+    else
     asm volatile(
         "{\n.reg .pred pa, pt;\n.reg .b64 ad, bd;\n"
         "setp.ne.b32 pa, %3, 0;\nsetp.eq.b32 pt, 0, 0;\n"
@@ -463,6 +492,15 @@ __device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const void *tmap, i
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
         "{%2, %3}], [%4], %5;" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(bar), "h"(static_cast<uint16_t>(3))
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void *tmap, int c0, int c1, int c2, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+        "{%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
 
@@ -791,7 +829,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     const int taps = p.KH * p.KW;  // kAHalo: stages run chunk by chunk, the taps of a chunk in turn
     volatile int *abort = &S->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nks = static_cast<int>((p.R + kKS - 1) / kKS);
+    const int cpt = is_box(ASRC) ? static_cast<int>((p.Cin + kKS - 1) / kKS) : 1;  // stages per tap (boxes)
+    const int nks = is_box(ASRC) ? taps * cpt : static_cast<int>((p.R + kKS - 1) / kKS);
     const uint32_t crank = C::kPairUnits ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
     // work units: tiles (CG = 1) or pair tiles of 2 x 128 rows (CG = 2), strided over
     // the CTAs (CG = 1) or the CTA pairs (CG = 2)
@@ -827,7 +866,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         S->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (ASRC == kA4d && box.rows < kM) {
+    if (is_box(ASRC) && box.rows < kM) {
         // rows past the box are never copied: keep them zero for the MMAs
         for (uint32_t o = static_cast<uint32_t>(tid) * 16; o < static_cast<uint32_t>(kStages * C::kStage);
              o += C::kThreads * 16)
@@ -851,7 +890,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     }
     if (tid == 288) {
         if constexpr (ASRC == kA2d) tc::tma_prefetch_desc(&tmA.m[0]);
-        if constexpr (ASRC == kA4d)
+        if constexpr (is_box(ASRC))
             for (int i = 0; i < p.sh * p.sw; ++i) tc::tma_prefetch_desc(&tmA.m[i]);
         if constexpr (ASRC == kAHalo) tc::tma_prefetch_desc(&tmA.m[0]);
         if constexpr (!PK) tc::tma_prefetch_desc(&tmB0);
@@ -873,9 +912,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // ------------------------------------------------------------ TMA issuers
         // bytes of one stage's copies: rows x the indices copied per stage (fewer than
         // the stage depth only for bf16 products of fewer than 64 reduction indices,
-        // which run in the two-group short-tile form)
-        const uint32_t erow = static_cast<uint32_t>(EPI == 2 ? p.kin : kKS) * (TF32 ? 4u : 2u);  // bytes per row
-        const uint32_t a_bytes = (ASRC == kA4d ? static_cast<uint32_t>(box.rows) : static_cast<uint32_t>(kM)) * erow;
+        // which run in the two-group short-tile form, and convolutions of fewer channels)
+        const uint32_t erow = static_cast<uint32_t>(EPI == 2 || C::kTapChunks ? p.kin : kKS) * (TF32 ? 4u : 2u);  // bytes per row
+        const uint32_t a_bytes = (is_box(ASRC) ? static_cast<uint32_t>(box.rows) : static_cast<uint32_t>(kM)) * erow;
         const uint32_t b_bytes = static_cast<uint32_t>(C::kBPlanes * C::kBRows) * erow;
         const uint32_t halo_bytes =
             static_cast<uint32_t>((box.QB + p.KW - 1) * (box.PB + p.KH - 1)) * 128u;  // kAHalo
@@ -926,9 +965,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             // a stage's place in its tile: (tap, chunk of kKS channels), chunks innermost
             // (kA4d) or taps innermost (kAHalo); one chunk after the other for products
             int kh = 0, kw = 0, c = 0;
-            const int cpt = ASRC == kA4d ? static_cast<int>(p.Cin / kKS) : 1;  // chunks per tap
             auto step = [&](int by) {
-                if constexpr (ASRC == kA4d) {
+                if constexpr (is_box(ASRC)) {
                     c += by;
                     while (c >= cpt) {
                         c -= cpt;
@@ -960,7 +998,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 if (u >= u_end) break;
                 if (fresh) {
                     split_unit(u, mt, ct);
-                    if constexpr (ASRC == kA4d) bi = box_of(mt, box);
+                    if constexpr (is_box(ASRC)) bi = box_of(mt, box);
                     fresh = false;
                 }
                 if (!tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
@@ -984,7 +1022,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         tc::mbar_arrive_expect_tx(&S->full[s],
                                                   CG * ((PK ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
                     if constexpr (!PK) {
-                        if constexpr (CG == 2) {
+                        if constexpr (C::kTapChunks) {
+                            if constexpr (CG == 2)
+                                tma_load_3d_pair(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, fb);
+                            else
+                                tc::tma_load_3d(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, &S->full[s]);
+                        } else if constexpr (CG == 2) {
                             tma_load_2d_pair(bst, &tmB0, ks * kKS, co0, fb);
                         } else if constexpr (MC) {
                             // this CTA's half of the B rows into both CTAs (the same offsets);
@@ -1006,7 +1049,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                             tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
                         else
                             tc::tma_load_2d(st, &tmA.m[0], ks * kKS, mt * kM, abar);
-                    } else if constexpr (ASRC == kA4d) {
+                    } else if constexpr (is_box(ASRC)) {
                         // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
                         const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
                         const CUtensorMap *m = &tmA.m[th.r * p.sw + tw.r];
@@ -1381,7 +1424,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 int s = 0;
                 uint32_t ph = 0u;  // parity of the full-barrier phase to wait for
                 const uint64_t sunits = C::kStage >> 4, bunits = C::kBOff >> 4;
-                const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;  // MMAs per stage (EPI = 2)
+                // MMAs per stage: the copied indices by 16 (EPI = 2, kTapChunks), fewer in a
+                // tap's last chunk of 64
+                const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;
+                const uint32_t n16_last =
+                    cpt > 1 ? (static_cast<uint32_t>(p.Cin - (cpt - 1) * kKS) + 15u) >> 4 : n16;
+                int left = cpt;  // chunks of the tap still to come, this one among them
                 for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
@@ -1395,14 +1443,20 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t ad = bdesc0 + static_cast<uint64_t>(s) * sunits;
+                        uint32_t n = n16;
+                        if constexpr (C::kTapChunks) {
+                            if (--left == 0) {
+                                left = cpt;
+                                n = n16_last;
+                            }
+                        }
                         if constexpr (CG == 2)
-                            stage_f16_pair<C::kIdesc>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, empty0 + 8u * s);
+                            stage_f16_pair<C::kIdesc, C::kTapChunks>(d, ad, ad + bunits, ks > 0 ? 1u : 0u,
+                                                                     empty0 + 8u * s, n);
+                        else if constexpr (EPI == 2 || C::kTapChunks)  // fewer than four MMAs: R < 64, few channels
+                            stage_f16<C::kIdesc, MC, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s, n);
                         else
-                            if constexpr (EPI == 2)  // short tiles: fewer than four MMAs when R < 64
-                                stage_f16<C::kIdesc, MC, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u,
-                                                               empty0 + 8u * s, n16);
-                            else
-                                stage_f16<C::kIdesc, MC>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
+                            stage_f16<C::kIdesc, MC>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
                         if (++s == kStages) {
                             s = 0;
                             ph ^= 1u;
@@ -1575,7 +1629,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 bias_ct = ct;
             }
             BoxIdx bi{0, 0, 0};
-            if constexpr (ASRC == kA4d || ASRC == kAHalo) bi = box_of(mt, box);
+            if constexpr (is_box(ASRC) || ASRC == kAHalo) bi = box_of(mt, box);
             ok = tc::mbar_wait(&S->tmem_full[acc], (t / 2) & 1, abort, p.status);
             ok = tc::named_and(ebar, 128, ok);
             if (!ok) break;
@@ -1630,7 +1684,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc::named_sync(ebar, 128);
                 if (storer) {
-                    if constexpr (ASRC == kA4d || ASRC == kAHalo)
+                    if constexpr (is_box(ASRC) || ASRC == kAHalo)
                         tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB, bi.bb * box.BB);
                     else
                         tc::tma_store_2d(&tmY, buf, co0 + c0, mt * kM);
@@ -1729,7 +1783,7 @@ inline bool build_a_maps(const FwdParams &p, const ConvBox &box, int asrc, bool 
         const int bx[4] = {64, box.QB + p.KW - 1, box.PB + p.KH - 1, 1};
         return make_map_strided(&am->m[0], p.X, dt, 4, dims, strides, bx);
     }
-    if (asrc != kA4d) return true;
+    if (!is_box(asrc)) return true;
     for (int rh = 0; rh < p.sh; ++rh)
         for (int rw = 0; rw < p.sw; ++rw) {
             const char *base = static_cast<const char *>(p.X) + (rh * p.W + rw) * p.Cin * e;
@@ -1786,14 +1840,16 @@ inline ConvBox choose_box(int64_t B, int64_t P, int64_t Q)
     return best;
 }
 
-// the activation source of a layer for stage depth ks (elements per 128-byte row)
-inline int a_source(const FwdParams &p, int ks)
+// the activation source of a layer for stage depth ks (elements per 128-byte row);
+// any_cin: the stages may be chunks of a tap's channels that end inside the depth
+inline int a_source(const FwdParams &p, int ks, bool any_cin)
 {
     const int64_t lim = int64_t(1) << 30;
     if (!p.is_conv) return p.N < lim ? kA2d : kAGather;
     const bool fits = p.H < lim && p.W < lim && p.N < lim && (p.N / (p.P * p.Q)) < lim;
     const bool strides_ok = p.sh >= 1 && p.sh <= 2 && p.sw >= 1 && p.sw <= 2 && p.H >= p.sh && p.W >= p.sw;
-    return (strides_ok && p.Cin % ks == 0 && fits) ? kA4d : kAGather;
+    if (!strides_ok || !fits) return kAGather;
+    return p.Cin % ks == 0 ? kA4d : (any_cin ? kATap : kAGather);
 }
 
 // N tile among {64, 128, 256} (up to max_bn): fewest rounds of tiles over the
@@ -1816,15 +1872,23 @@ inline int choose_bn(int64_t m_tiles, int64_t Cout, int max_bn, int cg = 1)
 }
 
 // reduction indices a stage copies: the stage depth, or for bf16 products with
-// fewer than 64 indices (one stage) the indices rounded up to 16: narrower copies
-// (no out-of-range fill for three quarters of the box when R = 16) and one MMA per
-// 16 indices (measured on the MobileNetV2 pointwise layers of 16-32 input channels:
-// 20-35 % faster)
+// fewer than 64 indices (one stage) and convolutions of fewer than 64 channels
+// (a stage per tap) that many rounded up to 16: narrower copies (no out-of-range
+// fill for three quarters of the box when R = 16) and one MMA per 16 indices
+// (measured on the MobileNetV2 pointwise layers of 16-32 input channels: 20-35 %
+// faster)
 inline int stage_k_in(const FwdParams &p, bool tf32, int asrc, bool pk)
 {
     if (tf32) return 32;
-    if (pk || asrc != kA2d || p.R >= 64) return 64;
-    return static_cast<int>((p.R + 15) / 16 * 16);
+    const int64_t k = asrc == kATap ? p.Cin : p.R;
+    if (pk || (asrc != kA2d && asrc != kATap) || k >= 64) return 64;
+    return static_cast<int>((k + 15) / 16 * 16);
+}
+
+// bf16 stages of a tile
+inline int64_t stages_of(const FwdParams &p, int asrc)
+{
+    return is_box(asrc) ? static_cast<int64_t>(p.KH) * p.KW * ((p.Cin + 63) / 64) : (p.R + 63) / 64;
 }
 
 template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false>
@@ -1851,10 +1915,16 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     const int elem = TF32 ? 4 : 2;
     const int64_t wdims[2] = {p.R, p.Cout};
     FwdParams q = p;
-    // narrower stage copies only in the short-tile form (one-stage layers land there)
-    q.kin = EPI == 2 ? stage_k_in(p, TF32, ASRC, PK) : C::kKS;
+    // narrower stage copies only in the short-tile form (one-stage products land there)
+    // and for convolutions
+    q.kin = EPI == 2 || C::kTapChunks ? stage_k_in(p, TF32, ASRC, PK) : C::kKS;
     const int wbox[2] = {q.kin, MC ? C::kBRows / 2 : C::kBRows};  // MC: each CTA copies half the rows
-    if (!PK && !make_map(&tmB0, p.wdense, dt, elem, 2, wdims, wbox)) return cudaErrorInvalidValue;
+    if constexpr (C::kTapChunks) {
+        // [co][tap][ci]: a box past the last channel of a tap is filled with zeros
+        const int64_t dims3[3] = {p.Cin, static_cast<int64_t>(p.KH) * p.KW, p.Cout};
+        const int box3[3] = {q.kin, 1, C::kBRows};
+        if (!make_map(&tmB0, p.wdense, dt, elem, 3, dims3, box3)) return cudaErrorInvalidValue;
+    } else if (!PK && !make_map(&tmB0, p.wdense, dt, elem, 2, wdims, wbox)) return cudaErrorInvalidValue;
     if (!PK && C::kBPlanes > 1) {
         // fp32: plane 1 of the split, bf16 [Cout][ceil(R / 32) * 64], one 128-byte row per stage
         const char *pl1 = static_cast<const char *>(p.wdense) + static_cast<size_t>(p.Cout) * p.R * elem;
@@ -1865,7 +1935,7 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     // output rows of 128 bytes: 32 fp32 or 64 bf16 channels
     const CUtensorMapDataType ydt = p.out_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const int yel = p.out_bf16 ? 2 : 4, ysc = p.out_bf16 ? 64 : 32;
-    if constexpr (ASRC == kA4d || ASRC == kAHalo) {
+    if constexpr (is_box(ASRC) || ASRC == kAHalo) {
         const int64_t dims[4] = {p.Cout, p.Q, p.P, box.B};
         const int bx[4] = {ysc, box.QB, box.PB, box.BB};
         if (!make_map(&tmY, p.Y, ydt, yel, 4, dims, bx)) return cudaErrorInvalidValue;
@@ -1877,7 +1947,7 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     const int64_t n_ct = (p.Cout + C::kN - 1) / C::kN;
     if constexpr (C::kHalo && !PK && CG == 1)  // resident weights: single-CTA tiles
         box.resident = (n_ct == 1 && (p.R + C::kKS - 1) / C::kKS <= C::kStages) ? 1 : 0;
-    const int64_t m_tiles = (ASRC == kA4d || ASRC == kAHalo)
+    const int64_t m_tiles = (is_box(ASRC) || ASRC == kAHalo)
                                 ? static_cast<int64_t>(box.nQ) * box.nP * ((box.B + box.BB - 1) / box.BB)
                                          : (p.N + C::kM - 1) / C::kM;
     // CG = 2 or MC: units are pair tiles (two M tiles), one per cluster of two CTAs
@@ -1945,11 +2015,11 @@ inline bool halo_box(const FwdParams &p, const ConvBox &a4d, int64_t min_cin, Co
 // they measured faster than the per-tap copies (128 -> 128 at 28 x 28, 64 images
 // 18.8 -> 16.6 us a pass, 128 images 29.1 -> 24.3 us).  The fused family, whose
 // producers bound it, takes them from 256 on.
-inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t halo_cin = 128)
+inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t halo_cin = 128, bool pk = false)
 {
-    pl->asrc = a_source(p, ks);
+    pl->asrc = a_source(p, ks, !tf32 && !pk);
     pl->box = ConvBox{1, 1, 1, 1, 1, 1, 1};
-    if (pl->asrc == kA4d) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
+    if (is_box(pl->asrc)) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
     ConvBox hb;
     if (pl->asrc == kA4d && !tf32 && halo_box(p, pl->box, halo_cin, &hb)) {
         pl->asrc = kAHalo;
@@ -1964,7 +2034,7 @@ inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t 
 // m tiles of the layer for the chosen activation source
 inline int64_t m_tiles_of(const FwdParams &p, int asrc, const ConvBox &box)
 {
-    if (asrc == kA4d || asrc == kAHalo)
+    if (is_box(asrc) || asrc == kAHalo)
         return static_cast<int64_t>(box.nQ) * box.nP * ((box.B + box.BB - 1) / box.BB);
     return (p.N + 127) / 128;
 }

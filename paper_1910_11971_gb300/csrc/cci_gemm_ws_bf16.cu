@@ -11,17 +11,19 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
     Plan pl;
     plan_layer(p, false, 64, &pl);
     const int asrc = pl.asrc;
-    // products of fewer than 64 reduction indices copy only those (stage_k_in)
+    // products of fewer than 64 reduction indices, and convolutions of fewer than 64
+    // channels, copy only those (stage_k_in)
     const int kin = stage_k_in(p, false, asrc, false);
     if (kin < 64 && !build_a_maps(p, pl.box, asrc, false, kin, &pl.am)) return cudaErrorInvalidValue;
     const int64_t m_tiles = m_tiles_of(p, asrc, pl.box);
-    const int64_t nks = (p.R + 63) / 64;
+    const int64_t nks = stages_of(p, asrc);
     // CTA pairs (256-row tiles, B split over the pair) halve each SM's B traffic,
     // which pays on long reductions with 256-wide N tiles; shorter or narrower
     // layers run faster on single CTAs (measured on the ResNet-50 stack)
-    const bool pair = (asrc == kA2d || asrc == kA4d) && nks >= 16 && choose_bn(m_tiles, p.Cout, 256, 2) == 256;
+    const bool pair = (asrc == kA2d || is_box(asrc)) && nks >= 16 && choose_bn(m_tiles, p.Cout, 256, 2) == 256;
     if (pair) {
         if (asrc == kA2d) return launch_cfg<false, kA2d, 256, 2>(p, pl.box, pl.am, stream);
+        if (asrc == kATap) return launch_cfg<false, kATap, 256, 2>(p, pl.box, pl.am, stream);
         return launch_cfg<false, kA4d, 256, 2>(p, pl.box, pl.am, stream);
     }
     if (asrc == kAHalo) {
@@ -37,7 +39,7 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
     const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
     // tiles of at most 4 stages: the output write dominates, two epilogue groups
     // with two staging buffers each; longer ones keep the shared memory for stages
-    const bool short_k = nks <= 4 && asrc != kAGather;
+    const bool short_k = nks <= 4 && (asrc == kA2d || asrc == kA4d);
     if (short_k) {
 #define CCI_WS_SHORT(A, N) \
     if (asrc == A && bn == N) return launch_cfg<false, A, N, 1, 2>(p, pl.box, pl.am, stream);
@@ -57,6 +59,9 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
     CCI_WS_CASE(kA4d, 64)
     CCI_WS_CASE(kA4d, 128)
     CCI_WS_CASE(kA4d, 256)
+    CCI_WS_CASE(kATap, 64)
+    CCI_WS_CASE(kATap, 128)
+    CCI_WS_CASE(kATap, 256)
     CCI_WS_CASE(kAGather, 64)
     CCI_WS_CASE(kAGather, 128)
     CCI_WS_CASE(kAGather, 256)

@@ -802,6 +802,45 @@ def test_halo_conv3x3_pairs_from_128_channels(dev, B, H, Wi, Cin, Cout):
     assert_within_tol(f64(Y).reshape(-1, Cout), Yo, S, f"halo pairs B={B} {H}x{Wi} {Cin}->{Cout}")
 
 
+# bf16 convolutions whose channel count is no multiple of the 64-deep stage: boxes
+# per tap, the last chunk filled past Cin in both operands.  Fewer channels than
+# one MMA (8), than a stage (24, 40), a ragged last chunk (72, 104, 152); both
+# strides, even kernels without padding, ragged N tiles, pair tiles (160 channels
+# into 512, 27 stages); weights and images with an infinity, whose column must not
+# spread into a neighbouring tap's padding.
+CONV_TAP = [(2, 9, 9, 8, 64, 3, 1, 1), (3, 14, 10, 24, 48, 3, 1, 1), (2, 11, 13, 40, 136, 3, 2, 1),
+            (1, 17, 9, 72, 96, 5, 1, 2), (2, 12, 12, 104, 64, 2, 2, 0), (4, 10, 10, 152, 264, 1, 2, 0),
+            (40, 28, 28, 160, 512, 3, 2, 1)]
+
+
+@pytest.mark.parametrize("B,H,Wi,Cin,Cout,k,stride,pad", CONV_TAP)
+def test_conv_ragged_channels(dev, B, H, Wi, Cin, Cout, k, stride, pad):
+    G, K = 8, 2
+    g = torch.Generator().manual_seed(B + H + Cin + Cout + k)
+    X = torch.randn((B, H, Wi, Cin), generator=g).clamp_min(0).to(BF16)
+    W = torch.randn((Cout, k * k * Cin), generator=g).to(BF16)
+    Y = run_conv(dev, X, W, (k, k, (stride, stride), (pad, pad), Cout), G, K, cci.ALGO_DENSE_TC_WS)
+    assert torch.isfinite(Y).all()
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    for b in {0, B - 1}:
+        Yo, S = oracle.conv2d(f64(X[b:b + 1]), Wd, mask, k, k, (stride, stride), (pad, pad))
+        assert_within_tol(f64(Y[b]).reshape(-1, Cout), Yo, S, f"ragged channels, image {b}")
+
+
+def test_conv_ragged_channels_keep_infinities_in_their_tap(dev):
+    """An infinite weight of tap (1, 1) makes infinities where its input is not
+    zero and NaN where it is, and leaves every other output channel alone."""
+    B, H, Cin, Cout, G, K = 1, 6, 24, 64, 8, 2
+    g = torch.Generator().manual_seed(5)
+    X = (torch.rand((B, H, H, Cin), generator=g) + 0.5).to(BF16)
+    W = torch.randn((Cout, 9, Cin), generator=g).to(BF16)
+    W[3, 4, 23] = float("inf")
+    Y = run_conv(dev, X, W.view(Cout, -1), (3, 3, (1, 1), (1, 1), Cout), G, K, cci.ALGO_DENSE_TC_WS)
+    assert torch.isinf(Y[..., 3]).all() and (Y[..., 3] > 0).all()
+    others = [c for c in range(Cout) if c != 3]
+    assert torch.isfinite(Y[..., others]).all()
+
+
 # ---------------------------------------------------------------------------
 # CTA-pair tiles (tcgen05 cta_group::2): bf16 layers with at least 16 stages of
 # 64 reduction indices and 256-wide N tiles run as 256-row tiles split over two
