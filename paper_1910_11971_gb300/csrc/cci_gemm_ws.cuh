@@ -934,10 +934,13 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     if constexpr (C::kPairUnits) cluster_sync();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S->tmem_base;
-    // launched as a programmatic dependent of the decompression: everything above
-    // overlaps its tail; the workspace (and anything else in memory) is read only
-    // after that grid has completed and its writes are visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // Launched as a programmatic dependent of the decompression: everything above
+    // overlaps its tail.  The workspace is read, and the output written, only after
+    // that grid has completed (tc::wait_prior_grid in each role).  The activations of
+    // a launch directly behind the decompression are read at once (p.a_early): this
+    // grid was scheduled when every block of the decompression had signalled, which
+    // each does after the grid before it, X's producer among all earlier ones, has
+    // completed and is visible.
 
     if (warp >= 9 && warp < 9 + C::kIssuers) {
         // ------------------------------------------------------------ TMA issuers
@@ -957,6 +960,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // 32 KB alike, 25-29 TB/s over the GPU from L2).
         if (C::kHalo && warp == 9) {
             // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows
+            if (!p.a_early) tc::wait_prior_grid();
             if (tc::elect_one()) {
                 int hb = 0;
                 uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
@@ -1020,7 +1024,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             int u = u0, mt = 0, ct = 0;
             BoxIdx bi{0, 0, 0};
             bool fresh = true;  // the tile's coordinates are to be formed
-            while (true) {
+            // kA, kB: the operands copied; both by the loop that runs to the end, and
+            // before it, over the stages of a fresh ring (`most` of them): the
+            // activations while the decompression still runs, then the weights
+            auto copy_stages = [&](auto kA, auto kB, int most) {
+            for (int done = 0; (decltype(kA)::value && decltype(kB)::value) || done < most; ++done) {
+                constexpr bool kCopyA = decltype(kA)::value, kCopyB = decltype(kB)::value;
                 while (ks >= nks && u < u_end) {
                     ks -= nks;
                     u += ustep;
@@ -1032,7 +1041,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     if constexpr (is_box(ASRC)) bi = box_of(mt, box);
                     fresh = false;
                 }
-                if (!tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
+                if (kCopyA && !tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
                 const uint32_t st = base + s * C::kStage;
                 const uint32_t bst = st + C::kBOff;
                 const int co0 = ct * kN + (CG == 2 ? static_cast<int>(crank) * C::kBRows : 0);  // this CTA's B rows
@@ -1048,11 +1057,11 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         tc::tma_load_2d(bst, &tmB0, x, co0, &S->full[s]);
                 } else {
                     // the activation copy completes on aux (raw fp32, split afterwards) or full
-                    if constexpr (C::kARaw) tc::mbar_arrive_expect_tx(&S->aux[s], a_bytes);
-                    if (CG == 1 || crank == 0)
+                    if constexpr (C::kARaw && kCopyA) tc::mbar_arrive_expect_tx(&S->aux[s], a_bytes);
+                    if (kCopyA && (CG == 1 || crank == 0))
                         tc::mbar_arrive_expect_tx(&S->full[s],
                                                   CG * ((PK ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
-                    if constexpr (!PK) {
+                    if constexpr (!PK && kCopyB) {
                         if constexpr (C::kTapChunks) {
                             if constexpr (CG == 2)
                                 tma_load_3d_pair(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, fb);
@@ -1075,12 +1084,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         }
                     }
                     uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
-                    if constexpr (ASRC == kA2d) {
+                    if constexpr (ASRC == kA2d && kCopyA) {
                         if constexpr (CG == 2)
                             tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
                         else
                             tc::tma_load_2d(st, &tmA.m[0], ks * kKS, mt * kM, abar);
-                    } else if constexpr (is_box(ASRC)) {
+                    } else if constexpr (is_box(ASRC) && kCopyA) {
                         // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
                         const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
                         const CUtensorMap *m = &tmA.m[th.r * p.sw + tw.r];
@@ -1099,6 +1108,31 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     ph ^= 1u;
                 }
             }
+            };
+            constexpr std::true_type kYes{};
+            if constexpr (!PK && (ASRC == kA2d || is_box(ASRC))) {
+                if (p.a_early) {
+                    constexpr std::false_type kNo{};
+                    const int most = (kStages - s + kBIssuers - 1) / kBIssuers;  // this warp's stages of the ring
+                    const int s0 = s, ks0 = ks, kh0 = kh, kw0 = kw, c0 = c;
+                    copy_stages(kYes, kNo, most);
+                    s = s0;
+                    ks = ks0;
+                    kh = kh0;
+                    kw = kw0;
+                    c = c0;
+                    u = u0;
+                    ph = 1u;
+                    fresh = true;
+                    tc::wait_prior_grid();
+                    copy_stages(kNo, kYes, most);
+                } else {
+                    tc::wait_prior_grid();
+                }
+            } else {
+                tc::wait_prior_grid();
+            }
+            copy_stages(kYes, kYes, 0);
         }
         __syncwarp();
     } else if (PK && ((warp >= 4 && warp < 8) || warp >= 9 + C::kIssuers)) {
@@ -1113,6 +1147,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // stage may still be in use, and stored once the stage's MMAs released it;
         // then each warp releases its writes to the stage's full barrier (pair: the
         // even CTA's).
+        tc::wait_prior_grid();
         const int q = warp >= 8 ? 1 : 0;
         const int pt = tid - (q ? 32 * (9 + C::kIssuers) : 128);
         const int m0 = (pt >> 3) * 8, c = pt & 7;
@@ -1225,6 +1260,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         if (bad) report(p.status, CCI_ERR_INDEX);
     } else if (warp >= 4 && warp < 8 && C::kEG == 1) {
         // ------------------------------------------------------------ producers
+        if (!C::kATma && !C::kARaw && !p.a_early) tc::wait_prior_grid();  // the gather reads X
         const int pt = tid - 128;
         const int chunk = pt & 7;  // 16-byte chunk of every activation row this thread handles
         const int rowb = pt >> 3;  // rows rowb + 16 i
@@ -1601,6 +1637,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         // ------------------------------------------------------------ epilogue (warps 0-3;
         // with EPI = 2 also warps 4-7 as a second group: group g takes the tiles
         // whose accumulator is g)
+        tc::wait_prior_grid();
         constexpr int kEG = C::kEG;
         const int eg = warp >> 2;              // this thread's group
         const int etid = tid - 128 * eg;       // thread within the group

@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     };
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // a programmatic dependent of the kernel before it
+    tc::wait_prior_grid();  // a programmatic dependent of the kernel before it
+    tc::launch_next_grid();
     if (warp < 4 * kGroups) {
 #pragma unroll
         for (int b = 0; b < NB; ++b)

@@ -106,6 +106,15 @@ __device__ __forceinline__ bool elect_one()
     return e != 0;
 }
 
+// Programmatic dependent launch: wait until the grid before this one has completed
+// and its writes are visible; let the grid after this one be scheduled (it waits
+// the same way before it touches memory).  The GEMM does not signal: with the next
+// layer's blocks scheduled early, at its start or behind its last MMA, a pass of the
+// 3x3 128 -> 128 layer at 28 x 28 went from 16.2 to 18.4 us and the 52-layer stack
+// from 600 to 623 us.
+__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0)
