@@ -160,7 +160,17 @@ struct Cfg {
     static constexpr int kAPlane = kM * 128;                    // bytes: 128-byte rows
     static constexpr int kBPlane = kBRows * 128;
     static constexpr int kBOff = kHalo ? 0 : kAPlanes * kAPlane;  // B planes within a stage
-    static constexpr int kStage = kBOff + kBPlanes * kBPlane;
+    // kRes: a CTA keeps the weights of its N tile, up to kResB chunks of 64 indices, in
+    // shared memory for all its tiles (the launch deals every CTA tiles of one N tile);
+    // the stages hold activations only.  Re-copied per tile, the few lines of a short
+    // tile's weights were read by all SMs at once, which bounded these layers: 16 ->
+    // 64 channels over 1.6 M pixels took longer (92 us) than 32 -> 64 (66 us), whose
+    // weights are twice as many lines.
+    static constexpr bool kRes = EPI == 2;
+    static_assert(!kRes || (kATma && CG == 1 && !PK && !MC && !kTapChunks && !kHalo), "resident weights: short bf16 tiles");
+    static constexpr int kResB = kN > 128 ? 2 : 4;
+    static constexpr int kResBytes = kRes ? kResB * kBPlane : 0;
+    static constexpr int kStage = kRes ? kAPlane : kBOff + kBPlanes * kBPlane;
     static_assert(kStage % 1024 == 0, "stages must keep the 1024-byte swizzle alignment");
     // halo copies: fewer weight stages, the rest of shared memory for a ring of
     // halo buffers whose size and count the host sets per layer (ConvBox)
@@ -177,14 +187,14 @@ struct Cfg {
     static constexpr int kYPerGroup = 2;
     static constexpr int kYBufs = kYPerGroup * kEG;
     static_assert(EPI == 1 || EPI == 2, "epilogue groups");
-    static constexpr int kBudget = static_cast<int>(kMaxSmemPerBlock) - 1024 - kYBufs * kYBuf - 1024;
+    static constexpr int kBudget = static_cast<int>(kMaxSmemPerBlock) - 1024 - kYBufs * kYBuf - kResBytes - kEG * kN * 4 - 1024;
     static constexpr int kStagesFit = (kBudget / kStage) < tc::kMaxStages ? (kBudget / kStage) : tc::kMaxStages;
     static constexpr int kStages = kHalo ? kHaloStages : kStagesFit;
     // accumulators: 2 x kN columns; kARaw adds per stage the A planes (32 + 32 columns)
     static constexpr int kAColBase = 2 * kN;
     static constexpr int kTmemCols = kARaw ? 512 : 2 * kN;
     static constexpr int kBiasBytes = kN * 4;  // biases of one N tile, per epilogue group
-    static constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * kStage + kYBufs * kYBuf +
+    static constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * kStage + kResBytes + kYBufs * kYBuf +
                                     kEG * kBiasBytes + sizeof(tc::Smem) + 64;  // + halo ring
     static constexpr uint32_t kBBytes = kBPlanes * kBPlane;
     static constexpr uint32_t kIdesc = (1u << 4)                                           // D f32
@@ -851,7 +861,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t raw = tc::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t hbuf = base + kStages * C::kStage;  // halo ring (kAHalo: box.nh buffers)
+    const uint32_t resb = base + kStages * C::kStage;  // resident weights (kRes)
+    const uint32_t hbuf = resb + C::kResBytes;         // halo ring (kAHalo: box.nh buffers)
     const uint32_t hbytes = static_cast<uint32_t>(box.hrows) * 128u;
     const uint32_t hring = C::kHalo ? static_cast<uint32_t>(box.nh) * hbytes : 0u;
     const uint32_t ybuf = hbuf + hring;  // output staging buffers, two per epilogue group
@@ -875,6 +886,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     };
 
     if (tid == 0) {
+        // aux[k], kRes: chunk k of the resident weights has landed
         // full[s]: the copy issuer's expect_tx arrival (none for PK halo stages) and
         // PK: one arrival per producer warp of the stage's group in each CTA of the
         // pair (after the warp's writes), else 128 producer arrivals when the
@@ -1060,8 +1072,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     if constexpr (C::kARaw && kCopyA) tc::mbar_arrive_expect_tx(&S->aux[s], a_bytes);
                     if (kCopyA && (CG == 1 || crank == 0))
                         tc::mbar_arrive_expect_tx(&S->full[s],
-                                                  CG * ((PK ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
-                    if constexpr (!PK && kCopyB) {
+                                                  CG * ((PK || C::kRes ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
+                    if constexpr (!PK && !C::kRes && kCopyB) {
                         if constexpr (C::kTapChunks) {
                             if constexpr (CG == 2)
                                 tma_load_3d_pair(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, fb);
@@ -1116,18 +1128,31 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     const int most = (kStages - s + kBIssuers - 1) / kBIssuers;  // this warp's stages of the ring
                     const int s0 = s, ks0 = ks, kh0 = kh, kw0 = kw, c0 = c;
                     copy_stages(kYes, kNo, most);
-                    s = s0;
-                    ks = ks0;
-                    kh = kh0;
-                    kw = kw0;
-                    c = c0;
-                    u = u0;
-                    ph = 1u;
-                    fresh = true;
+                    if constexpr (!C::kRes) {  // back to the first, for the weights
+                        s = s0;
+                        ks = ks0;
+                        kh = kh0;
+                        kw = kw0;
+                        c = c0;
+                        u = u0;
+                        ph = 1u;
+                        fresh = true;
+                    }
                     tc::wait_prior_grid();
-                    copy_stages(kNo, kYes, most);
+                    if constexpr (!C::kRes) copy_stages(kNo, kYes, most);
                 } else {
                     tc::wait_prior_grid();
+                }
+                if constexpr (C::kRes) {
+                    // the activations go on where they stopped; first the weights of this
+                    // CTA's N tile, chunk k by warp 9 + k (kResB <= kBIssuers)
+                    const int k = warp - 9;
+                    if (k < nks && u0 < n_tiles) {
+                        int mt0, ct0;
+                        split_unit(u0, mt0, ct0);
+                        tc::mbar_arrive_expect_tx(&S->aux[k], b_bytes);
+                        tc::tma_load_2d(resb + k * C::kBPlane, &tmB0, k * kKS, ct0 * kN, &S->aux[k]);
+                    }
                 }
             } else {
                 tc::wait_prior_grid();
@@ -1428,7 +1453,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         int it = 0, t = 0;
         bool ok = CG == 1 || crank == 0;
         const int hchunks = ASRC == kAHalo ? nks / taps : 0;
-        const uint64_t hdesc0 = tc::sw128_desc(hbuf), bdesc0 = tc::sw128_desc(base);
+        const uint64_t hdesc0 = tc::sw128_desc(hbuf), bdesc0 = tc::sw128_desc(base), rdesc0 = tc::sw128_desc(resb);
         const uint32_t empty0 = tc::smem_u32(&S->empty[0]);
         const uint32_t issue = tc::elect_one() ? 1u : 0u;  // the lane that issues (a predicate in the stage block)
         auto commit = [&](uint64_t *bar) {
@@ -1490,6 +1515,15 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t ad = bdesc0 + static_cast<uint64_t>(s) * sunits;
+                        uint64_t bd = ad + bunits;
+                        if constexpr (C::kRes) {
+                            if (t == 0) {  // the chunk's weights land once, for the first tile
+                                ok = tc::mbar_wait(&S->aux[ks], 0u, abort, p.status);
+                                if (!ok) break;
+                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            }
+                            bd = rdesc0 + static_cast<uint64_t>(ks) * (C::kBPlane >> 4);
+                        }
                         uint32_t n = n16;
                         if constexpr (C::kTapChunks) {
                             if (--left == 0) {
@@ -1498,12 +1532,11 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                             }
                         }
                         if constexpr (CG == 2)
-                            stage_f16_pair<C::kIdesc, C::kTapChunks>(d, ad, ad + bunits, ks > 0 ? 1u : 0u,
-                                                                     empty0 + 8u * s, n);
+                            stage_f16_pair<C::kIdesc, C::kTapChunks>(d, ad, bd, ks > 0 ? 1u : 0u, empty0 + 8u * s, n);
                         else if constexpr (EPI == 2 || C::kTapChunks)  // fewer than four MMAs: R < 64, few channels
-                            stage_f16<C::kIdesc, MC, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s, n);
+                            stage_f16<C::kIdesc, MC, true>(d, ad, bd, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s, n);
                         else
-                            stage_f16<C::kIdesc, MC>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
+                            stage_f16<C::kIdesc, MC>(d, ad, bd, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
                         if (++s == kStages) {
                             s = 0;
                             ph ^= 1u;
@@ -1919,6 +1952,10 @@ inline int choose_bn(int64_t m_tiles, int64_t Cout, int max_bn, int cg = 1)
     return best;
 }
 
+// CTAs of a launch with resident weights: whole rounds of the N tiles, so that a
+// CTA's tiles (every grid-th) are of one N tile
+inline int64_t resident_slots(int64_t n_ct) { return sm_count() / n_ct * n_ct; }
+
 // reduction indices a stage copies: the stage depth, or for bf16 products with
 // fewer than 64 indices (one stage) and convolutions of fewer than 64 channels
 // (a stage per tap) that many rounded up to 16: narrower copies (no out-of-range
@@ -2009,7 +2046,8 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
         box.byC = TileDiv(p.Cin);
         box.byKW = TileDiv(p.KW);
     }
-    const int64_t slots = sm_count() / kCl;
+    const int64_t slots = C::kRes ? resident_slots(n_ct) : sm_count() / kCl;
+    if (C::kRes && ((p.R + 63) / 64 > C::kResB || slots == 0)) return cudaErrorInvalidValue;
     const int64_t grid = kCl * (n_tiles < slots ? n_tiles : slots);
     // programmatic dependent launch: may start once every block of the preceding
     // kernel on the stream (the decompression) has signalled; it waits for that

@@ -36,13 +36,16 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
             return launch_cfg<false, kAHalo, 128, 2>(p, pl.box, pl.am, stream);
         return launch_cfg<false, kAHalo, 64, 1>(p, pl.box, pl.am, stream);  // 64 channels out, or one M tile
     }
-    const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
-    // tiles of at most 4 stages: the output write dominates, two epilogue groups
-    // with two staging buffers each; longer ones keep the shared memory for stages
-    const bool short_k = nks <= 4 && (asrc == kA2d || asrc == kA4d);
+    // tiles of at most 4 stages: the output write dominates, two epilogue groups with
+    // two staging buffers each, and the weights of a CTA's N tile resident (two chunks
+    // of 256 channels or four of 128), when the N tiles leave less than a tenth of the
+    // SMs without whole rounds of them; longer ones keep the shared memory for stages
+    const int sbn = choose_bn(m_tiles, p.Cout, nks <= 2 ? 256 : 128, 1);
+    const bool short_k = nks <= 4 && (asrc == kA2d || asrc == kA4d) &&
+                         10 * resident_slots((p.Cout + sbn - 1) / sbn) >= 9 * sm_count();
     if (short_k) {
 #define CCI_WS_SHORT(A, N) \
-    if (asrc == A && bn == N) return launch_cfg<false, A, N, 1, 2>(p, pl.box, pl.am, stream);
+    if (asrc == A && sbn == N) return launch_cfg<false, A, N, 1, 2>(p, pl.box, pl.am, stream);
         CCI_WS_SHORT(kA2d, 64)
         CCI_WS_SHORT(kA2d, 128)
         CCI_WS_SHORT(kA2d, 256)
@@ -51,6 +54,7 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
         CCI_WS_SHORT(kA4d, 256)
 #undef CCI_WS_SHORT
     }
+    const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
 #define CCI_WS_CASE(A, N) \
     if (asrc == A && bn == N) return launch_cfg<false, A, N, 1>(p, pl.box, pl.am, stream);
     CCI_WS_CASE(kA2d, 64)
