@@ -802,6 +802,24 @@ def test_halo_conv3x3_pairs_from_128_channels(dev, B, H, Wi, Cin, Cout):
     assert_within_tol(f64(Y).reshape(-1, Cout), Yo, S, f"halo pairs B={B} {H}x{Wi} {Cin}->{Cout}")
 
 
+# short tiles (1 to 4 stages) with resident weights: more tiles than SMs, so every
+# CTA runs several tiles of its N tile; 1, 2, 3 and 5 N tiles (152, 152, 150 and 150
+# CTAs), one that leaves too few whole rounds (100 N tiles: the form without), a
+# ragged last M tile, fewer indices than a chunk and a ragged last chunk
+@pytest.mark.parametrize("N,Cin,Cout,G,K", [(20005, 16, 96, 8, 2), (10011, 128, 512, 8, 2), (6500, 72, 520, 8, 2),
+                                            (4200, 256, 640, 16, 4), (20100, 200, 64, 4, 1), (260, 64, 25600, 8, 2)])
+def test_short_tiles_resident_weights(dev, N, Cin, Cout, G, K):
+    X, W = wl.random_small(N + Cin, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    st = cci.new_status(dev)
+    Y = cci.linear(X.to(dev), v, i, Cout, G, K, status=st)
+    assert cci.read_status(st) == 0 and torch.isfinite(Y).all()
+    rows = sample_rows(N, 200, seed=N)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X[rows]), Wd, mask)
+    assert_within_tol(f64(Y[torch.from_numpy(rows).to(dev)]), Yo, S, f"resident weights {N} x {Cin} -> {Cout}")
+
+
 # bf16 convolutions whose channel count is no multiple of the 64-deep stage: boxes
 # per tap, the last chunk filled past Cin in both operands.  Fewer channels than
 # one MMA (8), than a stage (24, 40), a ragged last chunk (72, 104, 152); both
