@@ -26,10 +26,10 @@
  *
  * Ownership and execution: the caller allocates every buffer; all data pointers
  * are DEVICE pointers (except the X_host / Y_host of cci_linear_host); the
- * library allocates nothing.  It keeps no state between calls except two
- * per-device caches, both filled on a device's first use: the dynamic
- * shared-memory limit set on each tensor-core kernel, and the device address of
- * the static scratch array of cci_linear_dense_tc_static (see there).  Every
+ * library allocates nothing.  It keeps no state between calls except three
+ * per-device caches, filled on a device's first use: the dynamic shared-memory
+ * limit set on each tensor-core kernel, the device's number of SMs, and the device
+ * address of the static scratch array of cci_linear_dense_tc_static (see there).  Every
  * call is asynchronous on `stream` (NULL = the legacy default stream) and
  * returns once its kernels are enqueued.  Calls on different streams may run
  * concurrently when their outputs do not overlap.

@@ -72,6 +72,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "cci_tc_common.cuh"
@@ -116,6 +117,7 @@ struct ConvBox {
                      // (one N tile, every stage of a tile a stage of the ring): the
                      // weights are copied for the CTA's first tile only
     TileDiv byQ, byP, byN;  // division by nQ, by nP and by the N tiles (set at the launch)
+    int log_split = 0;      // SK: a tile's reduction is split over a cluster of 1 << log_split CTAs
     TileDiv byC, byKW;      // gather: division of a reduction index by Cin, of a tap by KW
 };
 
@@ -132,7 +134,13 @@ struct AMaps {
 // EPI = 2: a second epilogue group (warps 4-7, idle when bf16 activations are
 // copied by TMA) and two staging buffers per group, for layers whose tiles have
 // few stages (the output write dominates); EPI = 1: one group, more stages
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
+// SK: few tiles with long reductions.  A tile is a cluster of 2, 4 or 8 CTAs, each
+// of which multiplies its share of the stages (one tile per cluster, so the grid is
+// the whole work); then each owns 1 / parts of the tile's columns: every CTA stores
+// its sums of them into the owner's shared memory (straight from tensor memory, 512
+// bytes a warp), and after one cluster barrier the owner adds them in rank order and
+// writes its columns with plain stores.
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false, bool SK = false>
 struct Cfg {
     static constexpr int kM = 128, kN = BN;
     static_assert(CG == 1 || (CG == 2 && !TF32 && ASRC != kAGather), "pair mode: bf16 with TMA activations");
@@ -185,7 +193,9 @@ struct Cfg {
     // 13.9 against 12.9 for 256 -> 64 at 56 x 56.
     static constexpr int kEG = (kATma && EPI == 2) ? 2 : 1;
     static constexpr int kYPerGroup = 2;
-    static constexpr int kYBufs = kYPerGroup * kEG;
+    static_assert(!SK || (CG == 1 && EPI == 1 && !PK && !MC && ASRC != kAHalo && BN <= 128), "split tiles");
+    // SK: the exchanged sums (parts x [BN / parts / 4][128 rows][4]) instead
+    static constexpr int kYBufs = SK ? BN * 512 / kYBuf : kYPerGroup * kEG;
     static_assert(EPI == 1 || EPI == 2, "epilogue groups");
     static constexpr int kBudget = static_cast<int>(kMaxSmemPerBlock) - 1024 - kYBufs * kYBuf - kResBytes - kEG * kN * 4 - 1024;
     static constexpr int kStagesFit = (kBudget / kStage) < tc::kMaxStages ? (kBudget / kStage) : tc::kMaxStages;
@@ -451,6 +461,19 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t local, uint32_t rank)
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
     return r;
+}
+
+// 16 bytes into the shared memory of a CTA of the cluster (shared::cluster address)
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
 }
 
 __device__ __forceinline__ void cluster_sync()
@@ -849,13 +872,13 @@ __device__ __forceinline__ TapSite tap_site(int a, int stride)
 
 // PK: tmB0 / tmB1 are the maps of the packed values and indices (2-D over
 // [Cout/G][R*K]); otherwise the maps of the workspace planes
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
-__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads, 1)
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false, bool SK = false>
+__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThreads, 1)
     gemm_ws_kernel(FwdParams p, const __grid_constant__ AMaps tmA, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmY, ConvBox box,
                    int n_tiles)
 {
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
     constexpr int kM = C::kM, kN = C::kN, kKS = C::kKS, kStages = C::kStages;
     constexpr int kLag = 2;  // bf16 gather: stages in flight before a producer's arrive
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -872,12 +895,17 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     volatile int *abort = &S->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cpt = is_box(ASRC) ? static_cast<int>((p.Cin + kKS - 1) / kKS) : 1;  // stages per tap (boxes)
-    const int nks = is_box(ASRC) ? taps * cpt : static_cast<int>((p.R + kKS - 1) / kKS);
-    const uint32_t crank = C::kPairUnits ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
+    const int nks_all = is_box(ASRC) ? taps * cpt : static_cast<int>((p.R + kKS - 1) / kKS);
+    const uint32_t crank = C::kPairUnits || SK ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
     // work units: tiles (CG = 1) or pair tiles of 2 x 128 rows (CG = 2), strided over
     // the CTAs (CG = 1) or the CTA pairs (CG = 2)
-    const int u0 = C::kPairUnits ? blockIdx.x / 2 : blockIdx.x;
-    const int ustep = C::kPairUnits ? gridDim.x / 2 : gridDim.x;
+    const int u0 = C::kPairUnits ? blockIdx.x / 2 : (SK ? blockIdx.x >> box.log_split : blockIdx.x);
+    const int ustep = C::kPairUnits ? gridDim.x / 2 : (SK ? gridDim.x >> box.log_split : gridDim.x);
+    // this CTA's stages of a tile: kbase .. kbase + nks - 1 (all of them unless SK)
+    const int kbase =
+        SK ? static_cast<int>((static_cast<int64_t>(crank) * nks_all) >> box.log_split) : 0;
+    const int nks =
+        SK ? static_cast<int>((static_cast<int64_t>(crank + 1) * nks_all) >> box.log_split) - kbase : nks_all;
     // unit u -> (M tile, N tile)
     auto split_unit = [&](int u, int &mt, int &ct) {
         const int q = static_cast<int>(box.byN.quot(static_cast<uint32_t>(u)));
@@ -943,7 +971,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     // the pair's barriers are initialised before either CTA signals the other's
-    if constexpr (C::kPairUnits) cluster_sync();
+    // (SK: every CTA of the cluster runs before another stores into it)
+    if constexpr (C::kPairUnits || SK) cluster_sync();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S->tmem_base;
     // Launched as a programmatic dependent of the decompression: everything above
@@ -1030,7 +1059,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     }
                 }
             };
-            step(ks);
+            step(ks + kbase);
             // resident weights (halo copies): only the first tile's stages are copied
             const int u_end = C::kHalo && box.resident ? (u0 + 1 < n_tiles ? u0 + 1 : n_tiles) : n_tiles;
             int u = u0, mt = 0, ct = 0;
@@ -1080,7 +1109,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                             else
                                 tc::tma_load_3d(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, &S->full[s]);
                         } else if constexpr (CG == 2) {
-                            tma_load_2d_pair(bst, &tmB0, ks * kKS, co0, fb);
+                            tma_load_2d_pair(bst, &tmB0, (ks + kbase) * kKS, co0, fb);
                         } else if constexpr (MC) {
                             // this CTA's half of the B rows into both CTAs (the same offsets);
                             // each CTA's full barrier expects the whole tile
@@ -1090,9 +1119,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                             if constexpr (C::kBPlanes > 1)
                                 tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, fb);
                         } else {
-                            tc::tma_load_2d(bst, &tmB0, ks * kKS, co0, &S->full[s]);
+                            tc::tma_load_2d(bst, &tmB0, (ks + kbase) * kKS, co0, &S->full[s]);
                             if constexpr (C::kBPlanes > 1)  // fp32 plane 1: 64 bf16 per stage
-                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, co0, &S->full[s]);
+                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, (ks + kbase) * 64, co0, &S->full[s]);
                         }
                     }
                     uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
@@ -1100,7 +1129,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         if constexpr (CG == 2)
                             tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
                         else
-                            tc::tma_load_2d(st, &tmA.m[0], ks * kKS, mt * kM, abar);
+                            tc::tma_load_2d(st, &tmA.m[0], (ks + kbase) * kKS, mt * kM, abar);
                     } else if constexpr (is_box(ASRC) && kCopyA) {
                         // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
                         const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
@@ -1318,7 +1347,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     }
                     xsite_tile = tile;
                 }
-                const int64_t r = static_cast<int64_t>(ks) * kKS + chunk * 4;
+                const int64_t r = static_cast<int64_t>(ks + kbase) * kKS + chunk * 4;
                 if (r >= p.R) return;
                 const GatherTap g = gather_tap(p, box, r);
                 const float *X = static_cast<const float *>(p.X) + g.off;
@@ -1336,10 +1365,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         auto advance = [&](int64_t &tile, int &ks) {
             if (++ks == nks) {
                 ks = 0;
-                tile += gridDim.x;
+                tile += ustep;
             }
         };
-        int64_t t2 = blockIdx.x;
+        int64_t t2 = u0;
         int k2 = 0;
         if constexpr (kRegs) {
             load_x(xa, t2, k2);
@@ -1375,7 +1404,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                     const uint32_t st = base + s * C::kStage;
                     if constexpr (!TF32) {
                         const uint16_t *X = static_cast<const uint16_t *>(p.X);
-                        const int64_t r = static_cast<int64_t>(ks) * kKS + chunk * 8;
+                        const int64_t r = static_cast<int64_t>(ks + kbase) * kKS + chunk * 8;
                         const GatherTap g = gather_tap(p, box, r < p.R ? r : 0);
                         const uint32_t H = static_cast<uint32_t>(p.H), W = static_cast<uint32_t>(p.W);
 #pragma unroll
@@ -1501,7 +1530,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                 const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;
                 const uint32_t n16_last =
                     cpt > 1 ? (static_cast<uint32_t>(p.Cin - (cpt - 1) * kKS) + 15u) >> 4 : n16;
-                int left = cpt;  // chunks of the tap still to come, this one among them
+                int left = cpt - kbase % cpt;  // chunks of the tap still to come, this one among them
                 for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
@@ -1716,6 +1745,24 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
             if (!ok) break;
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if constexpr (SK) {
+                // this part's sums of four columns and 128 rows to the columns' owner
+                const int log_cols = (BN == 64 ? 6 : 7) - box.log_split;  // columns of an owner: 1 << log_cols
+                const uint32_t at = ybuf + (crank << (log_cols - 2)) * 2048u + static_cast<uint32_t>(m) * 16u;
+#pragma unroll 1
+                for (int c0 = 0; c0 < kN && co0 + c0 < p.Cout; c0 += 32) {
+                    uint32_t v[32];
+                    tc::tmem_ld32(tmem + lane_off + static_cast<uint32_t>(acc * kN + c0), v);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t c = static_cast<uint32_t>(c0 + 4 * j);
+                        if (co0 + c0 + 4 * j >= p.Cout) break;
+                        st_cluster_v4(map_to_rank(at + ((c & ((1u << log_cols) - 1u)) >> 2) * 2048u, c >> log_cols),
+                                      v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    }
+                }
+                continue;
+            }
             const int sc = p.out_bf16 ? 64 : 32;  // output columns per staged 128-byte row
             const int cend = (p.Cout - co0) < kN ? static_cast<int>(p.Cout - co0) : kN;
 #pragma unroll 1
@@ -1780,7 +1827,57 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     __syncthreads();
     // CG = 2: neither CTA leaves (or frees tensor memory) while the other may still
     // signal its barriers or the pair's MMAs may read its shared memory
-    if constexpr (C::kPairUnits) cluster_sync();
+    if constexpr (C::kPairUnits || SK) cluster_sync();
+    if constexpr (SK) {
+        // every part's sums of this CTA's columns have landed (and nothing is stored into
+        // another CTA any more): row m of the tile, four columns at a time
+        if (warp < 4 && u0 < n_tiles) {
+            int mt, ct;
+            split_unit(u0, mt, ct);
+            int64_t n = -1;  // the row's column of the output, none past the box or the layer
+            if constexpr (is_box(ASRC)) {
+                const BoxIdx bi = box_of(mt, box);
+                const int qp = box.QB * box.PB, b = tid / qp, r = tid - b * qp, pi = r / box.QB, qi = r - pi * box.QB;
+                const int64_t ob = static_cast<int64_t>(bi.bb) * box.BB + b, op = bi.pb * box.PB + pi,
+                              oq = bi.qb * box.QB + qi;
+                if (tid < box.rows && ob < box.B && op < p.P && oq < p.Q) n = (ob * p.P + op) * p.Q + oq;
+            } else {
+                n = static_cast<int64_t>(mt) * kM + tid;
+                if (n >= p.N) n = -1;
+            }
+            const int cols = kN >> box.log_split, parts = 1 << box.log_split;
+            if (n >= 0) {
+                for (int q = 0; q < cols / 4; ++q) {
+                    const int cl = static_cast<int>(crank) * cols + 4 * q, co = ct * kN + cl;  // Cout is a multiple of 4
+                    if (co >= p.Cout) break;
+                    const uint32_t at = ybuf + static_cast<uint32_t>(q) * 2048u + static_cast<uint32_t>(tid) * 16u;
+                    float4 y = ld_shared_f4(at);
+                    for (int j = 1; j < parts; ++j) {
+                        const float4 z = ld_shared_f4(at + static_cast<uint32_t>(j * (cols / 4)) * 2048u);
+                        y.x += z.x;
+                        y.y += z.y;
+                        y.z += z.z;
+                        y.w += z.w;
+                    }
+                    if (p.bias) {
+                        const float4 b = ld_shared_f4(sbias + 4u * static_cast<uint32_t>(cl));
+                        y.x += b.x;
+                        y.y += b.y;
+                        y.z += b.z;
+                        y.w += b.w;
+                    }
+                    if (p.relu) y = make_float4(fmaxf(y.x, 0.f), fmaxf(y.y, 0.f), fmaxf(y.z, 0.f), fmaxf(y.w, 0.f));
+                    if (p.out_bf16)
+                        *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(p.Y) + n * p.Cout + co) =
+                            make_uint2(bf16x2_rn(__float_as_uint(y.x), __float_as_uint(y.y)),
+                                       bf16x2_rn(__float_as_uint(y.z), __float_as_uint(y.w)));
+                    else
+                        *reinterpret_cast<float4 *>(p.Y + n * p.Cout + co) = y;
+                }
+            }
+        }
+        __syncwarp();
+    }
     if (warp == 8) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if constexpr (CG == 2)
@@ -1876,12 +1973,20 @@ inline bool build_a_maps(const FwdParams &p, const ConvBox &box, int asrc, bool 
     return true;
 }
 
+// SMs of the current device (a constant of the device, looked up on its first use:
+// the choices of a launch ask for it a dozen times)
 inline int sm_count()
 {
+    static std::atomic<int> known[SmemAttrCache::kDevices];
     int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= SmemAttrCache::kDevices) return 1;
+    sms = known[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        sms = sms > 0 ? sms : 1;
+        known[dev].store(sms, std::memory_order_relaxed);
+    }
+    return sms;
 }
 
 // the next larger box extent that covers n in fewer boxes than extent e does (the
@@ -1894,22 +1999,27 @@ inline int next_extent(int n, int e)
 
 // the output-pixel box with the fewest M tiles (ties: longer runs along q, then
 // p).  Only the smallest box of each tile count along q and p is tried, and those
-// are stepped through directly: a call's host time is the floor of a small layer.
-inline ConvBox choose_box(int64_t B, int64_t P, int64_t Q)
+// are stepped through directly, in 32 bits: a call's host time is the floor of a
+// small layer.
+inline ConvBox choose_box(int64_t B_, int64_t P, int64_t Q)
 {
-    ConvBox best{1, 1, 1, 1, 1, 1, B};
+    ConvBox best{1, 1, 1, 1, 1, 1, B_};
     int64_t best_tiles = -1;
-    const int q_all = static_cast<int>(Q), p_all = static_cast<int>(P);  // below 2^30 (a_source)
+    const int q_all = static_cast<int>(Q), p_all = static_cast<int>(P), B = static_cast<int>(B_);  // below 2^30 (a_source)
+    int ext[128], num[128], n_ext = 0;  // extents along p up to 128 and the boxes they make
+    for (int PB = 1; PB <= p_all && PB <= 128; PB = next_extent(p_all, PB)) {
+        ext[n_ext] = PB;
+        num[n_ext++] = (p_all + PB - 1) / PB;
+    }
     for (int QB = 1; QB <= q_all && QB <= 128; QB = next_extent(q_all, QB)) {
-        const int64_t nq = (q_all + QB - 1) / QB;
-        for (int PB = 1; PB <= p_all && QB * PB <= 128; PB = next_extent(p_all, PB)) {
-            const int64_t np = (p_all + PB - 1) / PB;
-            const int BB = (128 / (QB * PB)) < B ? 128 / (QB * PB) : static_cast<int>(B);
-            const int64_t tiles = nq * np * ((B + BB - 1) / BB);
+        const int nq = (q_all + QB - 1) / QB;
+        for (int i = 0; i < n_ext && QB * ext[i] <= 128; ++i) {
+            const int fit = 128 / (QB * ext[i]), BB = fit < B ? fit : B;
+            const int64_t tiles = static_cast<int64_t>(nq) * num[i] * ((B + BB - 1) / BB);
             if (best_tiles < 0 || tiles <= best_tiles) {
                 best_tiles = tiles;
                 best.QB = QB;
-                best.PB = PB;
+                best.PB = ext[i];
                 best.BB = BB;
             }
         }
@@ -1917,7 +2027,7 @@ inline ConvBox choose_box(int64_t B, int64_t P, int64_t Q)
     best.nQ = static_cast<int>((Q + best.QB - 1) / best.QB);
     best.nP = static_cast<int>((P + best.PB - 1) / best.PB);
     best.rows = best.QB * best.PB * best.BB;
-    best.B = B;
+    best.B = B_;
     return best;
 }
 
@@ -1956,6 +2066,52 @@ inline int choose_bn(int64_t m_tiles, int64_t Cout, int max_bn, int cg = 1)
 // CTA's tiles (every grid-th) are of one N tile
 inline int64_t resident_slots(int64_t n_ct) { return sm_count() / n_ct * n_ct; }
 
+// clusters of 1 << log_parts CTAs (one per SM) that run at once: they stay inside a
+// GPC, so larger ones leave SMs over (152 SMs: 76, 36 and 15)
+inline int64_t cluster_slots(int log_parts, int64_t sms)
+{
+    return log_parts == 0 ? sms : (log_parts == 1 ? sms / 2 : (log_parts == 2 ? sms * 15 / 64 : sms / 10));
+}
+
+// Split of the reduction of a layer with few tiles (SK): N tile and CTAs per tile.
+// Costs in SM cycles, measured on GB300: a stage (c64, c128: for N tiles of 64 and
+// 128), a tile's fill and epilogue, the exchange of the parts' sums (distributed
+// shared memory takes about 20 bytes a cycle and SM: 64 KB of sums for a 128-wide
+// tile).  The layer is split when that saves a seventh; a part keeps four stages at
+// least.  Without the exchange's share the 512 -> 512 layer at 7 x 7, 32 images was
+// split in two and went from 15.2 to 16.5 us.
+struct Split {
+    int log_parts = 0, bn = 0;
+};
+inline Split choose_split(int64_t m_tiles, int64_t Cout, int64_t nks, int64_t c64, int64_t c128)
+{
+    constexpr int64_t kTile = 4500;
+    const int64_t sms = sm_count();
+    Split best;
+    int64_t whole = -1, cost = -1;
+    for (int bn = 64; bn <= 128; bn *= 2) {
+        const int64_t tiles = m_tiles * ((Cout + bn - 1) / bn), c = bn == 64 ? c64 : c128;
+        const int64_t t = (tiles + sms - 1) / sms * nks * c + kTile;
+        if (whole < 0 || t < whole) whole = t;
+        for (int l = 1; l <= 3 && tiles <= cluster_slots(l, sms) && nks >= (4 << l); ++l) {
+            const int64_t s = ((nks + (1 << l) - 1) >> l) * c + kTile + 1000 + 26 * bn;
+            if (cost < 0 || s < cost) {
+                cost = s;
+                best.log_parts = l;
+                best.bn = bn;
+            }
+        }
+    }
+    return cost >= 0 && 7 * cost < 6 * whole ? best : Split{};
+}
+
+// M tiles that the choice of a split counts: those of the whole call (a chunk of a
+// host-buffer product runs with the bits of the whole)
+inline int64_t call_m_tiles(const FwdParams &p, int64_t m_tiles)
+{
+    return p.N_call ? (p.N_call + 127) / 128 : m_tiles;
+}
+
 // reduction indices a stage copies: the stage depth, or for bf16 products with
 // fewer than 64 indices (one stage) and convolutions of fewer than 64 channels
 // (a stage per tap) that many rounded up to 16: narrower copies (no out-of-range
@@ -1976,11 +2132,13 @@ inline int64_t stages_of(const FwdParams &p, int asrc)
     return is_box(asrc) ? static_cast<int64_t>(p.KH) * p.KW * ((p.Cin + 63) / 64) : (p.R + 63) / 64;
 }
 
-template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false>
-cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &tmA, cudaStream_t stream)
+// log_split: SK only, the CTAs of a tile (1 << log_split)
+template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false, bool SK = false>
+cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &tmA, cudaStream_t stream,
+                       int log_split = 0)
 {
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
-    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK, MC>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
+    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
     ConvBox box = box_in;
     size_t smem = C::kSmem;
     if constexpr (C::kHalo) {
@@ -2048,7 +2206,8 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     }
     const int64_t slots = C::kRes ? resident_slots(n_ct) : sm_count() / kCl;
     if (C::kRes && ((p.R + 63) / 64 > C::kResB || slots == 0)) return cudaErrorInvalidValue;
-    const int64_t grid = kCl * (n_tiles < slots ? n_tiles : slots);
+    box.log_split = log_split;
+    const int64_t grid = SK ? n_tiles << log_split : kCl * (n_tiles < slots ? n_tiles : slots);
     // programmatic dependent launch: may start once every block of the preceding
     // kernel on the stream (the decompression) has signalled; it waits for that
     // kernel's completion before reading memory
@@ -2061,11 +2220,11 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     la[0].val.programmaticStreamSerializationAllowed = 1;
     la[1].id = cudaLaunchAttributeClusterDimension;
-    la[1].val.clusterDim.x = kCl;
+    la[1].val.clusterDim.x = SK ? 1u << log_split : kCl;
     la[1].val.clusterDim.y = 1;
     la[1].val.clusterDim.z = 1;
     cfg.attrs = la;
-    cfg.numAttrs = kCl == 2 ? 2 : 1;
+    cfg.numAttrs = kCl == 2 || SK ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box,
                                              static_cast<int>(n_tiles));
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -2077,6 +2236,7 @@ struct Plan {
     int asrc;
     ConvBox box;
     AMaps am;
+    ConvBox a4d;  // the pixel box that halo copies were taken instead of
 };
 // halo box of a bf16 3x3, stride-1, padding-1 convolution: PB output rows of
 // the full width per tile.  Used for layers of min_cin input channels or more
@@ -2105,13 +2265,15 @@ inline bool halo_box(const FwdParams &p, const ConvBox &a4d, int64_t min_cin, Co
 // they measured faster than the per-tap copies (128 -> 128 at 28 x 28, 64 images
 // 18.8 -> 16.6 us a pass, 128 images 29.1 -> 24.3 us).  The fused family, whose
 // producers bound it, takes them from 256 on.
+// halo_cin < 0: no halo copies
 inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t halo_cin = 128, bool pk = false)
 {
     pl->asrc = a_source(p, ks, !tf32 && !pk);
     pl->box = ConvBox{1, 1, 1, 1, 1, 1, 1};
     if (is_box(pl->asrc)) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
+    pl->a4d = pl->box;
     ConvBox hb;
-    if (pl->asrc == kA4d && !tf32 && halo_box(p, pl->box, halo_cin, &hb)) {
+    if (pl->asrc == kA4d && !tf32 && halo_cin >= 0 && halo_box(p, pl->box, halo_cin, &hb)) {
         pl->asrc = kAHalo;
         pl->box = hb;
     }

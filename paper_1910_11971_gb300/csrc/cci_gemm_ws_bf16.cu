@@ -17,6 +17,29 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
     if (kin < 64 && !build_a_maps(p, pl.box, asrc, false, kin, &pl.am)) return cudaErrorInvalidValue;
     const int64_t m_tiles = m_tiles_of(p, asrc, pl.box);
     const int64_t nks = stages_of(p, asrc);
+    // few tiles with a long reduction: split over clusters (3x3 layers of halo copies
+    // from per-tap boxes)
+    {
+        const int src = asrc == kAHalo ? kA4d : asrc;
+        const int64_t mt = call_m_tiles(p, m_tiles_of(p, src, pl.a4d)), stages = stages_of(p, src);
+        const Split sp = src == kAGather ? choose_split(mt, p.Cout, stages, 800, 800)
+                                         : choose_split(mt, p.Cout, stages, 220, 265);
+        if (sp.log_parts > 0) {
+            if (asrc == kAHalo) plan_layer(p, false, 64, &pl, -1);
+#define CCI_WS_SPLIT(A, N)       \
+    if (src == A && sp.bn == N) \
+        return launch_cfg<false, A, N, 1, 1, false, false, true>(p, pl.box, pl.am, stream, sp.log_parts);
+            CCI_WS_SPLIT(kA2d, 64)
+            CCI_WS_SPLIT(kA2d, 128)
+            CCI_WS_SPLIT(kA4d, 64)
+            CCI_WS_SPLIT(kA4d, 128)
+            CCI_WS_SPLIT(kATap, 64)
+            CCI_WS_SPLIT(kATap, 128)
+            CCI_WS_SPLIT(kAGather, 64)
+            CCI_WS_SPLIT(kAGather, 128)
+#undef CCI_WS_SPLIT
+        }
+    }
     // CTA pairs (256-row tiles, B split over the pair) halve each SM's B traffic,
     // which pays on long reductions with 256-wide N tiles; shorter or narrower
     // layers run faster on single CTAs (measured on the ResNet-50 stack)

@@ -76,16 +76,8 @@ struct Smem {
 };
 static_assert(sizeof(Smem) <= 1024, "barriers");
 
-__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
+using ws::ld_shared_f4;
+using ws::st_cluster_v4;
 
 // Y[n][co] in the output type
 __device__ __forceinline__ void store_y(const FwdParams &p, int n, int64_t co, float y)
@@ -425,8 +417,9 @@ cudaError_t launch(const FwdParams &p, cudaStream_t stream)
     const int64_t tiles = (p.Cout + kM - 1) / kM, nks = (p.R + 63) / 64;
     // parts of the reduction: doubled while the SMs hold them all and each keeps
     // kMinStages stages
+    const int64_t sms = ws::sm_count();
     int log_parts = 0;
-    while ((2 << log_parts) <= kMaxParts && (2 << log_parts) * tiles <= ws::sm_count() &&
+    while ((2 << log_parts) <= kMaxParts && tiles <= ws::cluster_slots(log_parts + 1, sms) &&
            nks >= (2 << log_parts) * kMinStages)
         ++log_parts;
     const int parts = 1 << log_parts;
