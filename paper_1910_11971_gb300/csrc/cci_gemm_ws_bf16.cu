@@ -11,12 +11,21 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
     Plan pl;
     plan_layer(p, false, 64, &pl);
     const int asrc = pl.asrc;
-    // products of fewer than 64 reduction indices, and convolutions of fewer than 64
-    // channels, copy only those (stage_k_in)
-    const int kin = stage_k_in(p, false, asrc, false);
-    if (kin < 64 && !build_a_maps(p, pl.box, asrc, false, kin, &pl.am)) return cudaErrorInvalidValue;
     const int64_t m_tiles = m_tiles_of(p, asrc, pl.box);
     const int64_t nks = stages_of(p, asrc);
+    // tiles of at most 4 stages: the output write dominates, two epilogue groups with
+    // two staging buffers each, and the weights of a CTA's N tile resident (two chunks
+    // of 256 channels or four of 128), when every CTA has one tile or the N tiles leave
+    // less than a tenth of the SMs without whole rounds of them; longer ones keep the
+    // shared memory for stages
+    const int sbn = choose_bn(m_tiles, p.Cout, nks <= 2 ? 256 : 128, 1);
+    const int64_t s_ct = (p.Cout + sbn - 1) / sbn, s_slots = resident_slots(s_ct);
+    const bool short_k = nks <= 4 && (asrc == kA2d || asrc == kA4d) &&
+                         (m_tiles * s_ct <= s_slots || 10 * s_slots >= 9 * sm_count());
+    // short products of fewer than 64 reduction indices, and convolutions of fewer than
+    // 64 channels, copy only those (stage_k_in; the kernels' q.kin is chosen alike)
+    const int kin = short_k || asrc == kATap ? stage_k_in(p, false, asrc, false) : 64;
+    if (kin < 64 && !build_a_maps(p, pl.box, asrc, false, kin, &pl.am)) return cudaErrorInvalidValue;
     // few tiles with a long reduction: split over clusters (3x3 layers of halo copies
     // from per-tap boxes)
     {
@@ -59,13 +68,6 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
             return launch_cfg<false, kAHalo, 128, 2>(p, pl.box, pl.am, stream);
         return launch_cfg<false, kAHalo, 64, 1>(p, pl.box, pl.am, stream);  // 64 channels out, or one M tile
     }
-    // tiles of at most 4 stages: the output write dominates, two epilogue groups with
-    // two staging buffers each, and the weights of a CTA's N tile resident (two chunks
-    // of 256 channels or four of 128), when the N tiles leave less than a tenth of the
-    // SMs without whole rounds of them; longer ones keep the shared memory for stages
-    const int sbn = choose_bn(m_tiles, p.Cout, nks <= 2 ? 256 : 128, 1);
-    const bool short_k = nks <= 4 && (asrc == kA2d || asrc == kA4d) &&
-                         10 * resident_slots((p.Cout + sbn - 1) / sbn) >= 9 * sm_count();
     if (short_k) {
 #define CCI_WS_SHORT(A, N) \
     if (asrc == A && sbn == N) return launch_cfg<false, A, N, 1, 2>(p, pl.box, pl.am, stream);

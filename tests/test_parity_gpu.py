@@ -804,10 +804,12 @@ def test_halo_conv3x3_pairs_from_128_channels(dev, B, H, Wi, Cin, Cout):
 
 # short tiles (1 to 4 stages) with resident weights: more tiles than SMs, so every
 # CTA runs several tiles of its N tile; 1, 2, 3 and 5 N tiles (152, 152, 150 and 150
-# CTAs), one that leaves too few whole rounds (100 N tiles: the form without), a
-# ragged last M tile, fewer indices than a chunk and a ragged last chunk
+# CTAs), ones that leave too few whole rounds (100 and 22 N tiles: the form without,
+# whose copies are whole stages also for fewer than 64 indices), one tile per CTA of
+# such a layer, a ragged last M tile, fewer indices than a chunk, a ragged last chunk
 @pytest.mark.parametrize("N,Cin,Cout,G,K", [(20005, 16, 96, 8, 2), (10011, 128, 512, 8, 2), (6500, 72, 520, 8, 2),
-                                            (4200, 256, 640, 16, 4), (20100, 200, 64, 4, 1), (260, 64, 25600, 8, 2)])
+                                            (4200, 256, 640, 16, 4), (20100, 200, 64, 4, 1), (260, 64, 25600, 8, 2),
+                                            (3000, 24, 5600, 8, 2), (150, 16, 1360, 8, 1)])
 def test_short_tiles_resident_weights(dev, N, Cin, Cout, G, K):
     X, W = wl.random_small(N + Cin, "bf16", N, Cin, Cout)
     v, i = cci.pack(W.to(dev), G, K)
