@@ -120,10 +120,10 @@ typedef enum cci_algo {
                                workspace: plane 0 [Cout][R] fp32 hi, then plane 1
                                [Cout][ceil(R/32)*64] bf16 (per 32-wide chunk of r, 32
                                bf16(hi(w)) then 32 bf16(lo(w))).  Cin % 4 == 0, R % 4 == 0.
-                               Needs cci_workspace_size() bytes.  bf16 products of at
-                               most 128 columns and at least 1024 reduction indices
-                               (K <= 8) expand the weights inside the product instead
-                               and leave the workspace as it is */
+                               Needs cci_workspace_size() bytes.  Most bf16 products
+                               of at most 128 columns (K <= 8) expand the weights
+                               inside the product instead and leave the workspace as
+                               it is */
 } cci_algo;
 
 /*

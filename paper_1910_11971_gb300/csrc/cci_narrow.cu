@@ -29,9 +29,11 @@
 //
 // Where the rule lies (device time per pass against decompression and GEMM): 16 x
 // 4096 -> 4096 9.8 us against 16.8, 100 x 2048 -> 1000 7.6 against 9.3, 100 x 1024
-// -> 4096 7.5 against 8.1, 32 x 4096 -> 1024 at G = 32, K = 8 7.1 against 16.6;
-// with 512 reduction indices, which make one part, 128 x 512 -> 2048 took 8.4
-// against 6.4, so those stay there.  At 128 columns 4096 -> 4096 takes 13.1 against
+// -> 4096 7.5 against 8.1, 32 x 4096 -> 1024 at G = 32, K = 8 7.1 against 16.6; up to
+// seven stages in one part it is even with them (25 x 432 -> 992 5.6 against 5.4, 7 x
+// 16 -> 1360 3.6 against 4.4) and saves the second launch, some 3 us of host time a
+// call; eight or nine stages are too few to split and take 8.0 against 6.0 (128 x
+// 512 -> 512), so those stay there.  At 128 columns 4096 -> 4096 takes 13.1 against
 // about 18; more would need smaller stages.
 #include "cci_gemm_ws.cuh"
 
@@ -45,7 +47,8 @@ constexpr int kThreads = 32 * kWarps;
 constexpr int kABytes = kM * 128;
 constexpr int kMaxN = 128;      // columns
 constexpr int kMinStages = 4;   // stages of a part, at least: one for each group
-constexpr int64_t kMinR = 1024;  // reduction indices, at least
+constexpr int kSplitStages = 10;  // stages of a reduction that is split, at least
+constexpr int kWholeStages = 7;   // stages of a reduction that one part takes, at most
 constexpr int kMaxParts = 8;    // portable cluster size
 
 template <int NP>
@@ -420,7 +423,7 @@ cudaError_t launch(const FwdParams &p, cudaStream_t stream)
     const int64_t sms = ws::sm_count();
     int log_parts = 0;
     while ((2 << log_parts) <= kMaxParts && tiles <= ws::cluster_slots(log_parts + 1, sms) &&
-           nks >= (2 << log_parts) * kMinStages)
+           nks >= kSplitStages && nks >= (2 << log_parts) * kMinStages)
         ++log_parts;
     const int parts = 1 << log_parts;
     if (tiles * parts > 0x7fffffff) return cudaErrorInvalidValue;
@@ -460,7 +463,7 @@ bool narrow_ok(const FwdParams &p, int dtype, int64_t N)
                     (p.K == 1 || p.K == 2 || p.K == 4 || p.K == 8) && 2 * p.K <= p.G;
     auto at16 = [](const void *q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };
     return dtype == CCI_BF16 && !p.is_conv && N > 0 && N <= narrow::kMaxN && gk && p.Cin == p.R && p.R % 8 == 0 &&
-           p.R >= narrow::kMinR && p.R < (int64_t(1) << 31) && p.Cout < (int64_t(1) << 31) && at16(p.X) && at16(p.Y) && at16(p.values) &&
+           ((p.R + 63) / 64 <= narrow::kWholeStages || (p.R + 63) / 64 >= narrow::kSplitStages) && p.R < (int64_t(1) << 31) && p.Cout < (int64_t(1) << 31) && at16(p.X) && at16(p.Y) && at16(p.values) &&
            at16(p.idx);
 }
 

@@ -1,6 +1,5 @@
-"""Products of at most 128 columns with 1024 reduction indices or more: one launch
-that expands the packed weights as it multiplies, the reduction split over a
-cluster.  Every output against the fp64 oracle at the tolerance of all products
+"""Products of at most 128 columns: one launch that expands the packed weights as it
+multiplies, the reduction of ten stages of 64 indices or more split over a cluster.  Every output against the fp64 oracle at the tolerance of all products
 (1e-5 of sum |w||x|), with the output stage's bf16 rounding where it applies."""
 import numpy as np
 import pytest
@@ -20,10 +19,11 @@ def dev():
     return torch.device("cuda:0")
 
 
-# columns at the edges of the MMA's N (16, 32, 64, 128); reductions at the edge of
-# the rule, with a ragged last stage, and deep enough for 2, 4 and 8 parts of
-# unequal length; channels below, at and past a tile of 128; every K, G 4 to 32
-CASES = [(1, 1024, 64, 4, 1), (16, 1032, 72, 8, 2), (17, 1536, 1000, 8, 4), (32, 2048, 128, 16, 8), (33, 1096, 136, 4, 2),
+# columns at the edges of the MMA's N (16, 32, 64, 128); reductions of one chunk and
+# less, at both edges of the rule (7 stages, 10), with a ragged last stage, and deep
+# enough for 2, 4 and 8 parts of unequal length; channels below, at and past a tile of 128; every K, G 4 to 32
+CASES = [(1, 8, 8, 8, 2), (7, 16, 1360, 8, 1), (33, 72, 24, 4, 2), (128, 448, 224, 32, 8), (100, 584, 136, 8, 4),
+         (16, 640, 96, 16, 8), (1, 1024, 64, 4, 1), (16, 1032, 72, 8, 2), (17, 1536, 1000, 8, 4), (32, 2048, 128, 16, 8), (33, 1096, 136, 4, 2),
          (64, 4096, 256, 32, 4), (65, 2056, 160, 32, 1), (100, 2048, 1000, 8, 1), (127, 1160, 96, 16, 2),
          (128, 3000, 264, 8, 2), (5, 1024, 20, 4, 1), (128, 4096, 4096, 16, 4)]
 
