@@ -1589,7 +1589,50 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 uint32_t hsph = 0u, hph = 0u;
                 const uint64_t wq_units = static_cast<uint64_t>(box.QB + p.KW - 1) * 8u;
                 const uint64_t hunits = hbytes >> 4, sunits = C::kStage >> 4;
-                const bool res = box.resident != 0;
+                if constexpr (CG == 1) {  // (pairs never keep their weights resident: slower, below)
+                    if (box.resident) {
+                        // One chunk, nine weight tiles.  The next tile's accumulator and halo are
+                        // waited for before the last kernel row of this one is issued, so that
+                        // the waits' latency passes while the tensor core still has work: with the
+                        // waits between the tiles it idled 680 of 2660 cycles a tile (64 -> 64 at
+                        // 56 x 56, 128 images: 40.2 us a pass, 30.9 so).  (In the loop below, whose
+                        // halos are re-copied with every chunk and come late, the same order
+                        // delays the last row: 128 -> 128 at 28 x 28, 128 images 24.3 -> 25.3.)  (CTA pairs, which read 5 KB of operands per SM and
+                        // MMA instead of 6, took 47.8 us.)
+                        auto ready = [&](int tt, int h, uint32_t parity) {
+                            if (tt >= 2 && !tc::mbar_wait(&S->tmem_empty[tt & 1], ((tt / 2) - 1) & 1, abort, p.status))
+                                return false;
+                            return tc::mbar_wait(&S->hfull[h], parity, abort, p.status);
+                        };
+                        if (u0 < n_tiles) ok = ready(0, 0, 0u);
+                        for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                            const uint32_t d = tmem + static_cast<uint32_t>((t & 1) * kN);
+                            const uint64_t hdesc = hdesc0 + static_cast<uint64_t>(hb) * hunits;
+                            const int nhb = hb + 1 == box.nh ? 0 : hb + 1;
+                            const uint32_t nph = nhb == 0 ? hph ^ 1u : hph;
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                            for (int kh = 0; kh < 3; ++kh) {
+                                if (t == 0) {  // the row's weights land once, for the first tile
+                                    for (int kw = 0; kw < 3 && ok; ++kw)
+                                        ok = tc::mbar_wait(&S->full[3 * kh + kw], 0u, abort, p.status);
+                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                                }
+                                if (kh == 2 && ok && u + ustep < n_tiles) ok = ready(t + 1, nhb, nph);
+                                if (!ok) break;
+                                row3_f16<C::kIdesc, (C::kStage >> 4)>(
+                                    d, hdesc + static_cast<uint64_t>(kh) * wq_units,
+                                    bdesc0 + static_cast<uint64_t>(3 * kh) * sunits, kh != 0 ? 1u : 0u);
+                            }
+                            if (!ok) break;
+                            commit(&S->hempty[hb]);
+                            commit(&S->tmem_full[t & 1]);
+                            hb = nhb;
+                            hph = nph;
+                        }
+                        ok = false;  // the loop below is not entered
+                    }
+                }
                 for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
@@ -1597,7 +1640,6 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t d = tmem + static_cast<uint32_t>(acc * kN);
-                    if (res) hs = 0;
                     for (int c = 0; c < hchunks && ok; ++c) {
                         ok = tc::mbar_wait(&S->hfull[hb], hph, abort, p.status);
                         if (!ok) break;
@@ -1605,32 +1647,19 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                         const uint64_t hdesc = hdesc0 + static_cast<uint64_t>(hb) * hunits;
                         for (int kh = 0; kh < 3 && ok; ++kh) {
                             const uint64_t arow = hdesc + static_cast<uint64_t>(kh) * wq_units;
-                            if (res) {
-                                if (t == 0) {  // the row's weights land once, for the first tile
-                                    for (int kw = 0; kw < 3 && ok; ++kw)
-                                        ok = tc::mbar_wait(&S->full[hs + kw], 0u, abort, p.status);
-                                    if (!ok) break;
-                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                }
-                                if constexpr (CG == 1)  // (pairs never keep their weights resident)
-                                    row3_f16<C::kIdesc, (C::kStage >> 4)>(
-                                        d, arow, bdesc0 + static_cast<uint64_t>(hs) * sunits, (c | kh) != 0 ? 1u : 0u);
-                                hs += 3;
-                            } else {
-                                for (int kw = 0; kw < 3 && ok; ++kw) {
-                                    ok = tc::mbar_wait(&S->full[hs], hsph, abort, p.status);
-                                    if (!ok) break;
-                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                    const uint64_t bd = bdesc0 + static_cast<uint64_t>(hs) * sunits;
-                                    const uint32_t accf = (c | kh | kw) != 0 ? 1u : 0u;
-                                    if constexpr (CG == 2)  // the pair's MMAs; the stage released in both CTAs
-                                        stage_f16_pair<C::kIdesc>(d, arow + kw * 8u, bd, accf, empty0 + 8u * hs);
-                                    else
-                                        stage_f16<C::kIdesc>(d, arow + kw * 8u, bd, accf, 1u, empty0 + 8u * hs);
-                                    if (++hs == kStages) {
-                                        hs = 0;
-                                        hsph ^= 1u;
-                                    }
+                            for (int kw = 0; kw < 3 && ok; ++kw) {
+                                ok = tc::mbar_wait(&S->full[hs], hsph, abort, p.status);
+                                if (!ok) break;
+                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                                const uint64_t bd = bdesc0 + static_cast<uint64_t>(hs) * sunits;
+                                const uint32_t accf = (c | kh | kw) != 0 ? 1u : 0u;
+                                if constexpr (CG == 2)  // the pair's MMAs; the stage released in both CTAs
+                                    stage_f16_pair<C::kIdesc>(d, arow + kw * 8u, bd, accf, empty0 + 8u * hs);
+                                else
+                                    stage_f16<C::kIdesc>(d, arow + kw * 8u, bd, accf, 1u, empty0 + 8u * hs);
+                                if (++hs == kStages) {
+                                    hs = 0;
+                                    hsph ^= 1u;
                                 }
                             }
                         }
