@@ -49,23 +49,34 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
 #undef CCI_WS_SPLIT
         }
     }
-    // CTA pairs (256-row tiles, B split over the pair) halve each SM's B traffic,
-    // which pays on long reductions with 256-wide N tiles; shorter or narrower
-    // layers run faster on single CTAs (measured on the ResNet-50 stack)
-    const bool pair = (asrc == kA2d || is_box(asrc)) && nks >= 16 && choose_bn(m_tiles, p.Cout, 256, 2) == 256;
+    // CTA pairs (256-row tiles, B split over the pair) halve each SM's B traffic.  With
+    // 256-wide N tiles that pays on long reductions of more than one round of pairs:
+    // a single round starts and ends faster on single CTAs (512 -> 512 at 7 x 7, 128
+    // images 28.0 us paired, 26.5 single)
+    const int64_t pairs = sm_count() / 2;
+    auto pair_units = [&](int64_t mt, int bn) { return (mt + 1) / 2 * ((p.Cout + bn - 1) / bn); };
+    const bool pair = (asrc == kA2d || is_box(asrc)) && nks >= 16 && choose_bn(m_tiles, p.Cout, 256, 2) == 256 &&
+                      pair_units(m_tiles, 256) > pairs;
     if (pair) {
         if (asrc == kA2d) return launch_cfg<false, kA2d, 256, 2>(p, pl.box, pl.am, stream);
         if (asrc == kATap) return launch_cfg<false, kATap, 256, 2>(p, pl.box, pl.am, stream);
         return launch_cfg<false, kA4d, 256, 2>(p, pl.box, pl.am, stream);
     }
     if (asrc == kAHalo) {
-        // 3x3 convolutions from halo copies (tiles of nine stages per chunk at least)
-        // CTA pairs (256-row tiles, each CTA copying its own halo and half of every
-        // weight tile) for every layer but the 64 -> 64 ones: a pair's stage brings 8 KB
-        // of weights per SM for 256 cycles of MMAs.  With the issue loops lean, 128-wide
-        // tiles beat 256-wide ones (256 channels at 14 x 14, 128 images 27.5 -> 26.7 us)
-        if (p.Cin >= 128 && p.Cout > 64 && m_tiles > 1)
+        // 3x3 convolutions from halo copies: pairs with 128-wide N tiles (each CTA copying
+        // its own halo and half of every weight tile, 8 KB a stage for 256 cycles of
+        // MMAs) for every layer but those of 64 channels out.  Images narrower than the
+        // tile leave rows of a halo tile unused; where pairs of per-tap boxes, which span
+        // images, take fewer rounds, those (256 -> 256 at 14 x 14, 128 images 25.7 us in
+        // four rounds of halos, 24.4 in three of boxes)
+        if (p.Cin >= 128 && p.Cout > 64 && m_tiles > 1) {
+            const int64_t m4 = m_tiles_of(p, kA4d, pl.a4d);
+            if ((pair_units(m4, 128) + pairs - 1) / pairs < (pair_units(m_tiles, 128) + pairs - 1) / pairs) {
+                plan_layer(p, false, 64, &pl, -1);
+                return launch_cfg<false, kA4d, 128, 2>(p, pl.box, pl.am, stream);
+            }
             return launch_cfg<false, kAHalo, 128, 2>(p, pl.box, pl.am, stream);
+        }
         return launch_cfg<false, kAHalo, 64, 1>(p, pl.box, pl.am, stream);  // 64 channels out, or one M tile
     }
     if (short_k) {
@@ -80,6 +91,11 @@ cudaError_t launch_gemm_ws_bf16(const FwdParams &p, cudaStream_t stream)
 #undef CCI_WS_SHORT
     }
     const int bn = choose_bn(m_tiles, p.Cout, 256, 1);
+    // per-tap boxes of long reductions, 128-wide N tiles, three rounds of pairs or more
+    // (256 -> 256, stride 2 at 28 x 28, 128 images: 29.2 us single, 26.5 paired; at 32
+    // images, one round, 12.0 and 12.7)
+    if (asrc == kA4d && nks >= 16 && bn == 128 && pair_units(m_tiles, 128) > 2 * pairs)
+        return launch_cfg<false, kA4d, 128, 2>(p, pl.box, pl.am, stream);
 #define CCI_WS_CASE(A, N) \
     if (asrc == A && bn == N) return launch_cfg<false, A, N, 1>(p, pl.box, pl.am, stream);
     CCI_WS_CASE(kA2d, 64)

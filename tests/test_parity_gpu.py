@@ -879,7 +879,8 @@ def test_pair_tiles_product(dev, N, Cin, Cout, G, K):
     assert_within_tol(f64(Y[torch.from_numpy(rows).to(dev)]), Yo, S, f"pair product {N}x{Cin}->{Cout}")
 
 
-@pytest.mark.parametrize("B,H,Cin,Cout,stride", [(63, 14, 128, 256, 1), (64, 28, 128, 256, 2)])
+@pytest.mark.parametrize("B,H,Cin,Cout,stride", [(63, 14, 128, 256, 1), (64, 28, 128, 256, 2), (301, 14, 128, 128, 1),
+                                                 (401, 14, 128, 200, 2)])
 def test_pair_tiles_conv(dev, B, H, Cin, Cout, stride):
     G, K = 8, 2
     g = torch.Generator().manual_seed(B * 31 + H)
