@@ -159,6 +159,14 @@ struct Cfg {
     static constexpr bool kATma = !TF32 && ASRC != kAGather;  // A copied by TMA into its plane
     static constexpr bool kTapChunks = ASRC == kATap;
     static_assert(!kTapChunks || (!TF32 && !PK && EPI == 1 && !MC), "ragged channels: bf16, workspace weights");
+    // kPrefetch: the activations of a CTA's next unit are prefetched into L2 while this
+    // one's are copied.  fp32 products read them from HBM through a ring of four stages
+    // that also carries the weights: a copy took 6000 cycles, and the MMAs waited for
+    // 360 of 910 cycles a stage (256 -> 1024 on 100352 columns: 166 -> 143 us).  Up to
+    // 16 stages a tile (the units ahead stay a fraction of L2) and from four N tiles on,
+    // whose units share the prefetches out: with one, a CTA prefetches as much as it
+    // copies (256 -> 64: 26.3 -> 27.3 us).
+    static constexpr bool kPrefetch = TF32 && ASRC == kA2d && !SK;
     static constexpr bool kHalo = ASRC == kAHalo;  // A: per-chunk halo buffers, stages hold B only
     static_assert(!kHalo || (!TF32 && (CG == 1 || !PK)), "halo copies: bf16 tiles (pairs: workspace weights)");
     // raw fp32 A by TMA; the producers split it into its two planes and write both to
@@ -1062,7 +1070,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
             step(ks + kbase);
             // resident weights (halo copies): only the first tile's stages are copied
             const int u_end = C::kHalo && box.resident ? (u0 + 1 < n_tiles ? u0 + 1 : n_tiles) : n_tiles;
-            int u = u0, mt = 0, ct = 0;
+            int u = u0, mt = 0, ct = 0, pmt = 0, pct = 0;
+            bool ahead = false;
             BoxIdx bi{0, 0, 0};
             bool fresh = true;  // the tile's coordinates are to be formed
             // kA, kB: the operands copied; both by the loop that runs to the end, and
@@ -1080,6 +1089,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 if (fresh) {
                     split_unit(u, mt, ct);
                     if constexpr (is_box(ASRC)) bi = box_of(mt, box);
+                    if constexpr (C::kPrefetch) {
+                        split_unit(u + ustep, pmt, pct);
+                        ahead = u + ustep < u_end && nks <= 16 && box.byN.d >= 4u;
+                    }
                     fresh = false;
                 }
                 if (kCopyA && !tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
@@ -1130,6 +1143,13 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                             tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
                         else
                             tc::tma_load_2d(st, &tmA.m[0], (ks + kbase) * kKS, mt * kM, abar);
+                        if constexpr (C::kPrefetch) {
+                            // the units of an M tile, which run at the same time, share its stages
+                            // out: ks modulo their number
+                            const int n = static_cast<int>(box.byN.d);
+                            if (ahead && ks - static_cast<int>(box.byN.quot(static_cast<uint32_t>(ks))) * n == pct)
+                                tc::tma_prefetch_2d(&tmA.m[0], ks * kKS, pmt * kM);
+                        }
                     } else if constexpr (is_box(ASRC) && kCopyA) {
                         // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
                         const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
