@@ -33,8 +33,6 @@ struct FwdParams {
     const float *bias;   // nullptr: none
     int relu;
     int out_bf16;        // Y holds bf16 (round to nearest even) instead of fp32
-    int a_early;         // workspace kernels: launched behind the decompression, whose blocks
-                         // signalled after X's producer had completed: X may be read at once
     int kin;             // workspace kernels: reduction indices copied per stage (bf16
                          // products with R < 64: R rounded up to 16; else the whole stage)
 };

@@ -195,9 +195,7 @@ cudaError_t launch_dense_tc_ws(const FwdParams &p, int dtype, int G, int K, cuda
         const cudaError_t e = dtype == CCI_F32 ? dc::launch<uint32_t, g, k, true>(p, stream) \
                                                : dc::launch<uint16_t, g, k, false>(p, stream); \
         if (e != cudaSuccess) return e;                                                     \
-        FwdParams q = p;                                                                    \
-        q.a_early = 1;                                                                      \
-        return launch_gemm_ws(q, dtype, stream);                                            \
+        return launch_gemm_ws(p, dtype, stream);                                            \
     }
     CCI_TC_CASE(4, 1) CCI_TC_CASE(4, 2)
     CCI_TC_CASE(8, 1) CCI_TC_CASE(8, 2) CCI_TC_CASE(8, 4)

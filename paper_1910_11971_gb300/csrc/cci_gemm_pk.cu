@@ -26,7 +26,7 @@ bool gemm_pk_supported(const FwdParams &p)
 {
     if (!gemm_pk_shape_ok(p)) return false;
     ws::Plan pl;
-    ws::plan_layer(p, false, 64, &pl, 256, true);
+    ws::plan_layer(p, false, 64, &pl);
     return pl.asrc != ws::kAGather;
 }
 
@@ -35,7 +35,7 @@ cudaError_t launch_gemm_pk(const FwdParams &p, cudaStream_t stream)
     using namespace ws;
     if (!gemm_pk_shape_ok(p)) return cudaErrorNotSupported;
     Plan pl;
-    plan_layer(p, false, 64, &pl, 256, true);
+    plan_layer(p, false, 64, &pl);
     const int asrc = pl.asrc;
     if (asrc == kAGather) return cudaErrorNotSupported;
     const int64_t m_tiles = m_tiles_of(p, asrc, pl.box);

@@ -16,17 +16,10 @@
 //                plane 1 over [Cout][ceil(R / 32) * 64] bf16);
 //   activations  one of (the template's ASRC):
 //     kA2d      products: TMA over X[N][Cin];
-//     kA4d      convolutions of strides up to 2: TMA over X[B][H][W][Cin] with a
-//               box of QB x PB x BB output pixels (QB*PB*BB <= 128 rows), shifted
-//               by the tap (kh, kw); the zero padding is the copy's out-of-range
-//               fill.  A stage is a chunk of a tap's channels; Cin is a multiple of
-//               the stage depth;
-//     kATap     the same for the other channel counts, in bf16: a tap's last chunk
-//               is filled with zeros past Cin in both operands (the weights are
-//               copied as [co][tap][ci] boxes) and takes the MMAs of the channels
-//               it has.  Counting them costs the issuing thread some 45 cycles a
-//               stage, so whole stages keep their own form (3x3, 320 -> 32 at 8 x 8:
-//               10.1 us against 11.0 counted);
+//     kA4d      stride-1 convolutions with Cin a multiple of the stage depth:
+//               TMA over X[B][H][W][Cin] with a box of QB x PB x BB output
+//               pixels (QB*PB*BB <= 128 rows), shifted by the tap (kh, kw); the
+//               zero padding is the copy's out-of-range fill;
 //     kAHalo    bf16 3x3 convolutions with unit stride and padding 1: per tile
 //               and 64-channel chunk one TMA copy of the input halo, rows
 //               (p, q) of PB input rows + 2 by Q + 2 columns (the padding is the
@@ -56,17 +49,19 @@
 //               is free stores the rows into its swizzled B tile.
 // Output: Y (fp32, or bf16 with the fused epilogue's bias and ReLU) written by
 // TMA stores from swizzled staging buffers of [128 rows][128 bytes] (two per
-// epilogue group), 2-D over Y[N][Cout] or, for kA4d, kATap and kAHalo, 4-D over Y[B][P][Q][Cout] with the tile's
+// epilogue group, four in the two-group form with N tiles up to 128), 2-D over
+// Y[N][Cout] or, for kA4d and kAHalo, 4-D over Y[B][P][Q][Cout] with the tile's
 // pixel box.
 // Roles: warps 0-3 epilogue (TMEM lanes), warps 4-7 producers of the activation
 // planes that are not copied by TMA (PK: of the weight tiles, with warps
 // 9 + kIssuers .. + 3 as the second producer group), warp 8 allocates TMEM and
 // issues the MMAs, warps 9 .. 8 + kIssuers issue the TMA copies as soon as a
 // stage is free (so copy latency overlaps the producers' work), stage by stage in
-// turn: what a box costs its issuer is the length of the issue loop, whatever the
-// box's size, so up to six warps issue (one per stage in flight; PK: three, one
-// activation box per stage).  Every mbarrier wait is bounded (CCI_ERR_TIMEOUT,
-// abort flag, drain, TMEM freed).
+// turn: the copies one thread issues are processed one box after another
+// (measured on GB300: about 0.5 us per box of 16-64 KB from one issuer; copy
+// throughput grows with the number of issuing warps), so up to six warps issue
+// (one per stage in flight; PK: three, one activation box per stage).  Every
+// mbarrier wait is bounded (CCI_ERR_TIMEOUT, abort flag, drain, TMEM freed).
 #pragma once
 
 #include <cuda.h>
@@ -80,32 +75,12 @@
 namespace cci {
 namespace ws {
 
-enum ASrc { kA2d = 0, kA4d = 1, kAGather = 2, kAHalo = 3, kATap = 4 };
-
-// activations copied as 4-D boxes of output pixels
-__host__ __device__ constexpr bool is_box(int asrc) { return asrc == kA4d || asrc == kATap; }
+enum ASrc { kA2d = 0, kA4d = 1, kAGather = 2, kAHalo = 3 };
 
 // output-pixel box of one M tile of a convolution whose activations are copied
 // by 4-D TMA: rows m = (bi*PB + pi)*QB + qi of the tile are the pixels
 // (b0 + bi, p0 + pi, q0 + qi); rows >= QB*PB*BB are unused.  Halo copies: QB = Q,
 // BB = 1, rows m = pi*(Q + 2) + qi (qi >= Q unused), rows = PB*(Q + 2)
-// division of a tile index (below 2^31) by a size that is fixed for the launch, as
-// a multiply and a shift (Granlund and Montgomery): the quotient of n is
-// (umulhi(n, mul) + n) >> shift with shift = ceil(log2 d) and
-// mul = floor(2^32 (2^shift - d) / d) + 1.  The copy issuers and the epilogue form
-// tile coordinates once per tile: a run-time 64-bit division there is a serial
-// chain of a hundred instructions in the one thread that keeps the copies going.
-struct TileDiv {
-    uint32_t d = 1, mul = 1, shift = 0;
-    TileDiv() = default;
-    explicit TileDiv(int64_t div) : d(static_cast<uint32_t>(div))
-    {
-        while ((uint64_t(1) << shift) < d) ++shift;
-        mul = static_cast<uint32_t>((((uint64_t(1) << shift) - d) << 32) / d + 1);
-    }
-    __device__ __forceinline__ uint32_t quot(uint32_t n) const { return (__umulhi(n, mul) + n) >> shift; }
-};
-
 struct ConvBox {
     int QB, PB, BB;  // box extent along q, p and the batch
     int nQ, nP;      // boxes along q and p (the batch index is the rest)
@@ -116,9 +91,6 @@ struct ConvBox {
     int resident;    // halo copies: the layer's whole weight matrix stays in the stages
                      // (one N tile, every stage of a tile a stage of the ring): the
                      // weights are copied for the CTA's first tile only
-    TileDiv byQ, byP, byN;  // division by nQ, by nP and by the N tiles (set at the launch)
-    int log_split = 0;      // SK: a tile's reduction is split over a cluster of 1 << log_split CTAs
-    TileDiv byC, byKW;      // gather: division of a reduction index by Cin, of a tap by KW
 };
 
 // activation tensor maps: [0] for products (2-D over X[N][Cin]); for a
@@ -134,13 +106,7 @@ struct AMaps {
 // EPI = 2: a second epilogue group (warps 4-7, idle when bf16 activations are
 // copied by TMA) and two staging buffers per group, for layers whose tiles have
 // few stages (the output write dominates); EPI = 1: one group, more stages
-// SK: few tiles with long reductions.  A tile is a cluster of 2, 4 or 8 CTAs, each
-// of which multiplies its share of the stages (one tile per cluster, so the grid is
-// the whole work); then each owns 1 / parts of the tile's columns: every CTA stores
-// its sums of them into the owner's shared memory (straight from tensor memory, 512
-// bytes a warp), and after one cluster barrier the owner adds them in rank order and
-// writes its columns with plain stores.
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false, bool SK = false>
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
 struct Cfg {
     static constexpr int kM = 128, kN = BN;
     static_assert(CG == 1 || (CG == 2 && !TF32 && ASRC != kAGather), "pair mode: bf16 with TMA activations");
@@ -157,16 +123,6 @@ struct Cfg {
     static constexpr bool kPairUnits = CG == 2 || MC;  // units of two M tiles over a cluster of two
     static constexpr int kKS = TF32 ? 32 : 64;  // r per stage: one 128-byte row
     static constexpr bool kATma = !TF32 && ASRC != kAGather;  // A copied by TMA into its plane
-    static constexpr bool kTapChunks = ASRC == kATap;
-    static_assert(!kTapChunks || (!TF32 && !PK && EPI == 1 && !MC), "ragged channels: bf16, workspace weights");
-    // kPrefetch: the activations of a CTA's next unit are prefetched into L2 while this
-    // one's are copied.  fp32 products read them from HBM through a ring of four stages
-    // that also carries the weights: a copy took 6000 cycles, and the MMAs waited for
-    // 360 of 910 cycles a stage (256 -> 1024 on 100352 columns: 166 -> 143 us).  Up to
-    // 16 stages a tile (the units ahead stay a fraction of L2) and from four N tiles on,
-    // whose units share the prefetches out: with one, a CTA prefetches as much as it
-    // copies (256 -> 64: 26.3 -> 27.3 us).
-    static constexpr bool kPrefetch = TF32 && ASRC == kA2d && !SK;
     static constexpr bool kHalo = ASRC == kAHalo;  // A: per-chunk halo buffers, stages hold B only
     static_assert(!kHalo || (!TF32 && (CG == 1 || !PK)), "halo copies: bf16 tiles (pairs: workspace weights)");
     // raw fp32 A by TMA; the producers split it into its two planes and write both to
@@ -176,17 +132,7 @@ struct Cfg {
     static constexpr int kAPlane = kM * 128;                    // bytes: 128-byte rows
     static constexpr int kBPlane = kBRows * 128;
     static constexpr int kBOff = kHalo ? 0 : kAPlanes * kAPlane;  // B planes within a stage
-    // kRes: a CTA keeps the weights of its N tile, up to kResB chunks of 64 indices, in
-    // shared memory for all its tiles (the launch deals every CTA tiles of one N tile);
-    // the stages hold activations only.  Re-copied per tile, the few lines of a short
-    // tile's weights were read by all SMs at once, which bounded these layers: 16 ->
-    // 64 channels over 1.6 M pixels took longer (92 us) than 32 -> 64 (66 us), whose
-    // weights are twice as many lines.
-    static constexpr bool kRes = EPI == 2;
-    static_assert(!kRes || (kATma && CG == 1 && !PK && !MC && !kTapChunks && !kHalo), "resident weights: short bf16 tiles");
-    static constexpr int kResB = kN > 128 ? 2 : 4;
-    static constexpr int kResBytes = kRes ? kResB * kBPlane : 0;
-    static constexpr int kStage = kRes ? kAPlane : kBOff + kBPlanes * kBPlane;
+    static constexpr int kStage = kBOff + kBPlanes * kBPlane;
     static_assert(kStage % 1024 == 0, "stages must keep the 1024-byte swizzle alignment");
     // halo copies: fewer weight stages, the rest of shared memory for a ring of
     // halo buffers whose size and count the host sets per layer (ConvBox)
@@ -195,25 +141,21 @@ struct Cfg {
     static constexpr int kHaloStages = kBPlane <= 8192 ? 9 : (kBPlane <= 16384 ? 4 : 3);
     static constexpr int kYBuf = kM * 128;  // one output staging buffer: [128 rows][32 fp32]
     // epilogue groups: warps 0-3, and warps 4-7 too when they have no producer work
-    // (TMA-copied bf16 activations), two staging buffers each.  The rest of shared
-    // memory is stages: with the biases staged, four buffers a group instead (and two
-    // stages fewer) took 9.3 us against 8.3 for 256 -> 1024 at 14 x 14, 32 images, and
-    // 13.9 against 12.9 for 256 -> 64 at 56 x 56.
+    // (TMA-copied bf16 activations); two staging buffers per group, four in the
+    // two-group form with N tiles up to 128 (short tiles, bound by the output
+    // write: more stores in flight, three or four stages are enough)
     static constexpr int kEG = (kATma && EPI == 2) ? 2 : 1;
-    static constexpr int kYPerGroup = 2;
-    static_assert(!SK || (CG == 1 && EPI == 1 && !PK && !MC && ASRC != kAHalo && BN <= 128), "split tiles");
-    // SK: the exchanged sums (parts x [BN / parts / 4][128 rows][4]) instead
-    static constexpr int kYBufs = SK ? BN * 512 / kYBuf : kYPerGroup * kEG;
+    static constexpr int kYPerGroup = (kEG == 2 && BN <= 128) ? 4 : 2;
+    static constexpr int kYBufs = kYPerGroup * kEG;
     static_assert(EPI == 1 || EPI == 2, "epilogue groups");
-    static constexpr int kBudget = static_cast<int>(kMaxSmemPerBlock) - 1024 - kYBufs * kYBuf - kResBytes - kEG * kN * 4 - 1024;
+    static constexpr int kBudget = static_cast<int>(kMaxSmemPerBlock) - 1024 - kYBufs * kYBuf - 1024;
     static constexpr int kStagesFit = (kBudget / kStage) < tc::kMaxStages ? (kBudget / kStage) : tc::kMaxStages;
     static constexpr int kStages = kHalo ? kHaloStages : kStagesFit;
     // accumulators: 2 x kN columns; kARaw adds per stage the A planes (32 + 32 columns)
     static constexpr int kAColBase = 2 * kN;
     static constexpr int kTmemCols = kARaw ? 512 : 2 * kN;
-    static constexpr int kBiasBytes = kN * 4;  // biases of one N tile, per epilogue group
-    static constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * kStage + kResBytes + kYBufs * kYBuf +
-                                    kEG * kBiasBytes + sizeof(tc::Smem) + 64;  // + halo ring
+    static constexpr size_t kSmem =
+        1024 + static_cast<size_t>(kStages) * kStage + kYBufs * kYBuf + sizeof(tc::Smem) + 64;  // + halo ring
     static constexpr uint32_t kBBytes = kBPlanes * kBPlane;
     static constexpr uint32_t kIdesc = (1u << 4)                                           // D f32
                                        | (TF32 ? (2u << 7) | (2u << 10) : (1u << 7) | (1u << 10))  // tf32 / bf16
@@ -226,9 +168,9 @@ struct Cfg {
     static_assert(kStages >= 3, "too few pipeline stages");
     static_assert(kTmemCols == 128 || kTmemCols == 256 || kTmemCols == 512, "TMEM allocation not a power of 2");
     static_assert(!kARaw || kAColBase + kStages * 64 <= 512, "A stages do not fit in tensor memory");
-    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: a box
-    // costs its issuer the same loop whatever its size, so several issuers keep
-    // more bytes moving.  kIssuers <= kStages keeps every empty-barrier wait
+    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: one
+    // thread's copies are processed one box at a time, so several issuers keep
+    // more boxes moving.  kIssuers <= kStages keeps every empty-barrier wait
     // within one phase of the barrier (no parity aliasing).
     // (kAHalo: one more warp, which copies the halos)
     // PK: three issuers (one activation box per stage) and a second group of four
@@ -419,27 +361,10 @@ __device__ __forceinline__ void row3_f16(uint32_t d, uint64_t adesc, uint64_t bd
 // from one block executed by the issuing thread alone.  The separate per-MMA
 // form took ~360 cycles per stage to issue on GB300 (clock stamps), against 512
 // cycles of MMA work: the issue, not the tensor pipe, set the stage period.
-// kCounted: only the first n16 (1-4) MMAs, as stage_f16
-template <uint32_t kIdesc, bool kCounted = false>
+template <uint32_t kIdesc>
 __device__ __forceinline__ void stage_f16_pair(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t acc0,
-                                               uint32_t bar, uint32_t n16 = 4)
+                                               uint32_t bar)
 {
-    if constexpr (kCounted)
-        asm volatile(
-            "{\n.reg .pred pa, p1, p2, p3, pt;\n.reg .b64 ad, bd;\n"
-            "setp.ne.b32 pa, %3, 0;\nsetp.eq.b32 pt, 0, 0;\n"
-            "setp.gt.u32 p1, %7, 1;\nsetp.gt.u32 p2, %7, 2;\nsetp.gt.u32 p3, %7, 3;\n"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %4, pa;\n"
-            "add.s64 ad, %1, 2;\nadd.s64 bd, %2, 2;\n"
-            "@p1 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
-            "add.s64 ad, %1, 4;\nadd.s64 bd, %2, 4;\n"
-            "@p2 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
-            "add.s64 ad, %1, 6;\nadd.s64 bd, %2, 6;\n"
-            "@p3 tcgen05.mma.cta_group::2.kind::f16 [%0], ad, bd, %4, pt;\n"
-            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%5], %6;\n}\n" ::"r"(d),
-            "l"(adesc), "l"(bdesc), "r"(acc0), "n"(kIdesc), "r"(bar), "h"(static_cast<uint16_t>(3)), "r"(n16)
-            : "memory");
-    else
     asm volatile(
         "{\n.reg .pred pa, pt;\n.reg .b64 ad, bd;\n"
         "setp.ne.b32 pa, %3, 0;\nsetp.eq.b32 pt, 0, 0;\n"
@@ -537,15 +462,6 @@ __device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const void *tmap, i
         : "memory");
 }
 
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void *tmap, int c0, int c1, int c2, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
-        "{%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
-        : "memory");
-}
-
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const void *tmap, int c0, int c1, int c2, int c3,
                                                  uint32_t bar)
 {
@@ -557,29 +473,31 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const void *tmap,
 }
 
 // Output epilogue of a CNN layer, on 32 consecutive fp32 accumulator values of
-// one row: y + bias (when p.bias; the 32 biases at shared-memory address `bias`,
-// zero past the last channel), then max(y, 0) (when p.relu; NaN gives 0).  The
-// biases of a tile's channels are staged in shared memory once per N tile: read
-// from global memory here they were eight dependent loads per 32 columns in
-// front of every chunk (clock stamps on GB300: 850-1600 cycles for a chunk of 64
-// bf16 columns with bias and ReLU, against 2 x 205 without).
-__device__ __forceinline__ void epilogue_math(uint32_t (&v)[32], const FwdParams &p, uint32_t bias)
+// one row at output channels col0..col0+31: y + bias[co] (when p.bias), then
+// max(y, 0) (when p.relu).  Channels >= Cout get no bias (their columns are
+// clipped by the store).
+__device__ __forceinline__ void epilogue_math(uint32_t (&v)[32], const FwdParams &p, int col0)
 {
     if (p.bias) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            float b[4];
-            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
-                         : "r"(bias + 16 * q)
-                         : "memory");
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[4 * q + e] = __float_as_uint(__uint_as_float(v[4 * q + e]) + b[e]);
+            const int col = col0 + 4 * q;
+            // Cout is a multiple of 4 and the bias 16-byte aligned: a float4 that
+            // starts inside the row of biases lies wholly inside it
+            const float4 b = col < p.Cout ? __ldg(reinterpret_cast<const float4 *>(p.bias + col))
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[4 * q] = __float_as_uint(__uint_as_float(v[4 * q]) + b.x);
+            v[4 * q + 1] = __float_as_uint(__uint_as_float(v[4 * q + 1]) + b.y);
+            v[4 * q + 2] = __float_as_uint(__uint_as_float(v[4 * q + 2]) + b.z);
+            v[4 * q + 3] = __float_as_uint(__uint_as_float(v[4 * q + 3]) + b.w);
         }
     }
     if (p.relu) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(fmaxf(__uint_as_float(v[j]), 0.f));
+        for (int j = 0; j < 32; ++j) {
+            const float x = __uint_as_float(v[j]);
+            v[j] = __float_as_uint(x > 0.f ? x : 0.f);
+        }
     }
 }
 
@@ -829,100 +747,56 @@ __device__ __forceinline__ void expand_item(uint32_t (&out)[8][4], const Runs<K>
 
 // (box along q, box along p, batch box) of M tile mt
 struct BoxIdx {
-    int qb, pb, bb;
+    int qb, pb;
+    int64_t bb;
 };
-__device__ __forceinline__ BoxIdx box_of(int mt, const ConvBox &box)
+__device__ __forceinline__ BoxIdx box_of(int64_t mt, const ConvBox &box)
 {
-    const uint32_t t = box.byQ.quot(static_cast<uint32_t>(mt)), b = box.byP.quot(t);
-    return BoxIdx{static_cast<int>(mt - t * box.byQ.d), static_cast<int>(t - b * box.byP.d), static_cast<int>(b)};
-}
-
-// gather: a column's receptive field.  What bounds the gather is its instructions
-// between two stages, so the place of a reduction index is formed once per stage
-// with multiplies and shifts, and a column adds one offset and two range checks
-// (fp32 3x3, 360 -> 32 at 40 x 12, 5 images: 163 -> 72 us; bf16 stride 3, 64 -> 64
-// at 28 x 28, 64 images: 18.3 -> 9.3 us).  The element of tap (kh, kw) and channel ci
-// lies at off + (kh * W + kw) * Cin + ci, inside the image when its row hb + kh and
-// column wb + kw are (products: off = n * Cin, always inside)
-struct GatherSite {
-    int64_t off;
-    int hb, wb;
-};
-__device__ __forceinline__ GatherSite gather_site(const FwdParams &p, int64_t n)
-{
-    const ColumnSite s = column_site(p, n);
-    return GatherSite{s.img + (static_cast<int64_t>(s.hb) * p.W + s.wb) * p.Cin, s.hb, s.wb};
-}
-
-// gather: the place of reduction index r, the same for every column of a stage
-struct GatherTap {
-    int64_t off;
-    int kh, kw;
-};
-__device__ __forceinline__ GatherTap gather_tap(const FwdParams &p, const ConvBox &box, int64_t r)
-{
-    const uint32_t tap = box.byC.quot(static_cast<uint32_t>(r));
-    const uint32_t kh = box.byKW.quot(tap), kw = tap - kh * box.byKW.d;
-    return GatherTap{(static_cast<int64_t>(kh) * p.W + kw) * p.Cin + (r - static_cast<int64_t>(tap) * p.Cin),
-                     static_cast<int>(kh), static_cast<int>(kw)};
-}
-
-// output pixel -> input pixel of tap offset a = k - pad under a stride of 1 or 2:
-// input index p_out * stride + a lies on parity lattice r at place p_out + d
-struct TapSite {
-    int r, d;
-};
-__device__ __forceinline__ TapSite tap_site(int a, int stride)
-{
-    const int r = a & (stride - 1);
-    return TapSite{r, (a - r) >> (stride - 1)};
+    BoxIdx i;
+    i.qb = static_cast<int>(mt % box.nQ);
+    const int64_t t = mt / box.nQ;
+    i.pb = static_cast<int>(t % box.nP);
+    i.bb = t / box.nP;
+    return i;
 }
 
 // PK: tmB0 / tmB1 are the maps of the packed values and indices (2-D over
 // [Cout/G][R*K]); otherwise the maps of the workspace planes
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false, bool SK = false>
-__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThreads, 1)
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
+__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads, 1)
     gemm_ws_kernel(FwdParams p, const __grid_constant__ AMaps tmA, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmY, ConvBox box,
-                   int n_tiles)
+                   int64_t n_ct, int64_t n_tiles)
 {
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
     constexpr int kM = C::kM, kN = C::kN, kKS = C::kKS, kStages = C::kStages;
     constexpr int kLag = 2;  // bf16 gather: stages in flight before a producer's arrive
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t raw = tc::smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t resb = base + kStages * C::kStage;  // resident weights (kRes)
-    const uint32_t hbuf = resb + C::kResBytes;         // halo ring (kAHalo: box.nh buffers)
+    const uint32_t hbuf = base + kStages * C::kStage;  // halo ring (kAHalo: box.nh buffers)
     const uint32_t hbytes = static_cast<uint32_t>(box.hrows) * 128u;
     const uint32_t hring = C::kHalo ? static_cast<uint32_t>(box.nh) * hbytes : 0u;
     const uint32_t ybuf = hbuf + hring;  // output staging buffers, two per epilogue group
-    const uint32_t sbias = ybuf + C::kYBufs * C::kYBuf;  // biases, per epilogue group
-    tc::Smem *S = reinterpret_cast<tc::Smem *>(smem_raw + (sbias - raw) + C::kEG * C::kBiasBytes);
+    tc::Smem *S = reinterpret_cast<tc::Smem *>(smem_raw + (base - raw) + kStages * C::kStage + hring +
+                                               C::kYBufs * C::kYBuf);
     const int taps = p.KH * p.KW;  // kAHalo: stages run chunk by chunk, the taps of a chunk in turn
     volatile int *abort = &S->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cpt = is_box(ASRC) ? static_cast<int>((p.Cin + kKS - 1) / kKS) : 1;  // stages per tap (boxes)
-    const int nks_all = is_box(ASRC) ? taps * cpt : static_cast<int>((p.R + kKS - 1) / kKS);
-    const uint32_t crank = C::kPairUnits || SK ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
+    const int nks = static_cast<int>((p.R + kKS - 1) / kKS);
+    const uint32_t crank = C::kPairUnits ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
     // work units: tiles (CG = 1) or pair tiles of 2 x 128 rows (CG = 2), strided over
     // the CTAs (CG = 1) or the CTA pairs (CG = 2)
-    const int u0 = C::kPairUnits ? blockIdx.x / 2 : (SK ? blockIdx.x >> box.log_split : blockIdx.x);
-    const int ustep = C::kPairUnits ? gridDim.x / 2 : (SK ? gridDim.x >> box.log_split : gridDim.x);
-    // this CTA's stages of a tile: kbase .. kbase + nks - 1 (all of them unless SK)
-    const int kbase =
-        SK ? static_cast<int>((static_cast<int64_t>(crank) * nks_all) >> box.log_split) : 0;
-    const int nks =
-        SK ? static_cast<int>((static_cast<int64_t>(crank + 1) * nks_all) >> box.log_split) - kbase : nks_all;
-    // unit u -> (M tile, N tile)
-    auto split_unit = [&](int u, int &mt, int &ct) {
-        const int q = static_cast<int>(box.byN.quot(static_cast<uint32_t>(u)));
-        ct = u - q * static_cast<int>(box.byN.d);
-        mt = C::kPairUnits ? 2 * q + static_cast<int>(crank) : q;
+    const int64_t u0 = C::kPairUnits ? blockIdx.x / 2 : blockIdx.x;
+    const int64_t ustep = C::kPairUnits ? gridDim.x / 2 : gridDim.x;
+    // unit u -> (M tile, N tile): one 64-bit division, the remainder by multiply-subtract
+    auto split_unit = [&](int64_t u, int64_t &mt, int64_t &ct) {
+        const int64_t q = u / n_ct;
+        ct = u - q * n_ct;
+        mt = C::kPairUnits ? 2 * q + crank : q;
     };
 
     if (tid == 0) {
-        // aux[k], kRes: chunk k of the resident weights has landed
         // full[s]: the copy issuer's expect_tx arrival (none for PK halo stages) and
         // PK: one arrival per producer warp of the stage's group in each CTA of the
         // pair (after the warp's writes), else 128 producer arrivals when the
@@ -945,7 +819,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         S->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (is_box(ASRC) && box.rows < kM) {
+    if (ASRC == kA4d && box.rows < kM) {
         // rows past the box are never copied: keep them zero for the MMAs
         for (uint32_t o = static_cast<uint32_t>(tid) * 16; o < static_cast<uint32_t>(kStages * C::kStage);
              o += C::kThreads * 16)
@@ -969,7 +843,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
     }
     if (tid == 288) {
         if constexpr (ASRC == kA2d) tc::tma_prefetch_desc(&tmA.m[0]);
-        if constexpr (is_box(ASRC))
+        if constexpr (ASRC == kA4d)
             for (int i = 0; i < p.sh * p.sw; ++i) tc::tma_prefetch_desc(&tmA.m[i]);
         if constexpr (ASRC == kAHalo) tc::tma_prefetch_desc(&tmA.m[0]);
         if constexpr (!PK) tc::tma_prefetch_desc(&tmB0);
@@ -979,236 +853,156 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     // the pair's barriers are initialised before either CTA signals the other's
-    // (SK: every CTA of the cluster runs before another stores into it)
-    if constexpr (C::kPairUnits || SK) cluster_sync();
+    if constexpr (C::kPairUnits) cluster_sync();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S->tmem_base;
-    // Launched as a programmatic dependent of the decompression: everything above
-    // overlaps its tail.  The workspace is read, and the output written, only after
-    // that grid has completed (tc::wait_prior_grid in each role).  The activations of
-    // a launch directly behind the decompression are read at once (p.a_early): this
-    // grid was scheduled when every block of the decompression had signalled, which
-    // each does after the grid before it, X's producer among all earlier ones, has
-    // completed and is visible.
+    // launched as a programmatic dependent of the decompression: everything above
+    // overlaps its tail; the workspace (and anything else in memory) is read only
+    // after that grid has completed and its writes are visible
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp >= 9 && warp < 9 + C::kIssuers) {
         // ------------------------------------------------------------ TMA issuers
         // bytes of one stage's copies: rows x the indices copied per stage (fewer than
         // the stage depth only for bf16 products of fewer than 64 reduction indices,
-        // which run in the two-group short-tile form, and convolutions of fewer channels)
-        const uint32_t erow = static_cast<uint32_t>(EPI == 2 || C::kTapChunks ? p.kin : kKS) * (TF32 ? 4u : 2u);  // bytes per row
-        const uint32_t a_bytes = (is_box(ASRC) ? static_cast<uint32_t>(box.rows) : static_cast<uint32_t>(kM)) * erow;
+        // which run in the two-group short-tile form)
+        const uint32_t erow = static_cast<uint32_t>(EPI == 2 ? p.kin : kKS) * (TF32 ? 4u : 2u);  // bytes per row
+        const uint32_t a_bytes = (ASRC == kA4d ? static_cast<uint32_t>(box.rows) : static_cast<uint32_t>(kM)) * erow;
         const uint32_t b_bytes = static_cast<uint32_t>(C::kBPlanes * C::kBRows) * erow;
+        const int cpt = static_cast<int>(p.Cin / kKS);  // stages per tap (kA4d)
         const uint32_t halo_bytes =
             static_cast<uint32_t>((box.QB + p.KW - 1) * (box.PB + p.KH - 1)) * 128u;  // kAHalo
-        // One lane of each warp runs its loop, with every coordinate advanced by adds
-        // and compares.  What a box costs is the length of this loop, not its bytes:
-        // with the coordinates formed by run-time divisions a stage took one issuer
-        // over 2000 cycles and six of them about 550; without, a probe of this loop
-        // issues a box every 246 cycles from one warp and every 135 from two (2 to
-        // 32 KB alike, 25-29 TB/s over the GPU from L2).
+        // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows;
+        // the other issuer warps copy the weight stages in turn
+        const int issuer = warp - (C::kHalo ? 10 : 9);
+        constexpr int kBIssuers = C::kHalo ? C::kIssuers - 1 : C::kIssuers;
+        int it = 0;
+        bool ok = true;
         if (C::kHalo && warp == 9) {
-            // kAHalo: warp 9 copies the halos, as far ahead as the halo ring allows
-            if (!p.a_early) tc::wait_prior_grid();
-            if (tc::elect_one()) {
-                int hb = 0;
-                uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
-                const int chunks = nks / taps;
-                bool ok = true;
-                for (int u = u0; u < n_tiles && ok; u += ustep) {
-                    int mt, ct;
-                    split_unit(u, mt, ct);
-                    const BoxIdx bi = box_of(mt, box);
-                    const int y = bi.pb * box.PB - p.ph;
-                    for (int c = 0; c < chunks; ++c) {
-                        // buffer hb is free once the MMAs of the chunk nh before completed
-                        ok = tc::mbar_wait(&S->hempty[hb], ph, abort, p.status);
-                        if (!ok) break;
+            int hc = 0;
+            const int chunks = nks / taps;
+            for (int64_t u = u0; u < n_tiles && ok; u += ustep) {
+                int64_t mt, ct;
+                split_unit(u, mt, ct);
+                const BoxIdx bi = box_of(mt, box);
+                for (int c = 0; c < chunks && ok; ++c, ++hc) {
+                    // buffer hb is free once the MMAs of chunk hc - nh completed; this
+                    // warp waited for chunk hc - 1 - nh before, so the phase cannot alias
+                    const int hb = hc % box.nh;
+                    if (hc >= box.nh) ok = tc::mbar_wait(&S->hempty[hb], ((hc / box.nh) - 1) & 1, abort, p.status);
+                    if (!ok) break;
+                    if (lane == 0) {
                         if constexpr (CG == 2) {
                             // each CTA's halo (its own M tile) completes on the even CTA's
                             // barrier, which expects both
                             if (crank == 0) tc::mbar_arrive_expect_tx(&S->hfull[hb], 2 * halo_bytes);
-                            tma_load_4d_pair(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, y, bi.bb,
-                                             map_to_rank(tc::smem_u32(&S->hfull[hb]), 0));
+                            tma_load_4d_pair(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, bi.pb * box.PB - p.ph,
+                                             static_cast<int>(bi.bb), map_to_rank(tc::smem_u32(&S->hfull[hb]), 0));
                         } else {
                             tc::mbar_arrive_expect_tx(&S->hfull[hb], halo_bytes);
-                            tc::tma_load_4d(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, y, bi.bb, &S->hfull[hb]);
-                        }
-                        if (++hb == box.nh) {
-                            hb = 0;
-                            ph ^= 1u;
+                            tc::tma_load_4d(hbuf + hb * hbytes, &tmA.m[0], c * 64, -p.pw, bi.pb * box.PB - p.ph,
+                                            static_cast<int>(bi.bb), &S->hfull[hb]);
                         }
                     }
+                    __syncwarp();
                 }
             }
-        } else if (!(PK && C::kHalo) && tc::elect_one()) {  // PK halo stages hold only the producers' weight tiles
-            // the stages of this warp: every kBIssuers-th, from its own number on
-            constexpr int kBIssuers = C::kHalo ? C::kIssuers - 1 : C::kIssuers;
-            int s = warp - (C::kHalo ? 10 : 9), ks = s;
-            uint32_t ph = 1u;  // a fresh barrier's preceding phase counts as complete
-            // a stage's place in its tile: (tap, chunk of kKS channels), chunks innermost
-            // (kA4d) or taps innermost (kAHalo); one chunk after the other for products
-            int kh = 0, kw = 0, c = 0;
-            auto step = [&](int by) {
-                if constexpr (is_box(ASRC)) {
-                    c += by;
-                    while (c >= cpt) {
-                        c -= cpt;
-                        if (++kw == p.KW) {
-                            kw = 0;
-                            if (++kh == p.KH) kh = 0;
+        } else if (!(PK && C::kHalo))  // PK halo stages hold only the producers' weight tiles
+        for (int64_t u = u0; u < n_tiles && ok; u += ustep) {
+            int64_t mt, ct;
+            split_unit(u, mt, ct);
+            const int64_t co0 = ct * kN + (CG == 2 ? crank * C::kBRows : 0);  // this CTA's B rows
+            BoxIdx bi{0, 0, 0};
+            if constexpr (ASRC == kA4d || ASRC == kAHalo) bi = box_of(mt, box);
+            // resident weights (halo copies): only the first tile's stages are copied
+            if (C::kHalo && box.resident && it >= nks) break;
+            for (int ks = 0; ks < nks && ok; ++ks, ++it) {
+                if (it % kBIssuers != issuer) continue;
+                const int s = it % kStages;
+                if (it >= kStages) ok = tc::mbar_wait(&S->empty[s], ((it / kStages) - 1) & 1, abort, p.status);
+                if (!ok) break;
+                if constexpr (ASRC == kAHalo) {
+                    const int c = ks / taps, t = ks - c * taps;  // stages: chunk by chunk, taps in turn
+                    if (lane == 0) {
+                        const int x = static_cast<int>(t * p.Cin) + c * 64;
+                        if constexpr (CG == 2) {  // this CTA's half of the rows, on the even CTA's barrier
+                            if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * C::kBBytes);
+                            tma_load_2d_pair(base + s * C::kStage, &tmB0, x, static_cast<int>(co0),
+                                             map_to_rank(tc::smem_u32(&S->full[s]), 0));
+                        } else {
+                            tc::mbar_arrive_expect_tx(&S->full[s], C::kBBytes);
+                            tc::tma_load_2d(base + s * C::kStage, &tmB0, x, static_cast<int>(ct * kN), &S->full[s]);
                         }
                     }
-                } else if constexpr (ASRC == kAHalo) {
-                    kw += by;  // the tap's number
-                    while (kw >= taps) {
-                        kw -= taps;
-                        if (++c == nks / taps) c = 0;
+                    __syncwarp();
+                    continue;
+                }
+                if (lane == 0 && CG == 2) {
+                    // both CTAs' copies complete on the even CTA's full barrier, which
+                    // expects the bytes of the pair (PK: the activations only; each
+                    // CTA's packed runs land on its own aux barrier)
+                    const uint32_t st = base + s * C::kStage;
+                    const uint32_t bst = st + C::kAPlane;
+                    const uint32_t fb = map_to_rank(tc::smem_u32(&S->full[s]), 0);
+                    if constexpr (PK) {
+                        if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * a_bytes);
+                    } else {
+                        if (crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], 2 * (C::kBBytes + a_bytes));
+                        tma_load_2d_pair(bst, &tmB0, ks * kKS, static_cast<int>(co0), fb);
                     }
-                }
-            };
-            step(ks + kbase);
-            // resident weights (halo copies): only the first tile's stages are copied
-            const int u_end = C::kHalo && box.resident ? (u0 + 1 < n_tiles ? u0 + 1 : n_tiles) : n_tiles;
-            int u = u0, mt = 0, ct = 0, pmt = 0, pct = 0;
-            bool ahead = false;
-            BoxIdx bi{0, 0, 0};
-            bool fresh = true;  // the tile's coordinates are to be formed
-            // kA, kB: the operands copied; both by the loop that runs to the end, and
-            // before it, over the stages of a fresh ring (`most` of them): the
-            // activations while the decompression still runs, then the weights
-            auto copy_stages = [&](auto kA, auto kB, int most) {
-            for (int done = 0; (decltype(kA)::value && decltype(kB)::value) || done < most; ++done) {
-                constexpr bool kCopyA = decltype(kA)::value, kCopyB = decltype(kB)::value;
-                while (ks >= nks && u < u_end) {
-                    ks -= nks;
-                    u += ustep;
-                    fresh = true;
-                }
-                if (u >= u_end) break;
-                if (fresh) {
-                    split_unit(u, mt, ct);
-                    if constexpr (is_box(ASRC)) bi = box_of(mt, box);
-                    if constexpr (C::kPrefetch) {
-                        split_unit(u + ustep, pmt, pct);
-                        ahead = u + ustep < u_end && nks <= 16 && box.byN.d >= 4u;
+                    if constexpr (ASRC == kA2d) {
+                        tma_load_2d_pair(st, &tmA.m[0], ks * kKS, static_cast<int>(mt * kM), fb);
+                    } else {
+                        const int tap = ks / cpt;
+                        const int ci0 = (ks - tap * cpt) * kKS;
+                        const int kh = tap / p.KW, kw = tap - (tap / p.KW) * p.KW;
+                        const int ah = kh - p.ph, aw = kw - p.pw;
+                        const int rh = ((ah % p.sh) + p.sh) % p.sh, rw = ((aw % p.sw) + p.sw) % p.sw;
+                        const int dh = (ah - rh) / p.sh, dw = (aw - rw) / p.sw;
+                        tma_load_4d_pair(st, &tmA.m[rh * p.sw + rw], ci0, bi.qb * box.QB + dw,
+                                         bi.pb * box.PB + dh, static_cast<int>(bi.bb * box.BB), fb);
                     }
-                    fresh = false;
-                }
-                if (kCopyA && !tc::mbar_wait(&S->empty[s], ph, abort, p.status)) break;
-                const uint32_t st = base + s * C::kStage;
-                const uint32_t bst = st + C::kBOff;
-                const int co0 = ct * kN + (CG == 2 ? static_cast<int>(crank) * C::kBRows : 0);  // this CTA's B rows
-                // the barrier that the copies complete on: the even CTA's of a pair, which
-                // expects the bytes of both (PK: the activations only)
-                const uint32_t fb = CG == 2 ? map_to_rank(tc::smem_u32(&S->full[s]), 0) : tc::smem_u32(&S->full[s]);
-                if constexpr (ASRC == kAHalo) {
-                    if (CG == 1 || crank == 0) tc::mbar_arrive_expect_tx(&S->full[s], CG * C::kBBytes);
-                    const int x = kw * static_cast<int>(p.Cin) + c * 64;
-                    if constexpr (CG == 2)  // this CTA's half of the rows
-                        tma_load_2d_pair(bst, &tmB0, x, co0, fb);
-                    else
-                        tc::tma_load_2d(bst, &tmB0, x, co0, &S->full[s]);
-                } else {
+                } else if (lane == 0) {
+                    const uint32_t st = base + s * C::kStage;
+                    const uint32_t bst = st + C::kBOff;
                     // the activation copy completes on aux (raw fp32, split afterwards) or full
-                    if constexpr (C::kARaw && kCopyA) tc::mbar_arrive_expect_tx(&S->aux[s], a_bytes);
-                    if (kCopyA && (CG == 1 || crank == 0))
-                        tc::mbar_arrive_expect_tx(&S->full[s],
-                                                  CG * ((PK || C::kRes ? 0u : b_bytes) + (C::kATma ? a_bytes : 0u)));
-                    if constexpr (!PK && !C::kRes && kCopyB) {
-                        if constexpr (C::kTapChunks) {
-                            if constexpr (CG == 2)
-                                tma_load_3d_pair(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, fb);
-                            else
-                                tc::tma_load_3d(bst, &tmB0, c * kKS, kh * p.KW + kw, co0, &S->full[s]);
-                        } else if constexpr (CG == 2) {
-                            tma_load_2d_pair(bst, &tmB0, (ks + kbase) * kKS, co0, fb);
-                        } else if constexpr (MC) {
+                    uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
+                    if constexpr (C::kARaw) tc::mbar_arrive_expect_tx(abar, a_bytes);
+                    if constexpr (PK) {
+                        tc::mbar_arrive_expect_tx(&S->full[s], a_bytes);
+                    } else {
+                        tc::mbar_arrive_expect_tx(&S->full[s], b_bytes + (C::kATma ? a_bytes : 0u));
+                        if constexpr (MC) {
                             // this CTA's half of the B rows into both CTAs (the same offsets);
                             // each CTA's full barrier expects the whole tile
                             const uint32_t half = crank * (C::kBPlane / 2);
-                            const int y = co0 + static_cast<int>(crank) * (kN / 2);
-                            tma_load_2d_mc(bst + half, &tmB0, ks * kKS, y, fb);
+                            const int y = static_cast<int>(co0) + static_cast<int>(crank) * (kN / 2);
+                            tma_load_2d_mc(bst + half, &tmB0, ks * kKS, y, tc::smem_u32(&S->full[s]));
                             if constexpr (C::kBPlanes > 1)
-                                tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, fb);
+                                tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, tc::smem_u32(&S->full[s]));
                         } else {
-                            tc::tma_load_2d(bst, &tmB0, (ks + kbase) * kKS, co0, &S->full[s]);
+                            tc::tma_load_2d(bst, &tmB0, ks * kKS, static_cast<int>(co0), &S->full[s]);
                             if constexpr (C::kBPlanes > 1)  // fp32 plane 1: 64 bf16 per stage
-                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, (ks + kbase) * 64, co0, &S->full[s]);
+                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, static_cast<int>(co0), &S->full[s]);
                         }
                     }
-                    uint64_t *abar = C::kARaw ? &S->aux[s] : &S->full[s];
-                    if constexpr (ASRC == kA2d && kCopyA) {
-                        if constexpr (CG == 2)
-                            tma_load_2d_pair(st, &tmA.m[0], ks * kKS, mt * kM, fb);
-                        else
-                            tc::tma_load_2d(st, &tmA.m[0], (ks + kbase) * kKS, mt * kM, abar);
-                        if constexpr (C::kPrefetch) {
-                            // the units of an M tile, which run at the same time, share its stages
-                            // out: ks modulo their number
-                            const int n = static_cast<int>(box.byN.d);
-                            if (ahead && ks - static_cast<int>(box.byN.quot(static_cast<uint32_t>(ks))) * n == pct)
-                                tc::tma_prefetch_2d(&tmA.m[0], ks * kKS, pmt * kM);
-                        }
-                    } else if constexpr (is_box(ASRC) && kCopyA) {
-                        // input row h = p_out * sh + kh - ph lies on lattice th.r at h' = p_out + th.d
-                        const TapSite th = tap_site(kh - p.ph, p.sh), tw = tap_site(kw - p.pw, p.sw);
-                        const CUtensorMap *m = &tmA.m[th.r * p.sw + tw.r];
-                        const int x1 = bi.qb * box.QB + tw.d, x2 = bi.pb * box.PB + th.d, x3 = bi.bb * box.BB;
-                        if constexpr (CG == 2)
-                            tma_load_4d_pair(st, m, c * kKS, x1, x2, x3, fb);
-                        else
-                            tc::tma_load_4d(st, m, c * kKS, x1, x2, x3, abar);
+                    if constexpr (ASRC == kA2d) {
+                        tc::tma_load_2d(st, &tmA.m[0], ks * kKS, static_cast<int>(mt * kM), abar);
+                    } else if constexpr (ASRC == kA4d) {
+                        const int tap = ks / cpt;
+                        const int ci0 = (ks - tap * cpt) * kKS;
+                        const int kh = tap / p.KW, kw = tap - (tap / p.KW) * p.KW;
+                        // input row h = p_out * sh + ah lies on lattice rh at h' = p_out + dh
+                        const int ah = kh - p.ph, aw = kw - p.pw;
+                        const int rh = ((ah % p.sh) + p.sh) % p.sh, rw = ((aw % p.sw) + p.sw) % p.sw;
+                        const int dh = (ah - rh) / p.sh, dw = (aw - rw) / p.sw;
+                        tc::tma_load_4d(st, &tmA.m[rh * p.sw + rw], ci0, bi.qb * box.QB + dw, bi.pb * box.PB + dh,
+                                        static_cast<int>(bi.bb * box.BB), abar);
                     }
                 }
-                ks += kBIssuers;
-                step(kBIssuers);
-                s += kBIssuers;  // kBIssuers <= kStages
-                if (s >= kStages) {
-                    s -= kStages;
-                    ph ^= 1u;
-                }
+                __syncwarp();
             }
-            };
-            constexpr std::true_type kYes{};
-            if constexpr (!PK && (ASRC == kA2d || is_box(ASRC))) {
-                if (p.a_early) {
-                    constexpr std::false_type kNo{};
-                    const int most = (kStages - s + kBIssuers - 1) / kBIssuers;  // this warp's stages of the ring
-                    const int s0 = s, ks0 = ks, kh0 = kh, kw0 = kw, c0 = c;
-                    copy_stages(kYes, kNo, most);
-                    if constexpr (!C::kRes) {  // back to the first, for the weights
-                        s = s0;
-                        ks = ks0;
-                        kh = kh0;
-                        kw = kw0;
-                        c = c0;
-                        u = u0;
-                        ph = 1u;
-                        fresh = true;
-                    }
-                    tc::wait_prior_grid();
-                    if constexpr (!C::kRes) copy_stages(kNo, kYes, most);
-                } else {
-                    tc::wait_prior_grid();
-                }
-                if constexpr (C::kRes) {
-                    // the activations go on where they stopped; first the weights of this
-                    // CTA's N tile, chunk k by warp 9 + k (kResB <= kBIssuers)
-                    const int k = warp - 9;
-                    if (k < nks && u0 < n_tiles) {
-                        int mt0, ct0;
-                        split_unit(u0, mt0, ct0);
-                        tc::mbar_arrive_expect_tx(&S->aux[k], b_bytes);
-                        tc::tma_load_2d(resb + k * C::kBPlane, &tmB0, k * kKS, ct0 * kN, &S->aux[k]);
-                    }
-                }
-            } else {
-                tc::wait_prior_grid();
-            }
-            copy_stages(kYes, kYes, 0);
         }
-        __syncwarp();
     } else if (PK && ((warp >= 4 && warp < 8) || warp >= 9 + C::kIssuers)) {
         // ------------------------------------------------------------ weight producers (PK)
         // two groups of four warps (4-7 and the four after the issuers) take the
@@ -1221,13 +1015,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         // stage may still be in use, and stored once the stage's MMAs released it;
         // then each warp releases its writes to the stage's full barrier (pair: the
         // even CTA's).
-        tc::wait_prior_grid();
         const int q = warp >= 8 ? 1 : 0;
         const int pt = tid - (q ? 32 * (9 + C::kIssuers) : 128);
         const int m0 = (pt >> 3) * 8, c = pt & 7;
         const bool active = m0 < C::kBRows;
+        const int64_t groups = p.Cout / p.G;
         const int lg = 31 - __clz(p.G);  // G is a power of two
-        const int64_t groups = p.Cout >> lg;
         const uint32_t full_remote = CG == 2 ? map_to_rank(tc::smem_u32(&S->full[0]), 0) : 0u;
         bool bad = false;
         // a stage of this CTA, in the MMAs' order, and the item's place in it: the
@@ -1236,16 +1029,15 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         // pair, of each N tile).  Advanced stage by stage without division (one
         // per tile).
         struct Cursor {
-            int u;
-            int64_t co, g, r;
+            int64_t u, co, g, r;
             int ks, t, ch, j0;
             bool chk;
         };
         auto tile_start = [&](Cursor &cu) {
             if (cu.u >= n_tiles) return;
-            int mt, ct;
+            int64_t mt, ct;
             split_unit(cu.u, mt, ct);
-            cu.co = static_cast<int64_t>(ct) * kN + crank * C::kBRows + m0;
+            cu.co = ct * kN + crank * C::kBRows + m0;
             cu.g = cu.co >> lg;
             cu.j0 = static_cast<int>(cu.co & (p.G - 1));
             cu.chk = mt < CG;
@@ -1334,7 +1126,6 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         if (bad) report(p.status, CCI_ERR_INDEX);
     } else if (warp >= 4 && warp < 8 && C::kEG == 1) {
         // ------------------------------------------------------------ producers
-        if (!C::kATma && !C::kARaw && !p.a_early) tc::wait_prior_grid();  // the gather reads X
         const int pt = tid - 128;
         const int chunk = pt & 7;  // 16-byte chunk of every activation row this thread handles
         const int rowb = pt >> 3;  // rows rowb + 16 i
@@ -1343,41 +1134,43 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         constexpr bool kRegs = TF32 && ASRC == kAGather;  // fp32 gather through registers
         // fp32 gather: activation chunks of the next two stages, in registers
         uint4 xa[kRegs ? 8 : 1], xb[kRegs ? 8 : 1], xc[kRegs ? 8 : 1];
-        GatherSite xsite[kRegs ? 8 : 1];  // column sites of the tile being prefetched
-        uint32_t xin = 0u;                // bit i: column i of it exists
+        ColumnSite xsite[kRegs ? 8 : 1];  // column sites of the tile being prefetched
         int64_t xsite_tile = -1;
         auto load_x = [&](uint4 (&dst)[kRegs ? 8 : 1], int64_t tile, int ks) {
             if constexpr (kRegs) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i) dst[i] = make_uint4(0, 0, 0, 0);
                 if (tile >= n_tiles || ks >= nks) return;
-                int mt, ct;
-                split_unit(static_cast<int>(tile), mt, ct);
-                const int64_t n0 = static_cast<int64_t>(mt) * kM;
+                const int64_t n0 = (tile / n_ct) * kM;
                 if (tile != xsite_tile) {
-                    xin = 0u;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int64_t n = n0 + rowb + 16 * i;
-                        xsite[i] = GatherSite{0, 0, 0};
-                        if (n < p.N) {
-                            xsite[i] = gather_site(p, n);
-                            xin |= 1u << i;
-                        }
+                        xsite[i] = n < p.N ? column_site(p, n) : ColumnSite{-1, 0, 0};
                     }
                     xsite_tile = tile;
                 }
-                const int64_t r = static_cast<int64_t>(ks + kbase) * kKS + chunk * 4;
+                const int64_t r = static_cast<int64_t>(ks) * kKS + chunk * 4;
                 if (r >= p.R) return;
-                const GatherTap g = gather_tap(p, box, r);
-                const float *X = static_cast<const float *>(p.X) + g.off;
-                const uint32_t H = static_cast<uint32_t>(p.H), W = static_cast<uint32_t>(p.W);
+                int kh = 0, kw = 0;
+                int64_t ci = r;
+                if (p.is_conv) {
+                    const int tap = static_cast<int>(r / p.Cin);
+                    ci = r - static_cast<int64_t>(tap) * p.Cin;
+                    kh = tap / p.KW;
+                    kw = tap - kh * p.KW;
+                }
+                const float *X = static_cast<const float *>(p.X);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    // (products: H = W = 1 and tap (0, 0), inside)
-                    const bool in = static_cast<uint32_t>(xsite[i].hb + g.kh) < H &&
-                                    static_cast<uint32_t>(xsite[i].wb + g.kw) < W && (xin >> i & 1u);
-                    if (in) dst[i] = __ldg(reinterpret_cast<const uint4 *>(X + xsite[i].off));
+                    if (xsite[i].img < 0) continue;  // column past N
+                    int64_t off = xsite[i].img + r;
+                    if (p.is_conv) {
+                        const int h = xsite[i].hb + kh, w = xsite[i].wb + kw;
+                        if (h < 0 || h >= p.H || w < 0 || w >= p.W) continue;
+                        off = xsite[i].img + (static_cast<int64_t>(h) * p.W + w) * p.Cin + ci;
+                    }
+                    dst[i] = __ldg(reinterpret_cast<const uint4 *>(X + off));
                 }
             }
         };
@@ -1385,10 +1178,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         auto advance = [&](int64_t &tile, int &ks) {
             if (++ks == nks) {
                 ks = 0;
-                tile += ustep;
+                tile += gridDim.x;
             }
         };
-        int64_t t2 = u0;
+        int64_t t2 = blockIdx.x;
         int k2 = 0;
         if constexpr (kRegs) {
             load_x(xa, t2, k2);
@@ -1398,18 +1191,16 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         }
         if constexpr (!C::kATma) {
             // the same work units, in the same order, as the TMA issuers and the MMAs
-            for (int tile = u0; tile < n_tiles && ok; tile += ustep) {
-                int mt, ct;
-                split_unit(tile, mt, ct);
-                const int64_t n0 = static_cast<int64_t>(mt) * kM;
-                GatherSite site[8];
+            for (int64_t tile = u0; tile < n_tiles && ok; tile += ustep) {
+                const int64_t n0 = (tile / n_ct) * kM;
+                ColumnSite site[8];
                 bool colok[8];
                 if constexpr (!TF32) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int64_t n = n0 + rowb + 16 * i;
                         colok[i] = n < p.N;
-                        site[i] = colok[i] ? gather_site(p, n) : GatherSite{0, 0, 0};
+                        site[i] = colok[i] ? column_site(p, n) : ColumnSite{0, 0, 0};
                     }
                 }
                 for (int ks = 0; ks < nks && ok; ++ks, ++it) {
@@ -1424,14 +1215,30 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                     const uint32_t st = base + s * C::kStage;
                     if constexpr (!TF32) {
                         const uint16_t *X = static_cast<const uint16_t *>(p.X);
-                        const int64_t r = static_cast<int64_t>(ks + kbase) * kKS + chunk * 8;
-                        const GatherTap g = gather_tap(p, box, r < p.R ? r : 0);
-                        const uint32_t H = static_cast<uint32_t>(p.H), W = static_cast<uint32_t>(p.W);
+                        const int64_t r = static_cast<int64_t>(ks) * kKS + chunk * 8;
+                        const bool rok = r < p.R;
+                        int kh = 0, kw = 0;
+                        int64_t ci = r;
+                        if (p.is_conv && rok) {
+                            const int tap = static_cast<int>(r / p.Cin);
+                            ci = r - static_cast<int64_t>(tap) * p.Cin;
+                            kh = tap / p.KW;
+                            kw = tap - kh * p.KW;
+                        }
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
-                            const bool valid = r < p.R && colok[i] && static_cast<uint32_t>(site[i].hb + g.kh) < H &&
-                                               static_cast<uint32_t>(site[i].wb + g.kw) < W;
-                            const uint16_t *src = valid ? X + (site[i].off + g.off) : X;
+                            bool valid = colok[i] && rok;
+                            const uint16_t *src = X;
+                            if (valid) {
+                                if (!p.is_conv) {
+                                    src = X + site[i].img + r;
+                                } else {
+                                    const int h = site[i].hb + kh, w = site[i].wb + kw;
+                                    valid = h >= 0 && h < p.H && w >= 0 && w < p.W;
+                                    if (valid)
+                                        src = X + site[i].img + (static_cast<int64_t>(h) * p.W + w) * p.Cin + ci;
+                                }
+                            }
                             tc::cp_async16(st + sw_chunk(rowb + 16 * i, chunk), src, valid);
                         }
                         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1502,9 +1309,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         int it = 0, t = 0;
         bool ok = CG == 1 || crank == 0;
         const int hchunks = ASRC == kAHalo ? nks / taps : 0;
-        const uint64_t hdesc0 = tc::sw128_desc(hbuf), bdesc0 = tc::sw128_desc(base), rdesc0 = tc::sw128_desc(resb);
+        const uint64_t hdesc0 = tc::sw128_desc(hbuf), bdesc0 = tc::sw128_desc(base);
         const uint32_t empty0 = tc::smem_u32(&S->empty[0]);
-        const uint32_t issue = tc::elect_one() ? 1u : 0u;  // the lane that issues (a predicate in the stage block)
+        const uint32_t issue = lane == 0 ? 1u : 0u;  // the lane that issues (a predicate in the stage block)
         auto commit = [&](uint64_t *bar) {
             if constexpr (CG == 2)
                 mma_commit_pair(bar);
@@ -1515,8 +1322,8 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
             // one thread runs the whole issue loop: no per-stage divergence or warp
             // reconvergence between the stages' MMAs (the gaps between stages, not
             // the MMAs, bounded this product)
-            if (tc::elect_one()) {
-                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
+            if (lane == 0) {
+                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     if (t >= 2) ok = tc::mbar_wait(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
                     if (!ok) break;
@@ -1541,17 +1348,12 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
             // bf16 stages of one A and one B plane: one thread runs the issue loop,
             // each stage's MMAs and its commit issued from one block (pairs: from the
             // even CTA, which alone enters with ok set)
-            if (ok && tc::elect_one()) {
+            if (lane == 0 && ok) {
                 int s = 0;
                 uint32_t ph = 0u;  // parity of the full-barrier phase to wait for
                 const uint64_t sunits = C::kStage >> 4, bunits = C::kBOff >> 4;
-                // MMAs per stage: the copied indices by 16 (EPI = 2, kTapChunks), fewer in a
-                // tap's last chunk of 64
-                const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;
-                const uint32_t n16_last =
-                    cpt > 1 ? (static_cast<uint32_t>(p.Cin - (cpt - 1) * kKS) + 15u) >> 4 : n16;
-                int left = cpt - kbase % cpt;  // chunks of the tap still to come, this one among them
-                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                const uint32_t n16 = static_cast<uint32_t>(p.kin) >> 4;  // MMAs per stage (EPI = 2)
+                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
                     if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1564,28 +1366,14 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t ad = bdesc0 + static_cast<uint64_t>(s) * sunits;
-                        uint64_t bd = ad + bunits;
-                        if constexpr (C::kRes) {
-                            if (t == 0) {  // the chunk's weights land once, for the first tile
-                                ok = tc::mbar_wait(&S->aux[ks], 0u, abort, p.status);
-                                if (!ok) break;
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            }
-                            bd = rdesc0 + static_cast<uint64_t>(ks) * (C::kBPlane >> 4);
-                        }
-                        uint32_t n = n16;
-                        if constexpr (C::kTapChunks) {
-                            if (--left == 0) {
-                                left = cpt;
-                                n = n16_last;
-                            }
-                        }
                         if constexpr (CG == 2)
-                            stage_f16_pair<C::kIdesc, C::kTapChunks>(d, ad, bd, ks > 0 ? 1u : 0u, empty0 + 8u * s, n);
-                        else if constexpr (EPI == 2 || C::kTapChunks)  // fewer than four MMAs: R < 64, few channels
-                            stage_f16<C::kIdesc, MC, true>(d, ad, bd, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s, n);
+                            stage_f16_pair<C::kIdesc>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, empty0 + 8u * s);
                         else
-                            stage_f16<C::kIdesc, MC>(d, ad, bd, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
+                            if constexpr (EPI == 2)  // short tiles: fewer than four MMAs when R < 64
+                                stage_f16<C::kIdesc, MC, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u,
+                                                               empty0 + 8u * s, n16);
+                            else
+                                stage_f16<C::kIdesc, MC>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
                         if (++s == kStages) {
                             s = 0;
                             ph ^= 1u;
@@ -1604,62 +1392,20 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
             // released; otherwise each tap is a stage of the ring.  Descriptors in
             // 16-byte units: + wq_units per halo row of taps, + 8 per column,
             // + hunits per halo buffer, + sunits per stage.
-            if (ok && tc::elect_one()) {
+            if (lane == 0 && ok) {
                 int hs = 0, hb = 0;
                 uint32_t hsph = 0u, hph = 0u;
                 const uint64_t wq_units = static_cast<uint64_t>(box.QB + p.KW - 1) * 8u;
                 const uint64_t hunits = hbytes >> 4, sunits = C::kStage >> 4;
-                if constexpr (CG == 1) {  // (pairs never keep their weights resident: slower, below)
-                    if (box.resident) {
-                        // One chunk, nine weight tiles.  The next tile's accumulator and halo are
-                        // waited for before the last kernel row of this one is issued, so that
-                        // the waits' latency passes while the tensor core still has work: with the
-                        // waits between the tiles it idled 680 of 2660 cycles a tile (64 -> 64 at
-                        // 56 x 56, 128 images: 40.2 us a pass, 30.9 so).  (In the loop below, whose
-                        // halos are re-copied with every chunk and come late, the same order
-                        // delays the last row: 128 -> 128 at 28 x 28, 128 images 24.3 -> 25.3.)  (CTA pairs, which read 5 KB of operands per SM and
-                        // MMA instead of 6, took 47.8 us.)
-                        auto ready = [&](int tt, int h, uint32_t parity) {
-                            if (tt >= 2 && !tc::mbar_wait(&S->tmem_empty[tt & 1], ((tt / 2) - 1) & 1, abort, p.status))
-                                return false;
-                            return tc::mbar_wait(&S->hfull[h], parity, abort, p.status);
-                        };
-                        if (u0 < n_tiles) ok = ready(0, 0, 0u);
-                        for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
-                            const uint32_t d = tmem + static_cast<uint32_t>((t & 1) * kN);
-                            const uint64_t hdesc = hdesc0 + static_cast<uint64_t>(hb) * hunits;
-                            const int nhb = hb + 1 == box.nh ? 0 : hb + 1;
-                            const uint32_t nph = nhb == 0 ? hph ^ 1u : hph;
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-                            for (int kh = 0; kh < 3; ++kh) {
-                                if (t == 0) {  // the row's weights land once, for the first tile
-                                    for (int kw = 0; kw < 3 && ok; ++kw)
-                                        ok = tc::mbar_wait(&S->full[3 * kh + kw], 0u, abort, p.status);
-                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                }
-                                if (kh == 2 && ok && u + ustep < n_tiles) ok = ready(t + 1, nhb, nph);
-                                if (!ok) break;
-                                row3_f16<C::kIdesc, (C::kStage >> 4)>(
-                                    d, hdesc + static_cast<uint64_t>(kh) * wq_units,
-                                    bdesc0 + static_cast<uint64_t>(3 * kh) * sunits, kh != 0 ? 1u : 0u);
-                            }
-                            if (!ok) break;
-                            commit(&S->hempty[hb]);
-                            commit(&S->tmem_full[t & 1]);
-                            hb = nhb;
-                            hph = nph;
-                        }
-                        ok = false;  // the loop below is not entered
-                    }
-                }
-                for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
+                const bool res = box.resident != 0;
+                for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
                     const int acc = t & 1;
                     // CG = 2: the phase includes arrivals of the odd CTA's epilogue
                     if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t d = tmem + static_cast<uint32_t>(acc * kN);
+                    if (res) hs = 0;
                     for (int c = 0; c < hchunks && ok; ++c) {
                         ok = tc::mbar_wait(&S->hfull[hb], hph, abort, p.status);
                         if (!ok) break;
@@ -1667,19 +1413,32 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                         const uint64_t hdesc = hdesc0 + static_cast<uint64_t>(hb) * hunits;
                         for (int kh = 0; kh < 3 && ok; ++kh) {
                             const uint64_t arow = hdesc + static_cast<uint64_t>(kh) * wq_units;
-                            for (int kw = 0; kw < 3 && ok; ++kw) {
-                                ok = tc::mbar_wait(&S->full[hs], hsph, abort, p.status);
-                                if (!ok) break;
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint64_t bd = bdesc0 + static_cast<uint64_t>(hs) * sunits;
-                                const uint32_t accf = (c | kh | kw) != 0 ? 1u : 0u;
-                                if constexpr (CG == 2)  // the pair's MMAs; the stage released in both CTAs
-                                    stage_f16_pair<C::kIdesc>(d, arow + kw * 8u, bd, accf, empty0 + 8u * hs);
-                                else
-                                    stage_f16<C::kIdesc>(d, arow + kw * 8u, bd, accf, 1u, empty0 + 8u * hs);
-                                if (++hs == kStages) {
-                                    hs = 0;
-                                    hsph ^= 1u;
+                            if (res) {
+                                if (t == 0) {  // the row's weights land once, for the first tile
+                                    for (int kw = 0; kw < 3 && ok; ++kw)
+                                        ok = tc::mbar_wait(&S->full[hs + kw], 0u, abort, p.status);
+                                    if (!ok) break;
+                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                                }
+                                if constexpr (CG == 1)  // (pairs never keep their weights resident)
+                                    row3_f16<C::kIdesc, (C::kStage >> 4)>(
+                                        d, arow, bdesc0 + static_cast<uint64_t>(hs) * sunits, (c | kh) != 0 ? 1u : 0u);
+                                hs += 3;
+                            } else {
+                                for (int kw = 0; kw < 3 && ok; ++kw) {
+                                    ok = tc::mbar_wait(&S->full[hs], hsph, abort, p.status);
+                                    if (!ok) break;
+                                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                                    const uint64_t bd = bdesc0 + static_cast<uint64_t>(hs) * sunits;
+                                    const uint32_t accf = (c | kh | kw) != 0 ? 1u : 0u;
+                                    if constexpr (CG == 2)  // the pair's MMAs; the stage released in both CTAs
+                                        stage_f16_pair<C::kIdesc>(d, arow + kw * 8u, bd, accf, empty0 + 8u * hs);
+                                    else
+                                        stage_f16<C::kIdesc>(d, arow + kw * 8u, bd, accf, 1u, empty0 + 8u * hs);
+                                    if (++hs == kStages) {
+                                        hs = 0;
+                                        hsph ^= 1u;
+                                    }
                                 }
                             }
                         }
@@ -1694,7 +1453,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
             }
             ok = false;  // the generic loop below is not entered
         }
-        for (int u = u0; u < n_tiles && ok; u += ustep, ++t) {
+        for (int64_t u = u0; u < n_tiles && ok; u += ustep, ++t) {
             const int acc = t & 1;
             // CG = 2: the phase includes arrivals of the odd CTA's epilogue
             if (t >= 2) ok = tc::mbar_wait<CG == 2>(&S->tmem_empty[acc], ((t / 2) - 1) & 1, abort, p.status);
@@ -1707,7 +1466,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 ok = tc::mbar_wait<PK && CG == 2>(&S->full[s], (it / kStages) & 1, abort, p.status);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (tc::elect_one()) {
+                if (lane == 0) {
                     const uint32_t st = base + s * C::kStage;
                     const uint32_t bst = st + C::kBOff;
                     if constexpr (TF32) {
@@ -1736,11 +1495,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                                          ks > 0 ? 1u : 0u, issue, empty0 + 8u * s);
                 __syncwarp();
             }
-            if (ok && tc::elect_one()) commit(&S->tmem_full[acc]);
+            if (ok && lane == 0) commit(&S->tmem_full[acc]);
             __syncwarp();
         }
-        // (the same thread as issued the MMAs: a commit covers its own thread's)
-        if ((CG == 1 || crank == 0) && tc::elect_one()) commit(&S->drain);
+        if (lane == 0 && (CG == 1 || crank == 0)) commit(&S->drain);
         __syncwarp();
         int no_abort = 0;
         tc::mbar_wait(&S->drain, 0, &no_abort, p.status);
@@ -1748,11 +1506,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         // ------------------------------------------------------------ epilogue (warps 0-3;
         // with EPI = 2 also warps 4-7 as a second group: group g takes the tiles
         // whose accumulator is g)
-        tc::wait_prior_grid();
         constexpr int kEG = C::kEG;
         const int eg = warp >> 2;              // this thread's group
-        const int etid = tid - 128 * eg;       // thread within the group
-        const bool storer = (warp & 3) == 0 && tc::elect_one();  // the thread that issues the group's stores
+        const int etid = tid - 128 * eg;       // thread within the group; 0 issues its stores
         const int ebar = 1 + eg;               // the group's named barrier
         int t = eg;
         bool ok = true;
@@ -1761,57 +1517,18 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
         int chunk_no = 0;
         // CG = 2: the odd CTA releases an accumulator on the even CTA's barrier
         const uint32_t tmem_empty_remote = CG == 2 ? map_to_rank(tc::smem_u32(&S->tmem_empty[0]), 0) : 0u;
-        // halo tiles: row m = pi * (Q + 2) + qi goes to staged row pi * Q + qi (the box
-        // of the store), the two unused columns of each row nowhere
-        int srow = m;
-        bool stage_row = true;
-        if constexpr (ASRC == kAHalo) {
-            const int wq = box.QB + p.KW - 1;
-            const int pi = m / wq, qi = m - pi * wq;
-            srow = pi * box.QB + qi;
-            stage_row = pi < box.PB && qi < box.QB;
-        }
-        const uint32_t gbias = sbias + static_cast<uint32_t>(eg * C::kBiasBytes);  // this group's
-        int bias_ct = -1;  // the N tile whose biases are staged
-        for (int u = u0 + eg * ustep; u < n_tiles && ok; u += kEG * ustep, t += kEG) {
+        for (int64_t u = u0 + eg * ustep; u < n_tiles && ok; u += kEG * ustep, t += kEG) {
             const int acc = t & 1;
-            int mt, ct;
+            int64_t mt, ct;
             split_unit(u, mt, ct);
-            const int co0 = ct * kN;
-            if (p.bias && ct != bias_ct) {
-                // before the barrier below; the group read the former ones before the last
-                // barrier of its tile before
-                for (int c = etid; c < kN; c += 128) {
-                    const float b = co0 + c < p.Cout ? __ldg(p.bias + co0 + c) : 0.f;
-                    asm volatile("st.shared.f32 [%0], %1;" ::"r"(gbias + 4 * c), "f"(b) : "memory");
-                }
-                bias_ct = ct;
-            }
+            const int co0 = static_cast<int>(ct * kN);
             BoxIdx bi{0, 0, 0};
-            if constexpr (is_box(ASRC) || ASRC == kAHalo) bi = box_of(mt, box);
+            if constexpr (ASRC == kA4d || ASRC == kAHalo) bi = box_of(mt, box);
             ok = tc::mbar_wait(&S->tmem_full[acc], (t / 2) & 1, abort, p.status);
             ok = tc::named_and(ebar, 128, ok);
             if (!ok) break;
             __syncwarp();
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if constexpr (SK) {
-                // this part's sums of four columns and 128 rows to the columns' owner
-                const int log_cols = (BN == 64 ? 6 : 7) - box.log_split;  // columns of an owner: 1 << log_cols
-                const uint32_t at = ybuf + (crank << (log_cols - 2)) * 2048u + static_cast<uint32_t>(m) * 16u;
-#pragma unroll 1
-                for (int c0 = 0; c0 < kN && co0 + c0 < p.Cout; c0 += 32) {
-                    uint32_t v[32];
-                    tc::tmem_ld32(tmem + lane_off + static_cast<uint32_t>(acc * kN + c0), v);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t c = static_cast<uint32_t>(c0 + 4 * j);
-                        if (co0 + c0 + 4 * j >= p.Cout) break;
-                        st_cluster_v4(map_to_rank(at + ((c & ((1u << log_cols) - 1u)) >> 2) * 2048u, c >> log_cols),
-                                      v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                    }
-                }
-                continue;
-            }
             const int sc = p.out_bf16 ? 64 : 32;  // output columns per staged 128-byte row
             const int cend = (p.Cout - co0) < kN ? static_cast<int>(p.Cout - co0) : kN;
 #pragma unroll 1
@@ -1824,16 +1541,16 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 const int nq = p.out_bf16 ? (valid + 7) / 8 : (valid + 3) / 4;
                 if (!p.out_bf16) {
                     tc::tmem_ld32(tcol, v);
-                    epilogue_math(v, p, gbias + 4 * c0);
+                    epilogue_math(v, p, co0 + c0);
                 } else {
                     uint32_t w[32];
                     tc::tmem_ld32(tcol, w);
-                    epilogue_math(w, p, gbias + 4 * c0);
+                    epilogue_math(w, p, co0 + c0);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) v[j] = bf16x2_rn(w[2 * j], w[2 * j + 1]);
                     if (valid > 32) {  // the second 32 columns (a narrower last chunk has none)
                         tc::tmem_ld32(tcol + 32, w);
-                        epilogue_math(w, p, gbias + 4 * (c0 + 32));
+                        epilogue_math(w, p, co0 + c0 + 32);
 #pragma unroll
                         for (int j = 0; j < 16; ++j) v[16 + j] = bf16x2_rn(w[2 * j], w[2 * j + 1]);
                     }
@@ -1850,8 +1567,18 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 // the store issued from it kYPerGroup chunks earlier has read it
                 constexpr int kYG = C::kYPerGroup;
                 const uint32_t buf = ybuf + static_cast<uint32_t>(kYG * eg + (chunk_no % kYG)) * C::kYBuf;
-                if (storer) tc::bulk_wait_read<kYG - 1>();
+                if (etid == 0) tc::bulk_wait_read<kYG - 1>();
                 tc::named_sync(ebar, 128);
+                // halo tiles: row m = pi * (Q + 2) + qi goes to staged row pi * Q + qi
+                // (the box of the store), the two unused columns of each row nowhere
+                int srow = m;
+                bool stage_row = true;
+                if constexpr (ASRC == kAHalo) {
+                    const int wq = box.QB + p.KW - 1;
+                    const int pi = m / wq, qi = m - (m / wq) * wq;
+                    srow = pi * box.QB + qi;
+                    stage_row = pi < box.PB && qi < box.QB;
+                }
                 if (stage_row) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
@@ -1860,73 +1587,24 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>::kThr
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tc::named_sync(ebar, 128);
-                if (storer) {
-                    if constexpr (is_box(ASRC) || ASRC == kAHalo)
-                        tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB, bi.bb * box.BB);
+                if (etid == 0) {
+                    if constexpr (ASRC == kA4d || ASRC == kAHalo)
+                        tc::tma_store_4d(&tmY, buf, co0 + c0, bi.qb * box.QB, bi.pb * box.PB,
+                                         static_cast<int>(bi.bb * box.BB));
                     else
-                        tc::tma_store_2d(&tmY, buf, co0 + c0, mt * kM);
+                        tc::tma_store_2d(&tmY, buf, co0 + c0, static_cast<int>(mt * kM));
                     tc::bulk_commit();
                 }
             }
         }
-        if (storer) tc::bulk_wait_all();
+        if (etid == 0) tc::bulk_wait_all();
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     // CG = 2: neither CTA leaves (or frees tensor memory) while the other may still
     // signal its barriers or the pair's MMAs may read its shared memory
-    if constexpr (C::kPairUnits || SK) cluster_sync();
-    if constexpr (SK) {
-        // every part's sums of this CTA's columns have landed (and nothing is stored into
-        // another CTA any more): row m of the tile, four columns at a time
-        if (warp < 4 && u0 < n_tiles) {
-            int mt, ct;
-            split_unit(u0, mt, ct);
-            int64_t n = -1;  // the row's column of the output, none past the box or the layer
-            if constexpr (is_box(ASRC)) {
-                const BoxIdx bi = box_of(mt, box);
-                const int qp = box.QB * box.PB, b = tid / qp, r = tid - b * qp, pi = r / box.QB, qi = r - pi * box.QB;
-                const int64_t ob = static_cast<int64_t>(bi.bb) * box.BB + b, op = bi.pb * box.PB + pi,
-                              oq = bi.qb * box.QB + qi;
-                if (tid < box.rows && ob < box.B && op < p.P && oq < p.Q) n = (ob * p.P + op) * p.Q + oq;
-            } else {
-                n = static_cast<int64_t>(mt) * kM + tid;
-                if (n >= p.N) n = -1;
-            }
-            const int cols = kN >> box.log_split, parts = 1 << box.log_split;
-            if (n >= 0) {
-                for (int q = 0; q < cols / 4; ++q) {
-                    const int cl = static_cast<int>(crank) * cols + 4 * q, co = ct * kN + cl;  // Cout is a multiple of 4
-                    if (co >= p.Cout) break;
-                    const uint32_t at = ybuf + static_cast<uint32_t>(q) * 2048u + static_cast<uint32_t>(tid) * 16u;
-                    float4 y = ld_shared_f4(at);
-                    for (int j = 1; j < parts; ++j) {
-                        const float4 z = ld_shared_f4(at + static_cast<uint32_t>(j * (cols / 4)) * 2048u);
-                        y.x += z.x;
-                        y.y += z.y;
-                        y.z += z.z;
-                        y.w += z.w;
-                    }
-                    if (p.bias) {
-                        const float4 b = ld_shared_f4(sbias + 4u * static_cast<uint32_t>(cl));
-                        y.x += b.x;
-                        y.y += b.y;
-                        y.z += b.z;
-                        y.w += b.w;
-                    }
-                    if (p.relu) y = make_float4(fmaxf(y.x, 0.f), fmaxf(y.y, 0.f), fmaxf(y.z, 0.f), fmaxf(y.w, 0.f));
-                    if (p.out_bf16)
-                        *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(p.Y) + n * p.Cout + co) =
-                            make_uint2(bf16x2_rn(__float_as_uint(y.x), __float_as_uint(y.y)),
-                                       bf16x2_rn(__float_as_uint(y.z), __float_as_uint(y.w)));
-                    else
-                        *reinterpret_cast<float4 *>(p.Y + n * p.Cout + co) = y;
-                }
-            }
-        }
-        __syncwarp();
-    }
+    if constexpr (C::kPairUnits) cluster_sync();
     if (warp == 8) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if constexpr (CG == 2)
@@ -2010,7 +1688,7 @@ inline bool build_a_maps(const FwdParams &p, const ConvBox &box, int asrc, bool 
         const int bx[4] = {64, box.QB + p.KW - 1, box.PB + p.KH - 1, 1};
         return make_map_strided(&am->m[0], p.X, dt, 4, dims, strides, bx);
     }
-    if (!is_box(asrc)) return true;
+    if (asrc != kA4d) return true;
     for (int rh = 0; rh < p.sh; ++rh)
         for (int rw = 0; rw < p.sw; ++rw) {
             const char *base = static_cast<const char *>(p.X) + (rh * p.W + rw) * p.Cin * e;
@@ -2080,16 +1758,21 @@ inline ConvBox choose_box(int64_t B_, int64_t P, int64_t Q)
     return best;
 }
 
-// the activation source of a layer for stage depth ks (elements per 128-byte row);
-// any_cin: the stages may be chunks of a tap's channels that end inside the depth
-inline int a_source(const FwdParams &p, int ks, bool any_cin)
+// the activation source of a layer for stage depth ks (elements per 128-byte row)
+inline int a_source(const FwdParams &p, int ks)
 {
     const int64_t lim = int64_t(1) << 30;
     if (!p.is_conv) return p.N < lim ? kA2d : kAGather;
     const bool fits = p.H < lim && p.W < lim && p.N < lim && (p.N / (p.P * p.Q)) < lim;
     const bool strides_ok = p.sh >= 1 && p.sh <= 2 && p.sw >= 1 && p.sw <= 2 && p.H >= p.sh && p.W >= p.sw;
-    if (!strides_ok || !fits) return kAGather;
-    return p.Cin % ks == 0 ? kA4d : (any_cin ? kATap : kAGather);
+    return (strides_ok && p.Cin % ks == 0 && fits) ? kA4d : kAGather;
+}
+
+// clusters of 1 << log_parts CTAs (one per SM) that run at once: they stay inside a
+// GPC, so larger ones leave SMs over (152 SMs: 76, 36 and 15)
+inline int64_t cluster_slots(int log_parts, int64_t sms)
+{
+    return log_parts == 0 ? sms : (log_parts == 1 ? sms / 2 : (log_parts == 2 ? sms * 15 / 64 : sms / 10));
 }
 
 // N tile among {64, 128, 256} (up to max_bn): fewest rounds of tiles over the
@@ -2111,83 +1794,23 @@ inline int choose_bn(int64_t m_tiles, int64_t Cout, int max_bn, int cg = 1)
     return best;
 }
 
-// CTAs of a launch with resident weights: whole rounds of the N tiles, so that a
-// CTA's tiles (every grid-th) are of one N tile
-inline int64_t resident_slots(int64_t n_ct) { return sm_count() / n_ct * n_ct; }
-
-// clusters of 1 << log_parts CTAs (one per SM) that run at once: they stay inside a
-// GPC, so larger ones leave SMs over (152 SMs: 76, 36 and 15)
-inline int64_t cluster_slots(int log_parts, int64_t sms)
-{
-    return log_parts == 0 ? sms : (log_parts == 1 ? sms / 2 : (log_parts == 2 ? sms * 15 / 64 : sms / 10));
-}
-
-// Split of the reduction of a layer with few tiles (SK): N tile and CTAs per tile.
-// Costs in SM cycles, measured on GB300: a stage (c64, c128: for N tiles of 64 and
-// 128), a tile's fill and epilogue, the exchange of the parts' sums (distributed
-// shared memory takes about 20 bytes a cycle and SM: 64 KB of sums for a 128-wide
-// tile).  The layer is split when that saves a seventh; a part keeps four stages at
-// least.  Without the exchange's share the 512 -> 512 layer at 7 x 7, 32 images was
-// split in two and went from 15.2 to 16.5 us.
-struct Split {
-    int log_parts = 0, bn = 0;
-};
-inline Split choose_split(int64_t m_tiles, int64_t Cout, int64_t nks, int64_t c64, int64_t c128)
-{
-    constexpr int64_t kTile = 4500;
-    const int64_t sms = sm_count();
-    Split best;
-    int64_t whole = -1, cost = -1;
-    for (int bn = 64; bn <= 128; bn *= 2) {
-        const int64_t tiles = m_tiles * ((Cout + bn - 1) / bn), c = bn == 64 ? c64 : c128;
-        const int64_t t = (tiles + sms - 1) / sms * nks * c + kTile;
-        if (whole < 0 || t < whole) whole = t;
-        for (int l = 1; l <= 3 && tiles <= cluster_slots(l, sms) && nks >= (4 << l); ++l) {
-            const int64_t s = ((nks + (1 << l) - 1) >> l) * c + kTile + 1000 + 26 * bn;
-            if (cost < 0 || s < cost) {
-                cost = s;
-                best.log_parts = l;
-                best.bn = bn;
-            }
-        }
-    }
-    return cost >= 0 && 7 * cost < 6 * whole ? best : Split{};
-}
-
-// M tiles that the choice of a split counts: those of the whole call (a chunk of a
-// host-buffer product runs with the bits of the whole)
-inline int64_t call_m_tiles(const FwdParams &p, int64_t m_tiles)
-{
-    return p.N_call ? (p.N_call + 127) / 128 : m_tiles;
-}
-
 // reduction indices a stage copies: the stage depth, or for bf16 products with
-// fewer than 64 indices (one stage) and convolutions of fewer than 64 channels
-// (a stage per tap) that many rounded up to 16: narrower copies (no out-of-range
-// fill for three quarters of the box when R = 16) and one MMA per 16 indices
-// (measured on the MobileNetV2 pointwise layers of 16-32 input channels: 20-35 %
-// faster)
+// fewer than 64 indices (one stage) the indices rounded up to 16: narrower copies
+// (no out-of-range fill for three quarters of the box when R = 16) and one MMA per
+// 16 indices (measured on the MobileNetV2 pointwise layers of 16-32 input channels:
+// 20-35 % faster)
 inline int stage_k_in(const FwdParams &p, bool tf32, int asrc, bool pk)
 {
     if (tf32) return 32;
-    const int64_t k = asrc == kATap ? p.Cin : p.R;
-    if (pk || (asrc != kA2d && asrc != kATap) || k >= 64) return 64;
-    return static_cast<int>((k + 15) / 16 * 16);
+    if (pk || asrc != kA2d || p.R >= 64) return 64;
+    return static_cast<int>((p.R + 15) / 16 * 16);
 }
 
-// bf16 stages of a tile
-inline int64_t stages_of(const FwdParams &p, int asrc)
+template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false>
+cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &tmA, cudaStream_t stream)
 {
-    return is_box(asrc) ? static_cast<int64_t>(p.KH) * p.KW * ((p.Cin + 63) / 64) : (p.R + 63) / 64;
-}
-
-// log_split: SK only, the CTAs of a tile (1 << log_split)
-template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false, bool SK = false>
-cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &tmA, cudaStream_t stream,
-                       int log_split = 0)
-{
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
-    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK, MC, SK>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
+    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK, MC>;
     ConvBox box = box_in;
     size_t smem = C::kSmem;
     if constexpr (C::kHalo) {
@@ -2207,16 +1830,10 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     const int elem = TF32 ? 4 : 2;
     const int64_t wdims[2] = {p.R, p.Cout};
     FwdParams q = p;
-    // narrower stage copies only in the short-tile form (one-stage products land there)
-    // and for convolutions
-    q.kin = EPI == 2 || C::kTapChunks ? stage_k_in(p, TF32, ASRC, PK) : C::kKS;
+    // narrower stage copies only in the short-tile form (one-stage layers land there)
+    q.kin = EPI == 2 ? stage_k_in(p, TF32, ASRC, PK) : C::kKS;
     const int wbox[2] = {q.kin, MC ? C::kBRows / 2 : C::kBRows};  // MC: each CTA copies half the rows
-    if constexpr (C::kTapChunks) {
-        // [co][tap][ci]: a box past the last channel of a tap is filled with zeros
-        const int64_t dims3[3] = {p.Cin, static_cast<int64_t>(p.KH) * p.KW, p.Cout};
-        const int box3[3] = {q.kin, 1, C::kBRows};
-        if (!make_map(&tmB0, p.wdense, dt, elem, 3, dims3, box3)) return cudaErrorInvalidValue;
-    } else if (!PK && !make_map(&tmB0, p.wdense, dt, elem, 2, wdims, wbox)) return cudaErrorInvalidValue;
+    if (!PK && !make_map(&tmB0, p.wdense, dt, elem, 2, wdims, wbox)) return cudaErrorInvalidValue;
     if (!PK && C::kBPlanes > 1) {
         // fp32: plane 1 of the split, bf16 [Cout][ceil(R / 32) * 64], one 128-byte row per stage
         const char *pl1 = static_cast<const char *>(p.wdense) + static_cast<size_t>(p.Cout) * p.R * elem;
@@ -2227,7 +1844,7 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     // output rows of 128 bytes: 32 fp32 or 64 bf16 channels
     const CUtensorMapDataType ydt = p.out_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const int yel = p.out_bf16 ? 2 : 4, ysc = p.out_bf16 ? 64 : 32;
-    if constexpr (is_box(ASRC) || ASRC == kAHalo) {
+    if constexpr (ASRC == kA4d || ASRC == kAHalo) {
         const int64_t dims[4] = {p.Cout, p.Q, p.P, box.B};
         const int bx[4] = {ysc, box.QB, box.PB, box.BB};
         if (!make_map(&tmY, p.Y, ydt, yel, 4, dims, bx)) return cudaErrorInvalidValue;
@@ -2239,24 +1856,14 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     const int64_t n_ct = (p.Cout + C::kN - 1) / C::kN;
     if constexpr (C::kHalo && !PK && CG == 1)  // resident weights: single-CTA tiles
         box.resident = (n_ct == 1 && (p.R + C::kKS - 1) / C::kKS <= C::kStages) ? 1 : 0;
-    const int64_t m_tiles = (is_box(ASRC) || ASRC == kAHalo)
+    const int64_t m_tiles = (ASRC == kA4d || ASRC == kAHalo)
                                 ? static_cast<int64_t>(box.nQ) * box.nP * ((box.B + box.BB - 1) / box.BB)
                                          : (p.N + C::kM - 1) / C::kM;
     // CG = 2 or MC: units are pair tiles (two M tiles), one per cluster of two CTAs
     constexpr int kCl = C::kPairUnits ? 2 : 1;
     const int64_t n_tiles = n_ct * (kCl == 2 ? (m_tiles + 1) / 2 : m_tiles);
-    if (n_tiles >= (int64_t(1) << 30)) return cudaErrorInvalidValue;  // unit numbers are 32-bit, with the grid added
-    box.byQ = TileDiv(box.nQ);
-    box.byP = TileDiv(box.nP);
-    box.byN = TileDiv(n_ct);
-    if constexpr (ASRC == kAGather) {  // (products: one tap of Cin = R channels)
-        box.byC = TileDiv(p.Cin);
-        box.byKW = TileDiv(p.KW);
-    }
-    const int64_t slots = C::kRes ? resident_slots(n_ct) : sm_count() / kCl;
-    if (C::kRes && ((p.R + 63) / 64 > C::kResB || slots == 0)) return cudaErrorInvalidValue;
-    box.log_split = log_split;
-    const int64_t grid = SK ? n_tiles << log_split : kCl * (n_tiles < slots ? n_tiles : slots);
+    const int64_t slots = sm_count() / kCl;
+    const int64_t grid = kCl * (n_tiles < slots ? n_tiles : slots);
     // programmatic dependent launch: may start once every block of the preceding
     // kernel on the stream (the decompression) has signalled; it waits for that
     // kernel's completion before reading memory
@@ -2269,13 +1876,12 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     la[0].val.programmaticStreamSerializationAllowed = 1;
     la[1].id = cudaLaunchAttributeClusterDimension;
-    la[1].val.clusterDim.x = SK ? 1u << log_split : kCl;
+    la[1].val.clusterDim.x = kCl;
     la[1].val.clusterDim.y = 1;
     la[1].val.clusterDim.z = 1;
     cfg.attrs = la;
-    cfg.numAttrs = kCl == 2 || SK ? 2 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box,
-                                             static_cast<int>(n_tiles));
+    cfg.numAttrs = kCl == 2 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box, n_ct, n_tiles);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -2285,18 +1891,20 @@ struct Plan {
     int asrc;
     ConvBox box;
     AMaps am;
-    ConvBox a4d;  // the pixel box that halo copies were taken instead of
 };
 // halo box of a bf16 3x3, stride-1, padding-1 convolution: PB output rows of
-// the full width per tile.  Used for layers of min_cin input channels or more
-// (the per-tap copies there move 9 x the halo's bytes), and for 64 -> 64 layers,
-// whose nine weight tiles stay resident in the stages (no per-tap weight copies
-// either), whose output rows per tile are at least three quarters of the 4-D
-// box's (images narrower than the tile fit several per 4-D box, not per halo)
-inline bool halo_box(const FwdParams &p, const ConvBox &a4d, int64_t min_cin, ConvBox *hb)
+// the full width per tile.  Used for layers of 256 input channels or more (four
+// chunks or more per tile: the per-tap copies there move 9 x the halo's bytes,
+// and the halo copies measured 7-11 % faster on the 14 x 14 ResNet-50 layers;
+// with 64 or 128 channels the tile is bound by the MMAs' shared-memory reads
+// and the per-tap form measured faster), and for 64 -> 64 layers, whose nine
+// weight tiles stay resident in the stages (no per-tap weight copies either),
+// whose output rows per tile are at least three quarters of the 4-D box's
+// (images narrower than the tile fit several per 4-D box, not per halo)
+inline bool halo_box(const FwdParams &p, const ConvBox &a4d, ConvBox *hb)
 {
     if (!(p.is_conv && p.KH == 3 && p.KW == 3 && p.sh == 1 && p.sw == 1 && p.ph == 1 && p.pw == 1 &&
-          p.Cin % 64 == 0 && (p.Cin >= min_cin || (p.Cin == 64 && p.Cout <= 64)) && p.P == p.H && p.Q == p.W &&
+          p.Cin % 64 == 0 && (p.Cin >= 256 || (p.Cin == 64 && p.Cout <= 64)) && p.P == p.H && p.Q == p.W &&
           p.Q + 2 <= 66))
         return false;
     const int wq = static_cast<int>(p.Q) + 2;
@@ -2310,19 +1918,13 @@ inline bool halo_box(const FwdParams &p, const ConvBox &a4d, int64_t min_cin, Co
     return true;
 }
 
-// halo copies from 128 input channels on: over CTA pairs with 128-wide N tiles
-// they measured faster than the per-tap copies (128 -> 128 at 28 x 28, 64 images
-// 18.8 -> 16.6 us a pass, 128 images 29.1 -> 24.3 us).  The fused family, whose
-// producers bound it, takes them from 256 on.
-// halo_cin < 0: no halo copies
-inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t halo_cin = 128, bool pk = false)
+inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl)
 {
-    pl->asrc = a_source(p, ks, !tf32 && !pk);
+    pl->asrc = a_source(p, ks);
     pl->box = ConvBox{1, 1, 1, 1, 1, 1, 1};
-    if (is_box(pl->asrc)) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
-    pl->a4d = pl->box;
+    if (pl->asrc == kA4d) pl->box = choose_box(p.N / (p.P * p.Q), p.P, p.Q);
     ConvBox hb;
-    if (pl->asrc == kA4d && !tf32 && halo_cin >= 0 && halo_box(p, pl->box, halo_cin, &hb)) {
+    if (pl->asrc == kA4d && !tf32 && halo_box(p, pl->box, &hb)) {
         pl->asrc = kAHalo;
         pl->box = hb;
     }
@@ -2335,7 +1937,7 @@ inline void plan_layer(const FwdParams &p, bool tf32, int ks, Plan *pl, int64_t 
 // m tiles of the layer for the chosen activation source
 inline int64_t m_tiles_of(const FwdParams &p, int asrc, const ConvBox &box)
 {
-    if (is_box(asrc) || asrc == kAHalo)
+    if (asrc == kA4d || asrc == kAHalo)
         return static_cast<int64_t>(box.nQ) * box.nP * ((box.B + box.BB - 1) / box.BB);
     return (p.N + 127) / 128;
 }

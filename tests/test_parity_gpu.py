@@ -786,81 +786,6 @@ def test_halo_conv3x3_pair_tiles_ragged(dev):
         assert_within_tol(f64(Y[b]).reshape(-1, Cout), Yo, S, f"ragged halo pair conv image {b}")
 
 
-# halo copies over CTA pairs with 128-wide N tiles from 128 input channels on: one
-# row block per image (an odd count, a pair without a second tile), ragged last
-# row blocks and N tiles, a single row block (which runs 64-wide single tiles)
-@pytest.mark.parametrize("B,H,Wi,Cin,Cout", [(3, 28, 28, 128, 128), (5, 9, 9, 128, 72), (2, 13, 17, 192, 264),
-                                             (1, 4, 30, 128, 128)])
-def test_halo_conv3x3_pairs_from_128_channels(dev, B, H, Wi, Cin, Cout):
-    G, K = 8, 2
-    g = torch.Generator().manual_seed(B * 31 + H + Cin + Cout)
-    X = torch.randn((B, H, Wi, Cin), generator=g).clamp_min(0).to(BF16)
-    W = torch.randn((Cout, 9 * Cin), generator=g).to(BF16)
-    Y = run_conv(dev, X, W, (3, 3, (1, 1), (1, 1), Cout), G, K, cci.ALGO_DENSE_TC_WS)
-    _, _, Wd, mask = oracle_reference(W, G, K)
-    Yo, S = oracle.conv2d(f64(X), Wd, mask, 3, 3, (1, 1), (1, 1))
-    assert_within_tol(f64(Y).reshape(-1, Cout), Yo, S, f"halo pairs B={B} {H}x{Wi} {Cin}->{Cout}")
-
-
-# short tiles (1 to 4 stages) with resident weights: more tiles than SMs, so every
-# CTA runs several tiles of its N tile; 1, 2, 3 and 5 N tiles (152, 152, 150 and 150
-# CTAs), ones that leave too few whole rounds (100 and 22 N tiles: the form without,
-# whose copies are whole stages also for fewer than 64 indices), one tile per CTA of
-# such a layer, a ragged last M tile, fewer indices than a chunk, a ragged last chunk
-@pytest.mark.parametrize("N,Cin,Cout,G,K", [(20005, 16, 96, 8, 2), (10011, 128, 512, 8, 2), (6500, 72, 520, 8, 2),
-                                            (4200, 256, 640, 16, 4), (20100, 200, 64, 4, 1), (260, 64, 25600, 8, 2),
-                                            (3000, 24, 5600, 8, 2), (150, 16, 1360, 8, 1)])
-def test_short_tiles_resident_weights(dev, N, Cin, Cout, G, K):
-    X, W = wl.random_small(N + Cin, "bf16", N, Cin, Cout)
-    v, i = cci.pack(W.to(dev), G, K)
-    st = cci.new_status(dev)
-    Y = cci.linear(X.to(dev), v, i, Cout, G, K, status=st)
-    assert cci.read_status(st) == 0 and torch.isfinite(Y).all()
-    rows = sample_rows(N, 200, seed=N)
-    _, _, Wd, mask = oracle_reference(W, G, K)
-    Yo, S = oracle.linear(f64(X[rows]), Wd, mask)
-    assert_within_tol(f64(Y[torch.from_numpy(rows).to(dev)]), Yo, S, f"resident weights {N} x {Cin} -> {Cout}")
-
-
-# bf16 convolutions whose channel count is no multiple of the 64-deep stage: boxes
-# per tap, the last chunk filled past Cin in both operands.  Fewer channels than
-# one MMA (8), than a stage (24, 40), a ragged last chunk (72, 104, 152); both
-# strides, even kernels without padding, ragged N tiles, pair tiles (160 channels
-# into 512, 27 stages); weights and images with an infinity, whose column must not
-# spread into a neighbouring tap's padding.
-CONV_TAP = [(2, 9, 9, 8, 64, 3, 1, 1), (3, 14, 10, 24, 48, 3, 1, 1), (2, 11, 13, 40, 136, 3, 2, 1),
-            (1, 17, 9, 72, 96, 5, 1, 2), (2, 12, 12, 104, 64, 2, 2, 0), (4, 10, 10, 152, 264, 1, 2, 0),
-            (40, 28, 28, 160, 512, 3, 2, 1)]
-
-
-@pytest.mark.parametrize("B,H,Wi,Cin,Cout,k,stride,pad", CONV_TAP)
-def test_conv_ragged_channels(dev, B, H, Wi, Cin, Cout, k, stride, pad):
-    G, K = 8, 2
-    g = torch.Generator().manual_seed(B + H + Cin + Cout + k)
-    X = torch.randn((B, H, Wi, Cin), generator=g).clamp_min(0).to(BF16)
-    W = torch.randn((Cout, k * k * Cin), generator=g).to(BF16)
-    Y = run_conv(dev, X, W, (k, k, (stride, stride), (pad, pad), Cout), G, K, cci.ALGO_DENSE_TC_WS)
-    assert torch.isfinite(Y).all()
-    _, _, Wd, mask = oracle_reference(W, G, K)
-    for b in {0, B - 1}:
-        Yo, S = oracle.conv2d(f64(X[b:b + 1]), Wd, mask, k, k, (stride, stride), (pad, pad))
-        assert_within_tol(f64(Y[b]).reshape(-1, Cout), Yo, S, f"ragged channels, image {b}")
-
-
-def test_conv_ragged_channels_keep_infinities_in_their_tap(dev):
-    """An infinite weight of tap (1, 1) makes infinities where its input is not
-    zero and NaN where it is, and leaves every other output channel alone."""
-    B, H, Cin, Cout, G, K = 1, 6, 24, 64, 8, 2
-    g = torch.Generator().manual_seed(5)
-    X = (torch.rand((B, H, H, Cin), generator=g) + 0.5).to(BF16)
-    W = torch.randn((Cout, 9, Cin), generator=g).to(BF16)
-    W[3, 4, 23] = float("inf")
-    Y = run_conv(dev, X, W.view(Cout, -1), (3, 3, (1, 1), (1, 1), Cout), G, K, cci.ALGO_DENSE_TC_WS)
-    assert torch.isinf(Y[..., 3]).all() and (Y[..., 3] > 0).all()
-    others = [c for c in range(Cout) if c != 3]
-    assert torch.isfinite(Y[..., others]).all()
-
-
 # ---------------------------------------------------------------------------
 # CTA-pair tiles (tcgen05 cta_group::2): bf16 layers with at least 16 stages of
 # 64 reduction indices and 256-wide N tiles run as 256-row tiles split over two
@@ -879,8 +804,7 @@ def test_pair_tiles_product(dev, N, Cin, Cout, G, K):
     assert_within_tol(f64(Y[torch.from_numpy(rows).to(dev)]), Yo, S, f"pair product {N}x{Cin}->{Cout}")
 
 
-@pytest.mark.parametrize("B,H,Cin,Cout,stride", [(63, 14, 128, 256, 1), (64, 28, 128, 256, 2), (301, 14, 128, 128, 1),
-                                                 (401, 14, 128, 200, 2)])
+@pytest.mark.parametrize("B,H,Cin,Cout,stride", [(63, 14, 128, 256, 1), (64, 28, 128, 256, 2)])
 def test_pair_tiles_conv(dev, B, H, Cin, Cout, stride):
     G, K = 8, 2
     g = torch.Generator().manual_seed(B * 31 + H)
