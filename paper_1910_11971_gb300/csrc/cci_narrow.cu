@@ -28,13 +28,13 @@
 // into chunks of columns gives the same bits as the whole.
 //
 // Where the rule lies (device time per pass against decompression and GEMM): 16 x
-// 4096 -> 4096 9.8 us against 16.8, 100 x 2048 -> 1000 7.6 against 9.3, 100 x 1024
-// -> 4096 7.5 against 8.1, 32 x 4096 -> 1024 at G = 32, K = 8 7.1 against 16.6; up to
-// seven stages in one part it is even with them (25 x 432 -> 992 5.6 against 5.4, 7 x
-// 16 -> 1360 3.6 against 4.4) and saves the second launch, some 3 us of host time a
-// call; eight or nine stages are too few to split and take 8.0 against 6.0 (128 x
-// 512 -> 512), so those stay there.  At 128 columns 4096 -> 4096 takes 13.1 against
-// about 18; more would need smaller stages.
+// 4096 -> 4096 9.4 us against 23.5, 100 x 2048 -> 1000 7.2 against 12.2, 100 x 1024
+// -> 4096 7.0 against 9.4, 32 x 4096 -> 1024 at G = 32, K = 8 6.3 against 23.6; up to
+// seven stages in one part it is even with them (25 x 432 -> 992 5.9 against 5.8, 7 x
+// 16 -> 1360 3.6 against 4.3) and saves the second launch, some 3 us of host time a
+// call; eight or nine stages are too few to split and take 7.7 against 6.2 (128 x
+// 512 -> 512) and 8.0 against 6.3 (64 x 576 -> 1024), so those stay there.  At 128
+// columns 4096 -> 4096 takes 12.5 against 23.7; more would need smaller stages.
 #include "cci_gemm_ws.cuh"
 
 namespace cci {
