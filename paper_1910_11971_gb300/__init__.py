@@ -121,7 +121,10 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _stream(device: torch.device) -> int:
-    # the handle alone: a Stream object for it costs 2 us a call
+    # the handle alone: a Stream object for it costs 2 us a call.  A tensor that is not
+    # on the GPU is refused here: its address must not reach a kernel
+    if device.type != "cuda":
+        raise ValueError(f"Expected a cuda device, but got: {device}")
     index = device.index
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 

@@ -4,8 +4,10 @@ status before anything is enqueued (these paths never touch the device)."""
 import ctypes
 import os
 import re
+from types import SimpleNamespace
 
 import pytest
+import torch
 
 import paper_1910_11971_gb300 as cci
 from paper_1910_11971_gb300 import build as cci_build
@@ -255,3 +257,25 @@ def test_bbs_rejects(lib):
     assert f(FAKE, 1, 16, 64, FAKE, FAKE, 16, 8, 2, FAKE, None, 2, None, 0, None) == UNSUP  # no such family
     assert f(FAKE, 1, 16, 64, FAKE, FAKE, 16, 8, 2, FAKE, None, 5, None, 0, None) == 11     # workspace
     assert f(FAKE, 1, 0, 64, FAKE, FAKE, 16, 8, 2, None, None, 1, None, 0, None) == OK      # empty
+
+
+def test_tensors_off_the_gpu_never_reach_a_kernel(monkeypatch):
+    """The calls that take the stream from a tensor's device refuse a host tensor before
+    they enter the library (a fake one here, which records any entry)."""
+    entered = []
+
+    class Fake:
+        def __getattr__(self, name):
+            return lambda *a: entered.append(name) or 0
+
+    monkeypatch.setattr(cci, "lib", lambda: Fake())
+    monkeypatch.setattr(cci, "_copy_streams", {0: (SimpleNamespace(cuda_stream=0),) * 2})
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda index: 0, raising=False)
+    with pytest.raises(ValueError):
+        cci.fma_probe(torch.empty(32), 1, 32, 1)
+    v, i = torch.zeros((8, 64, 2)), torch.zeros((8, 64, 2), dtype=torch.uint8)
+    with pytest.raises(ValueError):
+        cci.linear_host(torch.zeros((4, 64)), v, i, 64, 8, 2, out=torch.zeros((4, 64)), chunk=4,
+                        buffer=torch.zeros(1 << 16, dtype=torch.uint8))
+    assert entered == []
