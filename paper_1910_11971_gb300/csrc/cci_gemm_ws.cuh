@@ -106,21 +106,13 @@ struct AMaps {
 // EPI = 2: a second epilogue group (warps 4-7, idle when bf16 activations are
 // copied by TMA) and two staging buffers per group, for layers whose tiles have
 // few stages (the output write dominates); EPI = 1: one group, more stages
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false>
 struct Cfg {
     static constexpr int kM = 128, kN = BN;
     static_assert(CG == 1 || (CG == 2 && !TF32 && ASRC != kAGather), "pair mode: bf16 with TMA activations");
     static_assert(!PK || (!TF32 && ASRC != kAGather && EPI == 1 && (BN / CG) <= 128),
                   "packed weights: bf16, TMA activations, producers busy, one item per producer");
     static constexpr int kBRows = kN / CG;  // B rows held by one CTA
-    // MC: a cluster of two CTAs takes adjacent M tiles of the same N tile; each
-    // copies half of the B rows of a stage with multicast into both, and each
-    // CTA's MMAs release the stage in both (TMA activations, 2-D or 4-D)
-    static_assert(!MC || (ASRC != kAGather && ASRC != kAHalo && CG == 1 && EPI == 1 && !PK),
-                  "weight multicast: single-CTA TMA tiles with one epilogue group");
-    // (used for fp32 layers: measured on the bf16 3x3 convolutions it did not pay,
-    // conv3x3_28 0.0273 -> 0.0283 ms, the ResNet-50 stack unchanged)
-    static constexpr bool kPairUnits = CG == 2 || MC;  // units of two M tiles over a cluster of two
     static constexpr int kKS = TF32 ? 32 : 64;  // r per stage: one 128-byte row
     static constexpr bool kATma = !TF32 && ASRC != kAGather;  // A copied by TMA into its plane
     static constexpr bool kHalo = ASRC == kAHalo;  // A: per-chunk halo buffers, stages hold B only
@@ -220,8 +212,7 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
 // formed by adds: the MMA warp's instruction stream per stage bounds this
 // product (measured on GB300 with clock stamps for the three-pass form of twelve
 // MMAs: operands waited for ~130 cycles per stage, the issue of a stage took ~850).
-// kMC: the commit arrives on the barrier at this offset in both CTAs of the cluster.
-template <uint32_t kIdescT, uint32_t kIdescB, uint32_t kB1, bool kMC = false>
+template <uint32_t kIdescT, uint32_t kIdescB, uint32_t kB1>
 __device__ __forceinline__ void stage_tf32_split(uint32_t d, uint32_t a0, uint64_t b0, uint32_t acc0, uint32_t issue,
                                                  uint32_t bar)
 {
@@ -246,18 +237,11 @@ __device__ __forceinline__ void stage_tf32_split(uint32_t d, uint32_t a0, uint64
         "r"(a0), "l"(b0), "r"(acc0), "r"(issue), "n"(kIdescT), "n"(kIdescB),
         "n"(static_cast<uint64_t>(kB1 + 4)), "n"(static_cast<uint64_t>(kB1))
         : "memory");
-    if constexpr (kMC)
-        asm volatile(
-            "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
-            "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %2;\n}\n" ::"r"(bar),
-            "r"(issue), "h"(static_cast<uint16_t>(3))
-            : "memory");
-    else
-        asm volatile(
-            "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
-            "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
-            "r"(issue)
-            : "memory");
+    asm volatile(
+        "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
+        "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(issue)
+        : "memory");
 }
 
 // ---- one pipeline stage of bf16 MMAs ----
@@ -269,7 +253,7 @@ __device__ __forceinline__ void stage_tf32_split(uint32_t d, uint32_t a0, uint64
 // 64-wide N tile stage is 192 tensor cycles, and the issue path was 400-700).
 // kCounted: only the first n16 (1-4) MMAs of the stage, 16 reduction indices each
 // (a one-stage layer copying fewer than 64 indices); else all four
-template <uint32_t kIdesc, bool kMC = false, bool kCounted = false>
+template <uint32_t kIdesc, bool kCounted = false>
 __device__ __forceinline__ void stage_f16(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t acc0, uint32_t issue,
                                           uint32_t bar, uint32_t n16 = 4)
 {
@@ -300,19 +284,11 @@ __device__ __forceinline__ void stage_f16(uint32_t d, uint64_t adesc, uint64_t b
             "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %5, pt;\n}\n" ::"r"(d),
             "l"(adesc), "l"(bdesc), "r"(acc0), "r"(issue), "n"(kIdesc)
             : "memory");
-    // kMC: the commit arrives on the barrier at this offset in both CTAs of the cluster
-    if constexpr (kMC)
-        asm volatile(
-            "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
-            "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %2;\n}\n" ::"r"(bar),
-            "r"(issue), "h"(static_cast<uint16_t>(3))
-            : "memory");
-    else
-        asm volatile(
-            "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
-            "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
-            "r"(issue)
-            : "memory");
+    asm volatile(
+        "{\n.reg .pred pe;\nsetp.ne.b32 pe, %1, 0;\n"
+        "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(issue)
+        : "memory");
 }
 
 // ---- one kernel row of a 3x3 halo tile with resident weights ----
@@ -448,17 +424,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *tmap,
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
         "{%2, %3}], [%4];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
-// 2-D tile copy into the same shared-memory offset of both CTAs of a cluster of
-// two, completing on the barrier at the same offset in each
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const void *tmap, int x, int y, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-        "{%2, %3}], [%4], %5;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(bar), "h"(static_cast<uint16_t>(3))
         : "memory");
 }
 
@@ -762,13 +727,13 @@ __device__ __forceinline__ BoxIdx box_of(int64_t mt, const ConvBox &box)
 
 // PK: tmB0 / tmB1 are the maps of the packed values and indices (2-D over
 // [Cout/G][R*K]); otherwise the maps of the workspace planes
-template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false, bool MC = false>
-__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads, 1)
+template <bool TF32, int ASRC, int BN, int CG, int EPI, bool PK = false>
+__global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK>::kThreads, 1)
     gemm_ws_kernel(FwdParams p, const __grid_constant__ AMaps tmA, const __grid_constant__ CUtensorMap tmB0,
                    const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmY, ConvBox box,
                    int64_t n_ct, int64_t n_tiles)
 {
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK>;
     constexpr int kM = C::kM, kN = C::kN, kKS = C::kKS, kStages = C::kStages;
     constexpr int kLag = 2;  // bf16 gather: stages in flight before a producer's arrive
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -784,16 +749,16 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     volatile int *abort = &S->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nks = static_cast<int>((p.R + kKS - 1) / kKS);
-    const uint32_t crank = C::kPairUnits ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
+    const uint32_t crank = CG == 2 ? cluster_rank() : 0u;  // CG = 2: 0 issues the pair's MMAs
     // work units: tiles (CG = 1) or pair tiles of 2 x 128 rows (CG = 2), strided over
     // the CTAs (CG = 1) or the CTA pairs (CG = 2)
-    const int64_t u0 = C::kPairUnits ? blockIdx.x / 2 : blockIdx.x;
-    const int64_t ustep = C::kPairUnits ? gridDim.x / 2 : gridDim.x;
+    const int64_t u0 = CG == 2 ? blockIdx.x / 2 : blockIdx.x;
+    const int64_t ustep = CG == 2 ? gridDim.x / 2 : gridDim.x;
     // unit u -> (M tile, N tile): one 64-bit division, the remainder by multiply-subtract
     auto split_unit = [&](int64_t u, int64_t &mt, int64_t &ct) {
         const int64_t q = u / n_ct;
         ct = u - q * n_ct;
-        mt = C::kPairUnits ? 2 * q + crank : q;
+        mt = CG == 2 ? 2 * q + crank : q;
     };
 
     if (tid == 0) {
@@ -804,7 +769,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
         const uint32_t full_count = PK ? (C::kHalo ? 0u : 1u) + 4 * CG : (C::kATma ? 1u : 129u);
         for (int s = 0; s < kStages; ++s) {
             tc::mbar_init(&S->full[s], full_count);
-            tc::mbar_init(&S->empty[s], MC ? 2 : 1);  // MC: released by both CTAs' MMAs
+            tc::mbar_init(&S->empty[s], 1);
             tc::mbar_init(&S->aux[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
@@ -853,7 +818,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     // the pair's barriers are initialised before either CTA signals the other's
-    if constexpr (C::kPairUnits) cluster_sync();
+    if constexpr (CG == 2) cluster_sync();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S->tmem_base;
     // launched as a programmatic dependent of the decompression: everything above
@@ -972,19 +937,9 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         tc::mbar_arrive_expect_tx(&S->full[s], a_bytes);
                     } else {
                         tc::mbar_arrive_expect_tx(&S->full[s], b_bytes + (C::kATma ? a_bytes : 0u));
-                        if constexpr (MC) {
-                            // this CTA's half of the B rows into both CTAs (the same offsets);
-                            // each CTA's full barrier expects the whole tile
-                            const uint32_t half = crank * (C::kBPlane / 2);
-                            const int y = static_cast<int>(co0) + static_cast<int>(crank) * (kN / 2);
-                            tma_load_2d_mc(bst + half, &tmB0, ks * kKS, y, tc::smem_u32(&S->full[s]));
-                            if constexpr (C::kBPlanes > 1)
-                                tma_load_2d_mc(bst + C::kBPlane + half, &tmB1, ks * 64, y, tc::smem_u32(&S->full[s]));
-                        } else {
-                            tc::tma_load_2d(bst, &tmB0, ks * kKS, static_cast<int>(co0), &S->full[s]);
-                            if constexpr (C::kBPlanes > 1)  // fp32 plane 1: 64 bf16 per stage
-                                tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, static_cast<int>(co0), &S->full[s]);
-                        }
+                        tc::tma_load_2d(bst, &tmB0, ks * kKS, static_cast<int>(co0), &S->full[s]);
+                        if constexpr (C::kBPlanes > 1)  // fp32 plane 1: 64 bf16 per stage
+                            tc::tma_load_2d(bst + C::kBPlane, &tmB1, ks * 64, static_cast<int>(co0), &S->full[s]);
                     }
                     if constexpr (ASRC == kA2d) {
                         tc::tma_load_2d(st, &tmA.m[0], ks * kKS, static_cast<int>(mt * kM), abar);
@@ -1334,7 +1289,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                         ok = tc::mbar_wait(&S->full[s], (it / kStages) & 1, abort, p.status);
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        stage_tf32_split<C::kIdesc, C::kIdescB, (C::kBPlane >> 4), MC>(
+                        stage_tf32_split<C::kIdesc, C::kIdescB, (C::kBPlane >> 4)>(
                             d, tmem + static_cast<uint32_t>(C::kAColBase + s * 64),
                             bdesc0 + static_cast<uint64_t>(s) * (C::kStage >> 4) + (C::kBOff >> 4), ks > 0 ? 1u : 0u,
                             1u, empty0 + 8u * s);
@@ -1370,10 +1325,10 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
                             stage_f16_pair<C::kIdesc>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, empty0 + 8u * s);
                         else
                             if constexpr (EPI == 2)  // short tiles: fewer than four MMAs when R < 64
-                                stage_f16<C::kIdesc, MC, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u,
-                                                               empty0 + 8u * s, n16);
+                                stage_f16<C::kIdesc, true>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u,
+                                                           empty0 + 8u * s, n16);
                             else
-                                stage_f16<C::kIdesc, MC>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
+                                stage_f16<C::kIdesc>(d, ad, ad + bunits, ks > 0 ? 1u : 0u, 1u, empty0 + 8u * s);
                         if (++s == kStages) {
                             s = 0;
                             ph ^= 1u;
@@ -1604,7 +1559,7 @@ __global__ void __launch_bounds__(Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>::kThreads
     __syncthreads();
     // CG = 2: neither CTA leaves (or frees tensor memory) while the other may still
     // signal its barriers or the pair's MMAs may read its shared memory
-    if constexpr (C::kPairUnits) cluster_sync();
+    if constexpr (CG == 2) cluster_sync();
     if (warp == 8) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if constexpr (CG == 2)
@@ -1806,11 +1761,11 @@ inline int stage_k_in(const FwdParams &p, bool tf32, int asrc, bool pk)
     return static_cast<int>((p.R + 15) / 16 * 16);
 }
 
-template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false, bool MC = false>
+template <bool TF32, int ASRC, int BN, int CG, int EPI = 1, bool PK = false>
 cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &tmA, cudaStream_t stream)
 {
-    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK, MC>;
-    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK, MC>;
+    using C = Cfg<TF32, ASRC, BN, CG, EPI, PK>;
+    auto kern = gemm_ws_kernel<TF32, ASRC, BN, CG, EPI, PK>;
     ConvBox box = box_in;
     size_t smem = C::kSmem;
     if constexpr (C::kHalo) {
@@ -1832,13 +1787,13 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     FwdParams q = p;
     // narrower stage copies only in the short-tile form (one-stage layers land there)
     q.kin = EPI == 2 ? stage_k_in(p, TF32, ASRC, PK) : C::kKS;
-    const int wbox[2] = {q.kin, MC ? C::kBRows / 2 : C::kBRows};  // MC: each CTA copies half the rows
+    const int wbox[2] = {q.kin, C::kBRows};
     if (!PK && !make_map(&tmB0, p.wdense, dt, elem, 2, wdims, wbox)) return cudaErrorInvalidValue;
     if (!PK && C::kBPlanes > 1) {
         // fp32: plane 1 of the split, bf16 [Cout][ceil(R / 32) * 64], one 128-byte row per stage
         const char *pl1 = static_cast<const char *>(p.wdense) + static_cast<size_t>(p.Cout) * p.R * elem;
         const int64_t dims1[2] = {(p.R + 31) / 32 * 64, p.Cout};
-        const int box1[2] = {64, MC ? C::kBRows / 2 : C::kBRows};
+        const int box1[2] = {64, C::kBRows};
         if (!make_map(&tmB1, pl1, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 2, dims1, box1)) return cudaErrorInvalidValue;
     }
     // output rows of 128 bytes: 32 fp32 or 64 bf16 channels
@@ -1859,11 +1814,10 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     const int64_t m_tiles = (ASRC == kA4d || ASRC == kAHalo)
                                 ? static_cast<int64_t>(box.nQ) * box.nP * ((box.B + box.BB - 1) / box.BB)
                                          : (p.N + C::kM - 1) / C::kM;
-    // CG = 2 or MC: units are pair tiles (two M tiles), one per cluster of two CTAs
-    constexpr int kCl = C::kPairUnits ? 2 : 1;
-    const int64_t n_tiles = n_ct * (kCl == 2 ? (m_tiles + 1) / 2 : m_tiles);
-    const int64_t slots = sm_count() / kCl;
-    const int64_t grid = kCl * (n_tiles < slots ? n_tiles : slots);
+    // CG = 2: units are pair tiles (two M tiles), one per cluster of two CTAs
+    const int64_t n_tiles = n_ct * (CG == 2 ? (m_tiles + 1) / 2 : m_tiles);
+    const int64_t slots = sm_count() / CG;
+    const int64_t grid = CG * (n_tiles < slots ? n_tiles : slots);
     // programmatic dependent launch: may start once every block of the preceding
     // kernel on the stream (the decompression) has signalled; it waits for that
     // kernel's completion before reading memory
@@ -1876,11 +1830,11 @@ cudaError_t launch_cfg(const FwdParams &p, const ConvBox &box_in, const AMaps &t
     la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     la[0].val.programmaticStreamSerializationAllowed = 1;
     la[1].id = cudaLaunchAttributeClusterDimension;
-    la[1].val.clusterDim.x = kCl;
+    la[1].val.clusterDim.x = CG;
     la[1].val.clusterDim.y = 1;
     la[1].val.clusterDim.z = 1;
     cfg.attrs = la;
-    cfg.numAttrs = kCl == 2 ? 2 : 1;
+    cfg.numAttrs = CG == 2 ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, tmA, tmB0, tmB1, tmY, box, n_ct, n_tiles);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

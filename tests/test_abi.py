@@ -279,3 +279,13 @@ def test_tensors_off_the_gpu_never_reach_a_kernel(monkeypatch):
         cci.linear_host(torch.zeros((4, 64)), v, i, 64, 8, 2, out=torch.zeros((4, 64)), chunk=4,
                         buffer=torch.zeros(1 << 16, dtype=torch.uint8))
     assert entered == []
+
+
+def test_no_tile_copy_into_several_ctas():
+    """Every rank of a multi-GPU run loads this library, so no kernel in it copies a tile
+    into the CTAs of a cluster at once (commits to a CTA pair's barriers are no copies)."""
+    word = "multi" + "cast"
+    for name in sorted(os.listdir(os.path.dirname(cci.__file__) + "/csrc")):
+        text = open(os.path.join(os.path.dirname(cci.__file__), "csrc", name)).read()
+        copies = re.findall(r"cp\.async\.bulk[\w.:]*", text)
+        assert not [c for c in copies if word in c], name
