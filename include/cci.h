@@ -85,10 +85,14 @@ typedef enum cci_dtype {
 typedef enum cci_algo {
     CCI_ALGO_AUTO = 0,      /* the fastest family this build has for (G, K, dtype, shape): the
                                workspace tensor-core family when a large enough workspace is
-                               given (cci_linear_ws; its products of few columns need
-                               none); else the fused tensor-core family
+                               given (cci_linear_ws); else the fused tensor-core family
                                (CCI_ALGO_DENSE_TC) for bf16 layers that have it; else the
-                               CUDA-core families */
+                               CUDA-core families.  Most bf16 products of at most 128
+                               columns (K <= 8) run one launch instead of either tensor-core
+                               family: it expands the weights inside the product and
+                               neither reads nor writes the workspace.  Long reductions
+                               are summed there in up to eight parts, so a column's last
+                               bits may differ from those it has in a call of more columns */
     CCI_ALGO_GENERIC = 1,   /* generic kernel: any G <= 256, any K, any alignment */
     CCI_ALGO_REGTILE = 2,   /* register-tiled scatter on CUDA cores: Alg. 2 with the output
                                row chosen per (group, r) by a warp-uniform jump;
@@ -120,10 +124,7 @@ typedef enum cci_algo {
                                workspace: plane 0 [Cout][R] fp32 hi, then plane 1
                                [Cout][ceil(R/32)*64] bf16 (per 32-wide chunk of r, 32
                                bf16(hi(w)) then 32 bf16(lo(w))).  Cin % 4 == 0, R % 4 == 0.
-                               Needs cci_workspace_size() bytes.  Most bf16 products
-                               of at most 128 columns (K <= 8) expand the weights
-                               inside the product instead and leave the workspace as
-                               it is */
+                               Needs cci_workspace_size() bytes */
 } cci_algo;
 
 /*
@@ -211,10 +212,10 @@ size_t cci_workspace_size(cci_algo algo, cci_dtype dtype, int64_t Cout, int64_t 
 /*
  * As cci_linear_ex / cci_conv2d_ex with a caller workspace (device, 16-byte
  * aligned, `workspace_bytes` long; NULL / 0 allowed for families that need
- * none).  The call overwrites the workspace; calls that overlap on the GPU must
- * use different workspaces.  CCI_ALGO_AUTO uses the dense tensor-core family
- * when the layer has one and the workspace is large enough, else the CUDA-core
- * family.
+ * none).  The call overwrites the workspace (CCI_ALGO_AUTO may leave it as it
+ * is); calls that overlap on the GPU must use different workspaces.
+ * CCI_ALGO_AUTO uses the dense tensor-core family when the layer has one and the
+ * workspace is large enough, else the CUDA-core family.
  */
 cci_status cci_linear_ws(const void *X, cci_dtype dtype, int64_t N, int64_t Cin,
                          const void *values, const uint8_t *idx, int64_t Cout, int G, int K,
@@ -233,9 +234,10 @@ cci_status cci_conv2d_ws(const void *X, cci_dtype dtype, int64_t B, int64_t H, i
  * on the device).  The columns are processed in chunks of `chunk_cols`; chunk c
  * is copied in on `copy_in_stream`, multiplied on `stream` (the dense
  * tensor-core family AUTO picks: the fused one from the packed weights, else the
- * workspace one, the weights decompressed once by the first chunk) and copied
- * out on `copy_out_stream`, so that the copies of neighbouring chunks overlap
- * the product.  The result equals cci_linear_ws with CCI_ALGO_AUTO and a
+ * workspace one, the weights decompressed once by the first chunk, or for an N
+ * of few columns the one-launch product, which expands them in every chunk) and
+ * copied out on `copy_out_stream`, so that the copies of neighbouring chunks
+ * overlap the product.  The result equals cci_linear_ws with CCI_ALGO_AUTO and a
  * workspace on the same data bit for bit.
  *
  *   X_host, Y_host  host memory; page-locked (cudaHostAlloc / registered) for the
@@ -425,8 +427,8 @@ cci_status cci_dense_planes(const void *W, cci_dtype dtype, int64_t Cout, int64_
  *     stream capture.  The address is cached for the life of the process: after
  *     cudaDeviceReset() on that device the cached address is stale, so do not
  *     call this entry point again on a device that was reset;
- *   - every call shares the one array per device, which holds the dense weights of
- *     the last call that used it; each call rewrites the part it reads, so nothing
+ *   - every call shares the one array per device and leaves it holding the last
+ *     call's dense weights; each call rewrites the part it reads, so nothing
  *     needs clearing, but calls that overlap on the GPU (other streams, other
  *     threads) race on the array and must be serialised by the caller.
  * Errors: as cci_linear; CCI_ERR_UNSUPPORTED for shapes the dense kernel lacks;
@@ -442,7 +444,9 @@ cci_status cci_linear_dense_tc_static(const void *X, cci_dtype dtype, int64_t N,
  * Cin*KH*KW for a convolution, taken to have strides <= 2) when every pointer is
  * 16-byte aligned and, for CCI_ALGO_AUTO, the workspace is the one
  * cci_workspace_size(CCI_ALGO_AUTO) asks for: a static string, "" when the call
- * would be rejected.  No device work; used to label results.
+ * would be rejected.  The number of columns is not asked: for CCI_ALGO_AUTO the
+ * name is that of the family which runs for many columns.  No device work; used to
+ * label results.
  */
 const char *cci_kernel_name(cci_dtype dtype, int64_t Cin, int64_t R, int64_t Cout, int G, int K,
                             cci_algo algo);

@@ -164,6 +164,7 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
             if (r != 0) return fused_status(r);
         }
         if (!ws_ok) return CCI_ERR_WORKSPACE;
+        if (narrow_ok(p, dtype, p.N)) return to_status(launch_narrow(p, stream));
         algo = CCI_ALGO_DENSE_TC_WS;
     }
     if (p.N == 0) return CCI_OK;
@@ -172,12 +173,14 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
             const int r = try_fused(p, dtype, stream);
             if (r != 0) return fused_status(r);
         }
-        if (dense_ok && ws_ok && aligned(p.X, 16) && aligned(p.Y, 16)) {
-            algo = CCI_ALGO_DENSE_TC_WS;
-        } else if (narrow_ok(p, dtype, p.N) && fused_may(p, dtype)) {
-            // few columns: as fast and as strict about index sets as the fused family,
-            // for the layers that family takes
+        // few columns: one launch in place of the family that has the layer, as strict
+        // about index sets (a workspace is left as it is; CCI_ALGO_DENSE_TC_WS, asked
+        // for by name, leaves the dense weights there whatever the columns)
+        const bool ws_family = dense_ok && ws_ok && aligned(p.X, 16) && aligned(p.Y, 16);
+        if (narrow_ok(p, dtype, p.N) && (ws_family || fused_may(p, dtype)))
             return to_status(launch_narrow(p, stream));
+        if (ws_family) {
+            algo = CCI_ALGO_DENSE_TC_WS;
         } else if (!auto_prefers_fused(K)) {
             const int r = try_fused(p, dtype, stream);
             if (r != 0) return fused_status(r);
@@ -865,12 +868,13 @@ extern "C" cci_status cci_linear_host(const void *X_host, cci_dtype dtype, int64
         FwdParams p = linear_params(xd, nc, Cin, values, idx, Cout, yd, dev_status);
         p.G = G;
         p.K = K;
-        p.N_call = N;
         if (fused) {
             result = to_status(launch_gemm_pk(p, cs));
-        } else if (c == 0 || narrow_ok(p, dtype, N)) {
-            // the first chunk decompresses the weights into the workspace (few columns
-            // in all: every chunk expands them as it multiplies)
+        } else if (narrow_ok(p, dtype, N)) {
+            // few columns in all: every chunk expands the weights as it multiplies
+            result = to_status(launch_narrow(p, cs));
+        } else if (c == 0) {
+            // the first chunk decompresses the weights into the workspace
             result = forward(p, dtype, G, K, CCI_ALGO_DENSE_TC_WS, ws, l.ws, cs);
         } else {
             p.wdense = ws;

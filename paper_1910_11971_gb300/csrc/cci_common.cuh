@@ -19,7 +19,6 @@ struct FwdParams {
     float *Y;            // fp32 output, or bf16 when out_bf16
     uint32_t *status;
     int64_t N;      // columns = B*P*Q
-    int64_t N_call; // columns of the whole call when this is a chunk of it, else 0
     int64_t Cout;
     int64_t R;      // Cin*KH*KW
     int64_t Cin;

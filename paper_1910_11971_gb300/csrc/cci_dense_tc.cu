@@ -186,10 +186,8 @@ cudaError_t launch(const FwdParams &p, cudaStream_t stream)
 }  // namespace dc
 
 // (G, K) pairs of the workspace family: decompression into p.wdense, then the GEMM
-// (products of few columns: one launch that expands the weights as it multiplies)
 cudaError_t launch_dense_tc_ws(const FwdParams &p, int dtype, int G, int K, cudaStream_t stream)
 {
-    if (narrow_ok(p, dtype, p.N_call ? p.N_call : p.N)) return launch_narrow(p, stream);
 #define CCI_TC_CASE(g, k)                                                                   \
     if (G == g && K == k) {                                                                 \
         const cudaError_t e = dtype == CCI_F32 ? dc::launch<uint32_t, g, k, true>(p, stream) \

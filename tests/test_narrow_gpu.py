@@ -81,3 +81,30 @@ def test_host_chunks_keep_the_bits_of_the_whole(dev, N, chunk):
     Yh = cci.linear_host(X.pin_memory(), v, i, Cout, G, K, chunk=chunk)
     torch.cuda.synchronize()
     assert torch.equal(Y.view(torch.int32), Yh.view(torch.int32))
+
+
+@pytest.mark.parametrize("N,Cin,Cout,G,K", [(1, 256, 136, 8, 2), (100, 640, 96, 16, 8), (128, 1024, 64, 4, 1)])
+def test_workspace_family_by_name_leaves_the_dense_weights(dev, N, Cin, Cout, G, K):
+    """Asked for by name, the workspace family decompresses into the workspace whatever
+    the columns and gives a column the bits it has in a call of many columns; AUTO
+    leaves a workspace as it is there, which also shows that its one launch ran."""
+    X, W = wl.random_small(5 + N, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    many = torch.cat([X, X, torch.randn((300, Cin)).to(BF16)]).to(dev)
+    ws = torch.full((Cout * Cin * 2,), 0xA5, dtype=torch.uint8, device=dev)
+    args = (v, i, Cout, G, K)
+    Y = cci.linear(X.to(dev), *args, algo=cci.ALGO_AUTO, workspace=ws)
+    assert bool((ws == 0xA5).all())
+    Yw = cci.linear(X.to(dev), *args, algo=cci.ALGO_DENSE_TC_WS, workspace=ws)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    assert (f64(ws.view(BF16)).reshape(Cout, Cin) == Wd).all()
+    Ym = cci.linear(many, *args, algo=cci.ALGO_DENSE_TC_WS)
+    assert torch.equal(Yw.view(torch.int32), Ym[:N].view(torch.int32))
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    assert_within_tol(f64(Y), Yo, S, "AUTO")
+    assert_within_tol(f64(Yw), Yo, S, "workspace family by name")
+    Ys = torch.empty_like(Yw)  # the static-array entry is the workspace family by name
+    Xd = X.to(dev)
+    assert cci.lib().cci_linear_dense_tc_static(Xd.data_ptr(), cci.BF16, N, Cin, v.data_ptr(), i.data_ptr(), Cout, G, K,
+                                                Ys.data_ptr(), None, cci._stream(dev)) == 0
+    assert torch.equal(Ys.view(torch.int32), Yw.view(torch.int32))
