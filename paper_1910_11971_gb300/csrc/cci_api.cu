@@ -159,12 +159,13 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
         if (p.bias && !aligned(p.bias, 16)) return CCI_ERR_ALIGN;
         if (!aligned(p.X, 16) || !aligned(p.Y, 16)) return CCI_ERR_ALIGN;
         if (p.N == 0) return CCI_OK;
+        // few columns: as AUTO, with a workspace and without
+        if (narrow_ok(p, dtype, p.N) && (ws_ok || fused_may(p, dtype))) return to_status(launch_narrow(p, stream));
         if (auto_prefers_fused(K) || !ws_ok) {
             const int r = try_fused(p, dtype, stream);
             if (r != 0) return fused_status(r);
         }
         if (!ws_ok) return CCI_ERR_WORKSPACE;
-        if (narrow_ok(p, dtype, p.N)) return to_status(launch_narrow(p, stream));
         algo = CCI_ALGO_DENSE_TC_WS;
     }
     if (p.N == 0) return CCI_OK;

@@ -108,3 +108,49 @@ def test_workspace_family_by_name_leaves_the_dense_weights(dev, N, Cin, Cout, G,
     assert cci.lib().cci_linear_dense_tc_static(Xd.data_ptr(), cci.BF16, N, Cin, v.data_ptr(), i.data_ptr(), Cout, G, K,
                                                 Ys.data_ptr(), None, cci._stream(dev)) == 0
     assert torch.equal(Ys.view(torch.int32), Yw.view(torch.int32))
+
+
+def plain_call(X, v, i, Cout, G, K, epilogue, workspace=None):
+    """(status code, Y) of the C call without the binding's workspace: cci_linear_ws with
+    AUTO, or cci_linear_fused without bias and ReLU."""
+    Y = torch.zeros((X.shape[0], Cout), dtype=torch.float32, device=X.device)
+    head = (X.data_ptr(), cci.BF16, X.shape[0], X.shape[1], v.data_ptr(), i.data_ptr(), Cout, G, K)
+    ws = (None, 0) if workspace is None else (workspace.data_ptr(), workspace.numel())
+    if epilogue:
+        code = cci.lib().cci_linear_fused(*head, None, 0, cci.F32, Y.data_ptr(), None, *ws, cci._stream(X.device))
+    else:
+        code = cci.lib().cci_linear_ws(*head, Y.data_ptr(), None, cci.ALGO_AUTO, *ws, cci._stream(X.device))
+    return code, Y
+
+
+@pytest.mark.parametrize("N,Cin,Cout,G,K", [(8, 384, 40, 8, 2), (100, 2048, 144, 16, 8), (128, 1024, 264, 4, 1)])
+def test_one_launch_without_a_workspace(dev, N, Cin, Cout, G, K):
+    """Without a workspace the layer runs the same launch, with the same bits, through
+    the plain entry point and the one with an output stage as with a workspace (which
+    stays unwritten: the launch that reads none ran)."""
+    X, W = wl.random_small(9 + N, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    Xd = X.to(dev)
+    ws = torch.full((Cout * Cin * 2,), 0xA5, dtype=torch.uint8, device=dev)
+    outs = [plain_call(Xd, v, i, Cout, G, K, ep, w) for ep in (False, True) for w in (ws, None)]
+    assert [code for code, _ in outs] == [0] * 4
+    assert bool((ws == 0xA5).all())
+    for _, Y in outs[1:]:
+        assert torch.equal(Y.view(torch.int32), outs[0][1].view(torch.int32))
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    assert_within_tol(f64(outs[0][1]), Yo, S, "no workspace")
+
+
+def test_layers_that_need_a_workspace_still_ask_for_it(dev):
+    """R * K no multiple of 16: the fused family does not have the layer, so without a
+    workspace the output stage is refused and AUTO runs on the CUDA cores."""
+    N, Cin, Cout, G, K = 8, 1032, 72, 8, 1
+    X, W = wl.random_small(2, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    assert plain_call(X.to(dev), v, i, Cout, G, K, True)[0] == 11
+    code, Y = plain_call(X.to(dev), v, i, Cout, G, K, False)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    assert code == 0
+    assert_within_tol(f64(Y), Yo, S, "AUTO without a workspace")
