@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     };
     tc::wait_prior_grid();  // a programmatic dependent of the kernel before it
-    tc::launch_next_grid();
     if (warp < 4 * kGroups) {
 #pragma unroll
         for (int b = 0; b < NB; ++b)
@@ -253,6 +252,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = S->tmem_base;
+    // the next grid may be scheduled from here on: this block holds its tensor memory,
+    // so a block of the next grid that takes some and then waits for this grid cannot
+    // keep this one from its own
+    tc::launch_next_grid();
     // the wait for this arrival, before the first store into another CTA, sees that
     // every CTA of the cluster runs
     if (parts > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");

@@ -154,3 +154,38 @@ def test_layers_that_need_a_workspace_still_ask_for_it(dev):
     Yo, S = oracle.linear(f64(X), Wd, mask)
     assert code == 0
     assert_within_tol(f64(Y), Yo, S, "AUTO without a workspace")
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_launches_in_a_row_read_what_the_ones_before_wrote(dev, captured):
+    """Each launch may be scheduled before the one ahead has ended: a chain of layers in
+    one stream, called and as a CUDA graph, equals the same layers with a wait after
+    each, bit for bit."""
+    N, C, G, K, depth = 32, 1024, 8, 2, 40
+    g = torch.Generator().manual_seed(4)
+    X0 = torch.randn((N, C), generator=g).to(BF16).to(dev)
+    packed = [cci.pack((torch.randn((C, C), generator=g) * (2.0 / C) ** 0.5).to(BF16).to(dev), G, K)
+              for _ in range(3)]
+
+    def chain(wait):
+        x, outs = X0, []
+        for n in range(depth):
+            v, i = packed[n % 3]
+            x = cci.linear_fused(x, v, i, C, G, K, relu=n % 2 == 0, out_dtype=BF16)
+            outs.append(x)
+            if wait:
+                torch.cuda.synchronize()
+        return outs
+
+    want = chain(True)
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            got = chain(False)
+        graph.replay()
+    else:
+        got = chain(False)
+    torch.cuda.synchronize()
+    for n, (a, b) in enumerate(zip(got, want)):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16)), n
+    assert bool(want[-1].isfinite().all()) and bool((want[-1] != 0).any())
