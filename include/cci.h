@@ -339,8 +339,9 @@ cci_status cci_pack_stats(const void *W, cci_dtype dtype, int64_t Cout, int64_t 
  * cci_linear_fused / cci_conv2d_fused -- the product / convolution of
  * cci_linear_ws / cci_conv2d_ws on a tensor-core family (the fused one where AUTO
  * would pick it or no workspace is given, else CCI_ALGO_DENSE_TC_WS; products of few
- * columns in one launch, where AUTO runs it), followed by the usual output stage of a CNN layer, applied in the kernel's epilogue to each fp32
- * accumulator y[n][co] (the sum of Alg. 2, Sec. 3.2):
+ * columns in one launch, where AUTO runs it), followed by the usual output stage of
+ * a CNN layer, applied in the kernel's epilogue to each fp32 accumulator y[n][co]
+ * (the sum of Alg. 2, Sec. 3.2):
  *   y += bias[co]          when bias != NULL (fp32, Cout entries, 16-byte aligned);
  *   y = max(y, 0)          when relu != 0;
  *   Y[n][co] = y           as fp32 (out_dtype CCI_F32) or rounded to the nearest

@@ -500,7 +500,9 @@ def _auto_bytes(dtype: torch.dtype, Cin: int, R: int, Cout: int, G: int, K: int,
 @functools.lru_cache(maxsize=4096)
 def _epilogue_bytes(dtype: torch.dtype, Cin: int, R: int, Cout: int, G: int, K: int, wide_stride: bool) -> int:
     """Workspace bytes of the entry points with an output stage (0: none needed)."""
-    return 0 if _fused_first(dtype, Cin, R, Cout, G, K, wide_stride) else workspace_size(ALGO_DENSE_TC_WS, dtype, Cout, R)
+    if _fused_first(dtype, Cin, R, Cout, G, K, wide_stride):
+        return 0
+    return workspace_size(ALGO_DENSE_TC_WS, dtype, Cout, R)
 
 
 def _fused_first(dtype, Cin, R, Cout, G, K, wide_stride) -> bool:

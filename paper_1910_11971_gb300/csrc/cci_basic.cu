@@ -380,8 +380,9 @@ __device__ __forceinline__ void store_words(void *at, const uint32_t (&w)[kBytes
 // G = 8, two above (four would take the registers of half the warps: 44 us instead
 // of 33.7 at G = 16).  Measured on GB300, 4096 x 4096 fp32 (218 MB): G = 16, K = 2
 // 49.8 us one column per thread -> 33.7 us (6.5 TB/s), G = 8 38.9 -> 33.0, G = 32,
-// K = 8 96.8 -> 42.9; bf16 G = 16, K = 2 49.9 -> 24.7.  Needs R % 4 == 0, 16-byte aligned W, u and W_out, a 4-byte aligned mask (or
-// none) and Cout / G <= 65535.
+// K = 8 96.8 -> 42.9; bf16 G = 16, K = 2 49.9 -> 24.7 (device times in a CUDA graph).
+// Needs R % 4 == 0, 16-byte aligned W, u and W_out, a 4-byte aligned mask (or none)
+// and Cout / G <= 65535.
 template <typename TB, int GT, int KT>
 __global__ void __launch_bounds__(128) td_mask_vec_kernel(const TB *__restrict__ W, int64_t R, float rate,
                                                           const float *__restrict__ u, TB *__restrict__ Wout,

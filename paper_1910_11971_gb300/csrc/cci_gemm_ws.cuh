@@ -372,19 +372,6 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t local, uint32_t rank)
     return r;
 }
 
-// 16 bytes into the shared memory of a CTA of the cluster (shared::cluster address)
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
-__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
-{
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1687,7 +1674,8 @@ inline ConvBox choose_box(int64_t B_, int64_t P, int64_t Q)
 {
     ConvBox best{1, 1, 1, 1, 1, 1, B_};
     int64_t best_tiles = -1;
-    const int q_all = static_cast<int>(Q), p_all = static_cast<int>(P), B = static_cast<int>(B_);  // below 2^30 (a_source)
+    // all below 2^30 (a_source)
+    const int q_all = static_cast<int>(Q), p_all = static_cast<int>(P), B = static_cast<int>(B_);
     int ext[128], num[128], n_ext = 0;  // extents along p up to 128 and the boxes they make
     for (int PB = 1; PB <= p_all && PB <= 128; PB = next_extent(p_all, PB)) {
         ext[n_ext] = PB;
@@ -1721,13 +1709,6 @@ inline int a_source(const FwdParams &p, int ks)
     const bool fits = p.H < lim && p.W < lim && p.N < lim && (p.N / (p.P * p.Q)) < lim;
     const bool strides_ok = p.sh >= 1 && p.sh <= 2 && p.sw >= 1 && p.sw <= 2 && p.H >= p.sh && p.W >= p.sw;
     return (strides_ok && p.Cin % ks == 0 && fits) ? kA4d : kAGather;
-}
-
-// clusters of 1 << log_parts CTAs (one per SM) that run at once: they stay inside a
-// GPC, so larger ones leave SMs over (152 SMs: 76, 36 and 15)
-inline int64_t cluster_slots(int log_parts, int64_t sms)
-{
-    return log_parts == 0 ? sms : (log_parts == 1 ? sms / 2 : (log_parts == 2 ? sms * 15 / 64 : sms / 10));
 }
 
 // N tile among {64, 128, 256} (up to max_bn): fewest rounds of tiles over the

@@ -27,14 +27,20 @@
 // The number of parts depends on Cout and R alone, never on N, so a product cut
 // into chunks of columns gives the same bits as the whole.
 //
-// Where the rule lies (device time per pass against decompression and GEMM): 16 x
-// 4096 -> 4096 9.4 us against 23.5, 100 x 2048 -> 1000 7.2 against 12.2, 100 x 1024
-// -> 4096 7.0 against 9.4, 32 x 4096 -> 1024 at G = 32, K = 8 6.3 against 23.6; up to
-// seven stages in one part it is even with them (25 x 432 -> 992 5.9 against 5.8, 7 x
-// 16 -> 1360 3.6 against 4.3) and saves the second launch, some 3 us of host time a
-// call; eight or nine stages are too few to split and take 7.7 against 6.2 (128 x
-// 512 -> 512) and 8.0 against 6.3 (64 x 576 -> 1024), so those stay there.  At 128
-// columns 4096 -> 4096 takes 12.5 against 23.7; more would need smaller stages.
+// Where the rule lies (GB300, 348 shapes; device time per pass in a CUDA graph, in
+// brackets the time of a call from the host, against decompression and GEMM, bf16
+// G = 8, K = 2 unless said).  From 16 stages on 0.27 to 0.98 of their time, 0.55 in
+// the mean: 16 x 4096 -> 4096 9.6 us (13.5) against 23.6 (24.8), 128 x 4096 -> 4096 12.7
+// against 23.9, 16 x 4096 -> 1024 at G = 32, K = 8 6.2 against 23.2; also where the tiles
+// fill the SMs and no reduction is split (more than 9728 channels): 16 x 4096 -> 32768
+// 62.7 against 109.7, 128 x 4096 -> 9984 38.1 against 38.9.  Up to seven stages: 0.75 in
+// the mean and at most 1.01 up to 16 columns; 0.98 and up to 1.26 from 64 on (64 x
+// 448 -> 1000 7.4 against 5.9), as ten stages do (128 x 640 -> 512 7.8 against 6.7).
+// Those stay here for the launch that a call saves, 13.6 us (64 x 448 -> 1000) against
+// 20.2; in a captured graph they lose that up to 1.6 us.  Eight or nine stages are too
+// few to split and took 7.7 against 6.2 (128 x 512 -> 512) and 8.0 against 6.3 (64 x 576
+// -> 1024), measured on these two alone: they stay with the GEMM.  More than 128 columns
+// would need smaller stages.
 #include "cci_gemm_ws.cuh"
 
 namespace cci {
@@ -79,8 +85,22 @@ struct Smem {
 };
 static_assert(sizeof(Smem) <= 1024, "barriers");
 
-using ws::ld_shared_f4;
-using ws::st_cluster_v4;
+// 16 bytes into the shared memory of a CTA of the cluster (shared::cluster address)
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
 
 // Y[n][co] in the output type
 __device__ __forceinline__ void store_y(const FwdParams &p, int n, int64_t co, float y)
@@ -385,7 +405,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (warp < 4 * kGroups && co < p.Cout) {
             const float b = p.bias ? __ldg(p.bias + co) : 0.f;
             for (int i = tid >> 7; 4 * (i * parts + rank) < p.N; i += kGroups) {
-                const uint32_t at = sums + static_cast<uint32_t>(i * parts) * (kM * 16u) + static_cast<uint32_t>(tid & 127) * 16u;
+                const uint32_t at =
+                    sums + static_cast<uint32_t>(i * parts) * (kM * 16u) + static_cast<uint32_t>(tid & 127) * 16u;
                 float4 y = ld_shared_f4(at);
                 for (int j = 1; j < parts; ++j) {
                     const float4 z = ld_shared_f4(at + static_cast<uint32_t>(j) * (kM * 16u));
@@ -409,6 +430,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
+// clusters of 1 << log_parts CTAs (one per SM; log_parts 1, 2 or 3) that a launch
+// counts on running at once.  They stay inside a GPC, so larger ones leave SMs over:
+// on 152 SMs 76, 35 and 15 (36 clusters of four were seen resident)
+int64_t cluster_slots(int log_parts, int64_t sms)
+{
+    return log_parts == 1 ? sms / 2 : (log_parts == 2 ? sms * 15 / 64 : sms / 10);
+}
+
 template <int K, int NP>
 cudaError_t launch(const FwdParams &p, cudaStream_t stream)
 {
@@ -425,7 +454,7 @@ cudaError_t launch(const FwdParams &p, cudaStream_t stream)
     // kMinStages stages
     const int64_t sms = ws::sm_count();
     int log_parts = 0;
-    while ((2 << log_parts) <= kMaxParts && tiles <= ws::cluster_slots(log_parts + 1, sms) &&
+    while ((2 << log_parts) <= kMaxParts && tiles <= cluster_slots(log_parts + 1, sms) &&
            nks >= kSplitStages && nks >= (2 << log_parts) * kMinStages)
         ++log_parts;
     const int parts = 1 << log_parts;
@@ -465,9 +494,10 @@ bool narrow_ok(const FwdParams &p, int dtype, int64_t N)
     const bool gk = (p.G == 4 || p.G == 8 || p.G == 16 || p.G == 32) &&
                     (p.K == 1 || p.K == 2 || p.K == 4 || p.K == 8) && 2 * p.K <= p.G;
     auto at16 = [](const void *q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };
+    const int64_t lim = int64_t(1) << 31, nks = (p.R + 63) / 64;
     return dtype == CCI_BF16 && !p.is_conv && N > 0 && N <= narrow::kMaxN && gk && p.Cin == p.R && p.R % 8 == 0 &&
-           ((p.R + 63) / 64 <= narrow::kWholeStages || (p.R + 63) / 64 >= narrow::kSplitStages) && p.R < (int64_t(1) << 31) && p.Cout < (int64_t(1) << 31) && at16(p.X) && at16(p.Y) && at16(p.values) &&
-           at16(p.idx);
+           (nks <= narrow::kWholeStages || nks >= narrow::kSplitStages) && p.R < lim && p.Cout < lim && at16(p.X) &&
+           at16(p.Y) && at16(p.values) && at16(p.idx);
 }
 
 cudaError_t launch_narrow(const FwdParams &p, cudaStream_t stream)

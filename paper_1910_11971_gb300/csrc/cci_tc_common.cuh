@@ -98,7 +98,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
 // operands there, while behind a test of the lane number it moves every operand
 // over with a per-lane sequence.  Measured on GB300 for a loop of wait, four
 // 128 x 64 x 16 MMAs and a commit per stage: 361 cycles a stage behind lane == 0,
-// 222 behind the election (192 are the tensor core's).
+// 222 behind the election (192 are the tensor core's).  The few-column product
+// issues behind it; the workspace GEMM still tests the lane number.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t e;
