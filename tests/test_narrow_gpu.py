@@ -1,6 +1,8 @@
 """Products of at most 128 columns: one launch that expands the packed weights as it
-multiplies, the reduction of ten stages of 64 indices or more split over a cluster.  Every output against the fp64 oracle at the tolerance of all products
-(1e-5 of sum |w||x|), with the output stage's bf16 rounding where it applies."""
+multiplies, the reduction of ten stages of 64 indices or more split over a cluster
+where the SMs hold it.  Every output against the fp64 oracle at the tolerance of all
+products (1e-5 of sum |w||x|), with the output stage's bf16 rounding where it applies;
+that the launch ran is shown by the workspace, which it leaves as it is."""
 import numpy as np
 import pytest
 import torch
@@ -21,11 +23,16 @@ def dev():
 
 # columns at the edges of the MMA's N (16, 32, 64, 128); reductions of one chunk and
 # less, at both edges of the rule (7 stages, 10), with a ragged last stage, and deep
-# enough for 2, 4 and 8 parts of unequal length; channels below, at and past a tile of 128; every K, G 4 to 32
-CASES = [(1, 8, 8, 8, 2), (7, 16, 1360, 8, 1), (33, 72, 24, 4, 2), (128, 448, 224, 32, 8), (100, 584, 136, 8, 4),
-         (16, 640, 96, 16, 8), (1, 1024, 64, 4, 1), (16, 1032, 72, 8, 2), (17, 1536, 1000, 8, 4), (32, 2048, 128, 16, 8), (33, 1096, 136, 4, 2),
-         (64, 4096, 256, 32, 4), (65, 2056, 160, 32, 1), (100, 2048, 1000, 8, 1), (127, 1160, 96, 16, 2),
-         (128, 3000, 264, 8, 2), (5, 1024, 20, 4, 1), (128, 4096, 4096, 16, 4)]
+# enough for 2, 4 and 8 parts of unequal length; channels below, at and past a tile of
+# 128, at the last tile count that is split (76) and past it, and more tiles than SMs;
+# every K, G 4 to 32
+CASES = [
+    (1, 8, 8, 8, 2), (7, 16, 1360, 8, 1), (33, 72, 24, 4, 2), (128, 448, 224, 32, 8), (100, 584, 136, 8, 4),
+    (16, 640, 96, 16, 8), (1, 1024, 64, 4, 1), (16, 1032, 72, 8, 2), (17, 1536, 1000, 8, 4), (32, 2048, 128, 16, 8),
+    (33, 1096, 136, 4, 2), (64, 4096, 256, 32, 4), (65, 2056, 160, 32, 1), (100, 2048, 1000, 8, 1),
+    (127, 1160, 96, 16, 2), (128, 3000, 264, 8, 2), (5, 1024, 20, 4, 1), (128, 4096, 4096, 16, 4),
+    (40, 1024, 4608, 8, 2), (3, 640, 9728, 8, 2), (128, 640, 9736, 8, 4), (5, 1032, 19584, 8, 2),
+]
 
 
 @pytest.mark.parametrize("N,Cin,Cout,G,K", CASES)
@@ -33,11 +40,48 @@ def test_narrow_product(dev, N, Cin, Cout, G, K):
     X, W = wl.random_small(N + Cin + Cout, "bf16", N, Cin, Cout)
     v, i = cci.pack(W.to(dev), G, K)
     st = cci.new_status(dev)
-    Y = cci.linear(X.to(dev), v, i, Cout, G, K, status=st)
+    ws = torch.full((Cout * Cin * 2,), 0xA5, dtype=torch.uint8, device=dev)
+    Y = cci.linear(X.to(dev), v, i, Cout, G, K, status=st, workspace=ws)
     assert cci.read_status(st) == 0
+    assert bool((ws == 0xA5).all())  # the one launch ran
     _, _, Wd, mask = oracle_reference(W, G, K)
     Yo, S = oracle.linear(f64(X), Wd, mask)
     assert_within_tol(f64(Y), Yo, S, f"narrow product {N} x {Cin} -> {Cout}")
+
+
+# (N, Cin, G, K): one column too many, eight and nine stages (with ragged ends), K = 16
+@pytest.mark.parametrize("N,Cin,G,K", [(129, 1024, 8, 2), (1, 456, 8, 2), (64, 512, 8, 1), (128, 512, 16, 8),
+                                       (100, 576, 4, 2), (128, 576, 32, 8), (16, 1024, 32, 16)])
+def test_past_the_rule_the_workspace_family_runs(dev, N, Cin, G, K):
+    Cout = 224
+    X, W = wl.random_small(N + Cin, "bf16", N, Cin, Cout)
+    v, i = cci.pack(W.to(dev), G, K)
+    ws = torch.full((Cout * Cin * 2,), 0xA5, dtype=torch.uint8, device=dev)
+    Y = cci.linear(X.to(dev), v, i, Cout, G, K, workspace=ws)
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    assert (f64(ws.view(BF16)).reshape(Cout, Cin) == Wd).all()
+    Yo, S = oracle.linear(f64(X), Wd, mask)
+    assert_within_tol(f64(Y), Yo, S, f"workspace product {N} x {Cin} -> {Cout}")
+
+
+def test_infinite_and_nan_activations(dev):
+    """A pruned weight times an infinity or a NaN is NaN, as in the dense product of
+    the workspace family; the other columns are untouched by it."""
+    N, Cin, Cout, G, K = 33, 1096, 136, 8, 2
+    X, W = wl.random_small(6, "bf16", N, Cin, Cout)
+    X[3, 700] = float("inf")
+    X[20, 1095] = float("-inf")
+    X[32, 0] = float("nan")
+    v, i = cci.pack(W.to(dev), G, K)
+    Y = f64(cci.linear(X.to(dev), v, i, Cout, G, K))
+    Yw = f64(cci.linear(X.to(dev), v, i, Cout, G, K, algo=cci.ALGO_DENSE_TC_WS))
+    assert (np.isnan(Y) == np.isnan(Yw)).all() and np.isnan(Y[[3, 20, 32]]).any(axis=1).all()
+    assert (np.isposinf(Y) == np.isposinf(Yw)).all() and (np.isneginf(Y) == np.isneginf(Yw)).all()
+    assert np.isinf(Y[[3, 20]]).any()
+    rest = np.setdiff1d(np.arange(N), [3, 20, 32])
+    _, _, Wd, mask = oracle_reference(W, G, K)
+    Yo, S = oracle.linear(f64(X[rest]), Wd, mask)
+    assert_within_tol(Y[rest], Yo, S, "finite columns")
 
 
 @pytest.mark.parametrize("N,Cin,Cout,G,K", [(16, 1024, 136, 8, 2), (100, 2048, 1000, 8, 4), (3, 4096, 96, 32, 8)])
@@ -68,6 +112,42 @@ def test_narrow_product_reports_bad_index_sets(dev):
         st = cci.new_status(dev)
         cci.linear(X.to(dev), v, j, Cout, G, K, status=st)
         assert cci.read_status(st) == 10, bad
+
+
+def bad_sets(G, K):
+    """Index sets with one fault each: two neighbouring slots equal or swapped, for every
+    pair of slots, and a last index at and above G."""
+    good = list(range(K))
+    sets = [good[:-1] + [G], good[:-1] + [255]]
+    for s in range(K - 1):
+        sets += [good[:s + 1] + [s] + good[s + 2:], good[:s] + [s + 1, s] + good[s + 2:]]
+    return sets
+
+
+# few columns (the one launch); the decompression and the fused family, whatever the columns
+@pytest.mark.parametrize("G,K", [(4, 1), (32, 1), (4, 2), (32, 2), (8, 4), (32, 4), (16, 8), (32, 8)])
+@pytest.mark.parametrize("N,algo", [(8, cci.ALGO_AUTO), (8, cci.ALGO_DENSE_TC_WS), (200, cci.ALGO_DENSE_TC_WS),
+                                    (200, cci.ALGO_DENSE_TC)], ids=["few", "ws8", "ws200", "fused"])
+def test_bad_index_sets_are_reported(dev, N, algo, G, K):
+    """Each fault alone, in the first and the last set, and at a set that starts at
+    another byte of its word, is reported; the untouched sets are not."""
+    Cin, Cout = 1040, 96
+    X, W = wl.random_small(3, "bf16", N, Cin, Cout)
+    X = X.to(dev)
+    v, i = cci.pack(W.to(dev), G, K)
+
+    def status_of(j):
+        st = cci.new_status(dev)
+        cci.linear(X, v, j, Cout, G, K, status=st, algo=algo)
+        return cci.read_status(st)
+
+    assert status_of(i) == 0
+    assert status_of(torch.arange(G - K, G, dtype=torch.uint8, device=dev).expand_as(i).contiguous()) == 0
+    for bad in bad_sets(G, K):
+        for at in ((0, 0), (i.shape[0] // 2, 5), (-1, -1)):
+            j = i.clone()
+            j[at] = torch.tensor(bad, dtype=torch.uint8)
+            assert status_of(j) == 10, (bad, at)
 
 
 @pytest.mark.parametrize("N,chunk", [(100, 32), (300, 100)])
