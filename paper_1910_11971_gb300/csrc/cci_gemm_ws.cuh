@@ -57,11 +57,10 @@
 // 9 + kIssuers .. + 3 as the second producer group), warp 8 allocates TMEM and
 // issues the MMAs, warps 9 .. 8 + kIssuers issue the TMA copies as soon as a
 // stage is free (so copy latency overlaps the producers' work), stage by stage in
-// turn: the copies one thread issues are processed one box after another
-// (measured on GB300: about 0.5 us per box of 16-64 KB from one issuer; copy
-// throughput grows with the number of issuing warps), so up to six warps issue
-// (one per stage in flight; PK: three, one activation box per stage).  Every
-// mbarrier wait is bounded (CCI_ERR_TIMEOUT, abort flag, drain, TMEM freed).
+// turn: a box costs its issuer the length of the issue loop, whatever the box's
+// size (with the run-time divisions of this loop over 2000 cycles a stage, measured
+// on GB300), so up to six warps issue (one per stage in flight; PK: three, one
+// activation box per stage).  Every mbarrier wait is bounded (CCI_ERR_TIMEOUT, abort flag, drain, TMEM freed).
 #pragma once
 
 #include <cuda.h>
@@ -160,9 +159,9 @@ struct Cfg {
     static_assert(kStages >= 3, "too few pipeline stages");
     static_assert(kTmemCols == 128 || kTmemCols == 256 || kTmemCols == 512, "TMEM allocation not a power of 2");
     static_assert(!kARaw || kAColBase + kStages * 64 <= 512, "A stages do not fit in tensor memory");
-    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: one
-    // thread's copies are processed one box at a time, so several issuers keep
-    // more boxes moving.  kIssuers <= kStages keeps every empty-barrier wait
+    // warps issuing the TMA copies, stage `it` by warp 9 + it % kIssuers: a box
+    // costs its issuer the same loop whatever its size, so several issuers keep
+    // more bytes moving.  kIssuers <= kStages keeps every empty-barrier wait
     // within one phase of the barrier (no parity aliasing).
     // (kAHalo: one more warp, which copies the halos)
     // PK: three issuers (one activation box per stage) and a second group of four

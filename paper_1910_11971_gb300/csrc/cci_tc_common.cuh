@@ -1,5 +1,5 @@
 // cci_tc_common.cuh -- device helpers of the tensor-core kernels (tcgen05,
-// mbarrier, cp.async, TMA) shared by cci_dense_tc.cu and cci_gemm_ws.cu.
+// mbarrier, cp.async, TMA) shared by cci_dense_tc.cu, cci_gemm_ws.cuh and cci_narrow.cu.
 #pragma once
 
 #include "cci_kernels.h"
