@@ -37,10 +37,11 @@
 // the mean and at most 1.01 up to 16 columns; 0.98 and up to 1.26 from 64 on (64 x
 // 448 -> 1000 7.4 against 5.9), as ten stages do (128 x 640 -> 512 7.8 against 6.7).
 // Those stay here for the launch that a call saves, 13.6 us (64 x 448 -> 1000) against
-// 20.2; in a captured graph they lose that up to 1.6 us.  Eight or nine stages are too
-// few to split and took 7.7 against 6.2 (128 x 512 -> 512) and 8.0 against 6.3 (64 x 576
-// -> 1024), measured on these two alone: they stay with the GEMM.  More than 128 columns
-// would need smaller stages.
+// 20.2; in a captured graph they lose that up to 1.6 us.  Eight or nine stages, too few
+// to split, stay with the GEMM: in this form 0.36 to 1.36 of its time over 76 shapes,
+// slower from 64 columns on at up to 9728 channels (64 x 576 -> 512 8.6 against 6.3),
+// 1.06 at most up to 16 columns (16 x 576 -> 4096 6.9 against 7.9).  More than 128
+// columns would need smaller stages.
 #include "cci_gemm_ws.cuh"
 
 namespace cci {
