@@ -140,6 +140,16 @@ int try_fused(const FwdParams &p, int dtype, cudaStream_t stream)
 
 cci_status fused_status(int r) { return r > 0 ? CCI_OK : CCI_ERR_CUDA; }
 
+// the one-launch product of few columns (N: those of the whole call), as try_fused:
+// 0 also when its activations cannot be copied by TMA
+int try_narrow(const FwdParams &p, int dtype, int64_t N, cudaStream_t stream)
+{
+    if (!narrow_ok(p, dtype, N)) return 0;
+    const cudaError_t e = launch_narrow(p, stream);
+    if (e == cudaErrorNotSupported) return 0;
+    return e == cudaSuccess ? 1 : -1;
+}
+
 cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws, size_t ws_bytes,
                    cudaStream_t stream)
 {
@@ -160,7 +170,10 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
         if (!aligned(p.X, 16) || !aligned(p.Y, 16)) return CCI_ERR_ALIGN;
         if (p.N == 0) return CCI_OK;
         // few columns: as AUTO, with a workspace and without
-        if (narrow_ok(p, dtype, p.N) && (ws_ok || fused_may(p, dtype))) return to_status(launch_narrow(p, stream));
+        if (ws_ok || fused_may(p, dtype)) {
+            const int r = try_narrow(p, dtype, p.N, stream);
+            if (r != 0) return fused_status(r);
+        }
         if (auto_prefers_fused(K) || !ws_ok) {
             const int r = try_fused(p, dtype, stream);
             if (r != 0) return fused_status(r);
@@ -178,8 +191,10 @@ cci_status forward(FwdParams p, int dtype, int G, int K, cci_algo algo, void *ws
         // about index sets (a workspace is left as it is; CCI_ALGO_DENSE_TC_WS, asked
         // for by name, leaves the dense weights there whatever the columns)
         const bool ws_family = dense_ok && ws_ok && aligned(p.X, 16) && aligned(p.Y, 16);
-        if (narrow_ok(p, dtype, p.N) && (ws_family || fused_may(p, dtype)))
-            return to_status(launch_narrow(p, stream));
+        if (ws_family || fused_may(p, dtype)) {
+            const int r = try_narrow(p, dtype, p.N, stream);
+            if (r != 0) return fused_status(r);
+        }
         if (ws_family) {
             algo = CCI_ALGO_DENSE_TC_WS;
         } else if (!auto_prefers_fused(K)) {
@@ -849,6 +864,7 @@ extern "C" cci_status cci_linear_host(const void *X_host, cci_dtype dtype, int64
     if (e == cudaSuccess && so != cs) e = cudaStreamWaitEvent(so, ev[0], 0);
     cci_status result = to_status(e);
     int64_t issued = 0;  // chunks whose copy-out was enqueued
+    bool dense = false;  // the workspace holds the dense weights
     for (int64_t c = 0; c < chunks && result == CCI_OK; ++c) {
         const int k = static_cast<int>(c % kHostSlots);
         const int64_t n0 = c * chunk_cols;
@@ -869,14 +885,16 @@ extern "C" cci_status cci_linear_host(const void *X_host, cci_dtype dtype, int64
         FwdParams p = linear_params(xd, nc, Cin, values, idx, Cout, yd, dev_status);
         p.G = G;
         p.K = K;
-        if (fused) {
+        // few columns in all: every chunk expands the weights as it multiplies
+        const int few = fused ? 0 : try_narrow(p, dtype, N, cs);
+        if (few != 0) {
+            result = fused_status(few);
+        } else if (fused) {
             result = to_status(launch_gemm_pk(p, cs));
-        } else if (narrow_ok(p, dtype, N)) {
-            // few columns in all: every chunk expands the weights as it multiplies
-            result = to_status(launch_narrow(p, cs));
-        } else if (c == 0) {
+        } else if (!dense) {
             // the first chunk decompresses the weights into the workspace
             result = forward(p, dtype, G, K, CCI_ALGO_DENSE_TC_WS, ws, l.ws, cs);
+            dense = true;
         } else {
             p.wdense = ws;
             result = to_status(launch_gemm_ws(p, dtype, cs));

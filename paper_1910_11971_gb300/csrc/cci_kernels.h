@@ -38,7 +38,9 @@ cudaError_t launch_gemm_ws_tf32(const FwdParams &p, cudaStream_t stream);
 // products of at most 128 columns in one launch (cci_narrow.cu; bf16, no
 // workspace): the packed weights (p.values, p.idx, p.G, p.K) expanded and
 // multiplied once, the reduction split over a cluster.  N: the columns of the
-// whole call (a host-buffer product runs chunks of it, with the bits of the whole)
+// whole call (a host-buffer product runs chunks of it, with the bits of the whole).
+// launch_narrow returns cudaErrorNotSupported, before any launch, when the activations
+// cannot be copied by TMA
 bool narrow_ok(const FwdParams &p, int dtype, int64_t N);
 cudaError_t launch_narrow(const FwdParams &p, cudaStream_t stream);
 

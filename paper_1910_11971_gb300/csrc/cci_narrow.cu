@@ -446,7 +446,7 @@ cudaError_t launch(const FwdParams &p, cudaStream_t stream)
     CUtensorMap tmX{};
     const int64_t dims[2] = {p.Cin, p.N};
     const int box[2] = {64, NP};
-    if (!ws::make_map(&tmX, p.X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 2, dims, box)) return cudaErrorInvalidValue;
+    if (!ws::make_map(&tmX, p.X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 2, dims, box)) return cudaErrorNotSupported;
     static SmemAttrCache attr_cache;
     const cudaError_t attr = smem_attr_once(narrow_kernel<K, NP>, static_cast<int>(C::kSmem), attr_cache);
     if (attr != cudaSuccess) return attr;
