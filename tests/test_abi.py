@@ -209,10 +209,12 @@ def test_fused_rejects(lib):
     assert fused(lib, bias=FAKE + 4) == ALIGN             # bias must be 16-byte aligned
     assert fused(lib, Y=FAKE + 8) == ALIGN
     assert fused(lib, X=FAKE + 8) == ALIGN
-    assert fused(lib, ws=None, wsb=0) == 11               # CCI_ERR_WORKSPACE
-    assert fused(lib, wsb=64 * 64 * 2 - 2) == 11
-    assert fused(lib, ws=FAKE + 8) == 11
-    assert lib.cci_conv2d_fused(FAKE, 1, 1, 4, 4, 64, FAKE, FAKE, 64, 3, 3, 1, 1, 1, 1, 8, 2, None, 1, 1,
+    # CCI_ERR_WORKSPACE: K = 16, a layer that needs a workspace.  (Layers that run without
+    # one would be launched on these addresses where there is a GPU.)
+    assert fused(lib, G=32, K=16, ws=None, wsb=0) == 11
+    assert fused(lib, G=32, K=16, wsb=64 * 64 * 2 - 2) == 11
+    assert fused(lib, G=32, K=16, ws=FAKE + 8) == 11
+    assert lib.cci_conv2d_fused(FAKE, 1, 1, 4, 4, 64, FAKE, FAKE, 64, 3, 3, 1, 1, 1, 1, 32, 16, None, 1, 1,
                                 FAKE, None, None, 0, None) == 11
     assert lib.cci_conv2d_fused(FAKE, 1, 1, 4, 4, 64, FAKE, FAKE, 64, 3, 3, 1, 1, 1, 1, 8, 2, None, 1, 7,
                                 FAKE, None, FAKE, 1 << 20, None) == DTYPE
